@@ -359,6 +359,13 @@ struct Lds<__half, OFF> {
     }
 };
 
+// 1 / x for normal x, to an ulp (one MUFU instruction)
+__device__ __forceinline__ float rcp_approx(float x) {
+    float y;
+    asm("rcp.approx.ftz.f32 %0, %1;" : "=f"(y) : "f"(x));
+    return y;
+}
+
 // address bias: (row + kMagicBits) * 4 WD wraps to row * 4 WD in 32 bits once
 // tbase absorbs -kMagicBits * 4 WD (keeps the unsigned arithmetic explicit)
 constexpr int kMagicBits = 0x4B400000;
@@ -548,19 +555,24 @@ bp_tma_kernel(const __grid_constant__ CUtensorMap tmap, BpTmaParams a) {
 
 // ---------------------------------------------------------------------------
 // Mirrored-pair form of the staged backprojection (whole volumes).  Each
-// thread owns kZP slices p0 .. p0 + kZP - 1 of the lower half of its (x, y)
+// thread owns ZP slices p0 .. p0 + ZP - 1 of the lower half of its (x, y)
 // column and their mirror images N - 1 - p about the mid-plane z = 0.  A
 // voxel and its mirror read the same column (Eq. 1 does not involve z) and
 // mirrored rows: z/U + (Nv-1)/2 and -z/U + (Nv-1)/2 add up to Nv - 1.  So
 // the column weights, the row fraction and the per-view set-up are shared
 // by the pair, and with the two windows of a view staged at row origins vlo
 // and vlo', the mirror's window row is C - v for C = Nv - 1 - vlo - vlo'.
-// Row coordinates are 9.23 fixed point: v = V 2^-23 advances by an integer
-// step per slice, the row is V >> 23 and the fraction's float is the
-// mantissa bits of V under the exponent of 1.0.  Where every thread of a
-// warp has 1/U <= 1 for the view, consecutive slices move by 0 or 1 row,
-// so each slice loads only its new row of the pair (two samples per voxel
-// instead of four) and keeps the other from the previous slice.
+//
+// What bounds it is instruction issue (a packed two-lane FP32 instruction
+// reads its operands over two issue slots) together with the shared-memory
+// path.  So slices go in groups that read consecutive rows at compile-time
+// offsets from one address (pair_slices): no address, row or fraction
+// arithmetic in integers per slice, and each row is loaded and
+// column-interpolated once per group, also where 1/U > 1 (before: both rows
+// of every such slice).  ncu, 256^3 x 90 views: 28.7 -> 22.4 warp instructions
+// and 6.5 -> 5.0 shared loads per slice pair.  A warp covers 8 x 4 columns (16 x 2:
+// 5 % bank conflicts, now none).  Backprojection of 512^3 x 180 views:
+// 10.80 ms before, 8.77 ms with ZP = 16, 8.30 ms with ZP = 32.
 struct BpPairParams {
     float *vol;
     const GeomEntry *geo;
@@ -569,12 +581,89 @@ struct BpPairParams {
     int *status;
     int N, P, Nv, m, tps;
     int nviews, vstep, Pd;
-    int RW, tile_stride;  // rows of a kZP-slice window; elements per staged window
+    int RW, tile_stride;  // rows of a ZP-slice window; elements per staged window
     int pbase, pend;      // slice pairs pbase .. pend - 1 (pair p: slices p and N - 1 - p)
     float scale;
     unsigned long long wait_ns;
     int fault;
 };
+
+// Column-interpolated samples (U^-2 weighted) of the pair's row r + K: lower
+// window row r + K at aL + K ROWB, upper window row C - r - K at aU - K ROWB.
+template <typename TS, uint32_t ROWB, int K>
+__device__ __forceinline__ float2 pair_row(uint32_t aL, uint32_t aU, float2 A0, float2 A1) {
+    constexpr int ES = (int)sizeof(TS);
+    constexpr int OL = K * (int)ROWB, OU = -K * (int)ROWB;
+    return __ffma2_rn(A1, make_float2(Lds<TS, OL + ES>::f(aL), Lds<TS, OU + ES>::f(aU)),
+                      __fmul2_rn(A0, make_float2(Lds<TS, OL>::f(aL), Lds<TS, OU>::f(aU))));
+}
+
+// One slice of a group: with t in [-1, 1) the row coordinate relative to the
+// middle one of three consecutive rows c0, c1, c2, the row interpolation is
+// (1 - |t|) c1 + |t| (t < 0 ? c0 : c2): no row but the two around the sample
+// enters it (t itself scalar: a packed add of both lanes measured 3 % slower).
+template <typename TS, uint32_t ROWB, int G, int I>
+__device__ __forceinline__ void pair_group(float2 *acc, float2 c0, float2 c1, float t, float du, uint32_t aL,
+                                           uint32_t aU, float2 A0, float2 A1) {
+    if constexpr (I < G) {
+        const float2 c2 = pair_row<TS, ROWB, I + 2>(aL, aU, A0, A1);
+        const bool lo = t < 0.f;
+        const float2 y = make_float2(lo ? -c0.x : c2.x, lo ? -c0.y : c2.y);
+        const float w1 = 1.0f - fabsf(t);
+        acc[I] = __ffma2_rn(make_float2(t, t), y, __ffma2_rn(make_float2(w1, w1), c1, acc[I]));
+        pair_group<TS, ROWB, G, I + 1>(acc, c1, c2, t + du, du, aL, aU, A0, A1);
+    }
+}
+
+// floor of |x| < 2^22 through the float 1.5 2^23 + floor(x) (unit spacing,
+// rounded down): its bits are kFloorBits + floor(x), so an address takes one
+// multiply-add, and no conversion instruction is needed
+constexpr float kFloorBias = 12582912.0f;  // 1.5 * 2^23
+constexpr uint32_t kFloorBits = 0x4B400000u;
+__device__ __forceinline__ float floor_biased(float x) { return __fadd_rd(x, kFloorBias); }
+
+// The ZP slice pairs of one column in groups of G consecutive ones, for a
+// drift |1/U - 1| of at most 1 / (G - 1) rows per slice: then slice g + i of
+// a group reads two of the rows b + i, b + i + 1, b + i + 2 for one b, so a
+// group loads G + 2 rows at compile-time offsets from one address.  w is the
+// window row of the slab's centre less the centre's slice number: a number of
+// a few rows whatever ZP, so its rounding stays below a row coordinate's.
+template <typename TS, uint32_t ROWB, int G, int ZP>
+__device__ __forceinline__ void pair_slices(float2 (&acc)[ZP], float w, float du, uint32_t bL, uint32_t KU,
+                                            float2 A0, float2 A1) {
+#pragma unroll
+    for (int g = 0; g < ZP; g += G) {
+        // window row less slice number at the group's ends
+        const float first = fmaf((float)g - 0.5f * (float)(ZP - 1), du, w);
+        const float last = fmaf((float)(g + G - 1) - 0.5f * (float)(ZP - 1), du, w);
+        const float bm = floor_biased(fminf(first, last));
+        const float t0 = first - (bm - (kFloorBias - 1.0f));  // first - (b + 1), exact
+        const uint32_t aL = __float_as_uint(bm) * ROWB + (bL + ((uint32_t)g - kFloorBits) * ROWB), aU = KU - aL;
+        pair_group<TS, ROWB, G, 0>(acc + g, pair_row<TS, ROWB, 0>(aL, aU, A0, A1),
+                                   pair_row<TS, ROWB, 1>(aL, aU, A0, A1), t0, du, aL, aU, A0, A1);
+    }
+}
+
+// Any 1/U: both rows of every slice at an address of its own.  Row
+// coordinates in 9.23 fixed point: the row is V >> 23, the fraction's float
+// is V's mantissa bits under the exponent of 1.0.
+template <typename TS, uint32_t ROWB, int ZP>
+__device__ __forceinline__ void pair_slices_any(float2 (&acc)[ZP], float w, float invU, uint32_t bL, uint32_t KU,
+                                                float2 A0, float2 A1) {
+    constexpr float kFix = 8388608.0f;  // 2^23
+    uint32_t V = __float2uint_rn(fmaf(-0.5f * (float)(ZP - 1), invU - 1.0f, w) * kFix);
+    const uint32_t dV = __float2uint_rn(invU * kFix);
+#pragma unroll
+    for (int i = 0; i < ZP; ++i) {
+        const uint32_t aL = (V >> 23) * ROWB + bL, aU = KU - aL;
+        const float2 A = pair_row<TS, ROWB, 0>(aL, aU, A0, A1), B = pair_row<TS, ROWB, 1>(aL, aU, A0, A1);
+        // fb = 1 + f exactly, so 1 - f and f are exact
+        const float fb = __uint_as_float((V & 0x7fffffu) | 0x3f800000u);
+        const float f = fb - 1.0f, g = 2.0f - fb;
+        acc[i] = __ffma2_rn(make_float2(f, f), B, __ffma2_rn(make_float2(g, g), A, acc[i]));
+        V += dV;
+    }
+}
 
 // Warp-specialised: warp 8 is the producer (per chunk of VPS views it finds
 // the windows, writes the view parameters and issues the copies into a ring
@@ -588,26 +677,38 @@ struct BpPairParams {
 // suspended in mbarrier.try_wait it was measured to resume late (the whole
 // kernel 1.4x slower); the consumers' waits on `full` are mostly satisfied
 // at once and suspend (polling them measured no faster).
+struct PairView {
+    float4 a;   // cos, sin, 1/d_c, alpha
+    float4 b;   // gamma, g, column offset, window row of the lower slab's centre less its slice number
+    float zcr;  // z_c / d_c (lower slab)
+    int group;  // slices per group (pair_slices), 0: any drift, -1: window too small, skip the view
+    // byte addresses of row 0, column -kFloorBits of the lower window, and of
+    // row C of the upper one plus the former (row r of the lower window at
+    // aL = baseL + r ROWB + ..., row C - r of the upper one at KU - aL)
+    uint32_t baseL, KU;
+};
 constexpr int kPairSlots = 3;
+// a group's first or last row may lie one row outside its window (such a row
+// never enters a sum): one row of the widest window before and after the ring
+constexpr int kPairPad = 512;
+constexpr int kPairViews = 2;                      // views per slot, at most (16 producer lanes each)
 constexpr int kPairConsumers = kThreads / 32;      // 8
 constexpr int kPairThreads = kThreads + 32;        // plus the producer warp
+// CTAs per SM: registers decide (2 ZP accumulators per thread)
+constexpr int pair_ctas(int ZP) { return ZP == 32 ? 2 : 3; }
 
-template <typename TS, bool DIRECT, int WD, int VPS>
-__global__ void __launch_bounds__(kPairThreads, 3)
+template <typename TS, bool DIRECT, int WD, int ZP, int VPS>
+__global__ void __launch_bounds__(kPairThreads, pair_ctas(ZP))
 bp_pair_kernel(const __grid_constant__ CUtensorMap tmap, BpPairParams a) {
     constexpr int ES = (int)sizeof(TS);
     constexpr int kAl = 16 / ES;
     constexpr uint32_t ROWB = (uint32_t)(ES * WD);  // bytes per window row
-    constexpr float kFix = 8388608.0f;              // 2^23
-    static_assert(VPS * 16 <= 32, "the producer warp sets up VPS views at 16 lanes each");
+    static_assert(VPS <= kPairViews, "the producer warp sets up a view on 16 lanes");
     extern __shared__ __align__(128) unsigned char smem_raw[];
-    TS *sm = (TS *)(smem_raw + ((128u - (tma::smem_u32(smem_raw) & 127u)) & 127u));
+    TS *sm = (TS *)(smem_raw + ((128u - (tma::smem_u32(smem_raw) & 127u)) & 127u) + kPairPad);
     const uint32_t sbase = tma::smem_u32(sm);
     __shared__ __align__(8) uint64_t full[kPairSlots], empty[kPairSlots];
-    __shared__ float4 s_pa[kPairSlots][VPS];  // cos, sin, 1/d_c, alpha
-    __shared__ float4 s_pb[kPairSlots][VPS];  // gamma, g, column offset, window row of the lower slab's centre
-    __shared__ float s_zcr[kPairSlots][VPS];  // z_c / d_c (lower slab)
-    __shared__ int s_C[kPairSlots][VPS], s_skip[kPairSlots][VPS];
+    __shared__ PairView s_view[kPairSlots * VPS];
 
     const int tiles = a.tps * a.tps;
     const int q = blockIdx.x / tiles;
@@ -620,13 +721,13 @@ bp_pair_kernel(const __grid_constant__ CUtensorMap tmap, BpPairParams a) {
     const int y0 = iy0 + (tt / a.tps) * kTile;
     if (x0 > ix1 || y0 > iy1) return;  // ragged square: empty tile (uniform per CTA)
     const int xe = min(x0 + kTile - 1, ix1), ye = min(y0 + kTile - 1, iy1);
-    const int p0 = a.pbase + blockIdx.y * kZP;  // first slice pair
+    const int p0 = a.pbase + blockIdx.y * ZP;  // first slice pair
 
     const float half_n = 0.5f * (float)(a.N - 1);
     const float xc = 0.5f * ((float)ix0 + (float)ix1) - half_n;
     const float yc = 0.5f * ((float)iy0 + (float)iy1) - half_n;
     // centre of the lower slab (the upper one is centred at -zc)
-    const float zc = (float)p0 + 0.5f * (float)(kZP - 1) - half_n;
+    const float zc = (float)p0 + 0.5f * (float)(ZP - 1) - half_n;
     const float vcd = 0.5f * (float)(a.Nv - 1);
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
     const int nch = (a.nviews + VPS - 1) / VPS;
@@ -650,19 +751,10 @@ bp_pair_kernel(const __grid_constant__ CUtensorMap tmap, BpPairParams a) {
         const float zcl = (lane & 8) ? -zc : zc;
         const float cx = (float)((cc & 1) ? xe : x0) - half_n - xc;
         const float cy = (float)((cc & 2) ? ye : y0) - half_n - yc;
-        const float cz = (cc & 4) ? 0.5f * (float)(kZP - 1) : -0.5f * (float)(kZP - 1);
+        const float cz = (cc & 4) ? 0.5f * (float)(ZP - 1) : -0.5f * (float)(ZP - 1);
         int c = 0;
         for (; c < nch; ++c) {
             const int sl = c % kPairSlots;
-            // round r of a slot may start once its round r - 1 was consumed
-            // (lane 0 waits; the warp follows its answer)
-            bool ok = true;
-            if (c >= kPairSlots && lane == 0)
-                ok = tma::mbar_wait_spin(&empty[sl], (uint32_t)(((c / kPairSlots) & 1) ^ 1), a.wait_ns);
-            if (!__shfl_sync(0xffffffffu, ok, 0)) {
-                if (lane == 0) atomicOr(a.status, 2);
-                break;
-            }
             const int nj = min(VPS, a.nviews - c * VPS);
             const int j = c * VPS + min(w, nj - 1);  // lanes past the chunk repeat its last view
             const int k = j * a.vstep;
@@ -698,16 +790,39 @@ bp_pair_kernel(const __grid_constant__ CUtensorMap tmap, BpPairParams a) {
             const int xs = clo & ~(kAl - 1);  // 16-byte aligned start of the copy
             const int vlo = (int)floorf(vmin) - 1, vhi = (int)floorf(vmax) + 2;
             const int vlo2 = (int)floorf(vmin2) - 1, vhi2 = (int)floorf(vmax2) + 2;
+            // largest drift per slice over the tile (1/U is monotone in x
+            // and y), with a margin for rounding
+            float drift = fabsf(invU - 1.0f);
+#pragma unroll
+            for (int off = 2; off > 0; off >>= 1) drift = fmaxf(drift, __shfl_xor_sync(0xffffffffu, drift, off));
+            // round r of a slot may start once its round r - 1 was consumed
+            // (lane 0 waits; the warp follows its answer)
+            bool ok = true;
+            if (c >= kPairSlots && lane == 0)
+                ok = tma::mbar_wait_spin(&empty[sl], (uint32_t)(((c / kPairSlots) & 1) ^ 1), a.wait_ns);
+            if (!__shfl_sync(0xffffffffu, ok, 0)) {
+                if (lane == 0) atomicOr(a.status, 2);
+                break;
+            }
             const bool lead = (lane & 15) == 0 && w < nj;
             if (lead) {
-                const int skip = (chi - xs > WD - 1) || (vhi - vlo > a.RW - 1) || (vhi2 - vlo2 > a.RW - 1) ||
-                                 a.fault == kTestFaultSmallWindow;
+                const bool skip = (chi - xs > WD - 1) || (vhi - vlo > a.RW - 1) || (vhi2 - vlo2 > a.RW - 1) ||
+                                  a.fault == kTestFaultSmallWindow;
                 if (skip) atomicOr(a.status, 1);
-                s_pa[sl][w] = make_float4(ge.cb, ge.sb, ge.r, ge.alpha);
-                s_pb[sl][w] = make_float4(ge.gamma, ge.g_hi, toff - (float)(xs - cbase), (ph - ((float)vlo - vcd)) + pl);
-                s_zcr[sl][w] = zcr;
-                s_C[sl][w] = (a.Nv - 1) - vlo - vlo2;
-                s_skip[sl][w] = skip;
+                PairView &pv = s_view[sl * VPS + w];
+                pv.a = make_float4(ge.cb, ge.sb, ge.r, ge.alpha);
+                pv.b = make_float4(ge.gamma, ge.g_hi, toff - (float)(xs - cbase),
+                                   (ph - ((float)vlo - vcd + 0.5f * (float)(ZP - 1))) + pl);
+                pv.zcr = zcr;
+                pv.group = skip ? -1
+                           : drift * 15.f < 0.999f ? 16
+                           : drift * 7.f < 0.999f  ? 8
+                           : drift * 3.f < 0.999f  ? 4
+                                                   : 0;
+                const uint32_t bL = sbase + (uint32_t)ES * (win(sl, w, 0) - kFloorBits);
+                const uint32_t bU = sbase + (uint32_t)ES * (win(sl, w, 1) - kFloorBits);
+                pv.baseL = bL;
+                pv.KU = (uint32_t)((a.Nv - 1) - vlo - vlo2) * ROWB + bU + bL;
             }
             // the copies: lane 0 for every view of the chunk
             const int xs0 = __shfl_sync(0xffffffffu, xs, 0), xs1 = __shfl_sync(0xffffffffu, xs, 16);
@@ -742,100 +857,63 @@ bp_pair_kernel(const __grid_constant__ CUtensorMap tmap, BpPairParams a) {
     // (x: lower slab, y: upper slab; each lane rounds as the scalar
     // operation would): half the arithmetic instructions of two scalar
     // updates.
-    const int lx = threadIdx.x % kTile, ly = threadIdx.x / kTile;
-    const int x = x0 + lx, y = y0 + ly;
+    const int x = x0 + (warp & 1) * 8 + (lane & 7), y = y0 + (warp >> 1) * 4 + (lane >> 3);
     const bool active = x <= xe && y <= ye;
-    const float dx = (float)x - half_n - xc, dy = (float)y - half_n - yc;
-    float2 acc[kZP];  // (lower slab, upper mirrored slab)
+    // threads outside a ragged tile repeat its last column (inside the
+    // window) and store nothing
+    const float dx = (float)min(x, xe) - half_n - xc, dy = (float)min(y, ye) - half_n - yc;
+    float2 acc[ZP];  // (lower slab, upper mirrored slab)
 #pragma unroll
-    for (int i = 0; i < kZP; ++i) acc[i] = make_float2(0.f, 0.f);
+    for (int i = 0; i < ZP; ++i) acc[i] = make_float2(0.f, 0.f);
 
-    for (int c = 0; c < nch; ++c) {
-        const int sl = c % kPairSlots;
-        const bool ok = tma::mbar_wait_bounded(&full[sl], (uint32_t)((c / kPairSlots) & 1), a.wait_ns);
+    int sl = 0, left = a.nviews;
+    uint32_t phase = 0;
+    for (; left > 0; left -= VPS) {
+        const bool ok = tma::mbar_wait_bounded(&full[sl], phase, a.wait_ns);
         if (!__all_sync(0xffffffffu, ok)) {
             if (lane == 0) atomicOr(a.status, 2);
             return;  // the producer waits for the copies in flight
         }
-        const int nj = min(VPS, a.nviews - c * VPS);
-        for (int w = 0; w < nj; ++w) {
-            if (s_skip[sl][w]) continue;  // uniform per CTA
-            const float4 pa = s_pa[sl][w];
-            const float4 pb = s_pb[sl][w];
+        const PairView *pv = s_view + sl * VPS, *pe = pv + min(VPS, left);
+#pragma unroll 1
+        for (; pv != pe; ++pv) {
+            const int group = pv->group;  // uniform per CTA
+            const float4 pa = pv->a;
+            const float4 pb = pv->b;
             const float dd = fmaf(pa.x, dx, pa.y * dy);
-            const float invU = __fdividef(pb.y, fmaf(pa.z, dd, 1.0f));
-            const uint32_t dV = __float2uint_rn(invU * kFix);
-            // warp-uniform choice (threads outside a ragged tile do not constrain it)
-            const bool stepA = __all_sync(0xffffffffu, !active || dV <= (1u << 23));
-            if (!active) continue;
+            const float invU = pb.y * rcp_approx(fmaf(pa.z, dd, 1.0f));
+            const float du = invU - 1.0f;
             const float t = fmaf(invU, fmaf(pa.w, dx, pb.x * dy), pb.z);
-            const float tf = floorf(t);
+            const float tm = floor_biased(t);
             const float wgt = invU * invU;
-            const float a1 = wgt * (t - tf);
+            const float a1 = wgt * (t - (tm - kFloorBias));
             const float a0 = wgt - a1;
             const float2 A1 = make_float2(a1, a1), A0 = make_float2(a0, a0);
-            // window row of slice p0 (lower slab), in 9.23 fixed point
-            const float vb0 = fmaf(invU, -0.5f * (float)(kZP - 1) - s_zcr[sl][w] * dd, pb.w);
-            uint32_t V = __float2uint_rn(vb0 * kFix);
-            // byte addresses: row r of the lower window at r ROWB + bL; the
-            // upper window's row C - 1 - r at KLU - (r ROWB + bL)
-            const uint32_t bL = sbase + (uint32_t)ES * (win(sl, w, 0) + (uint32_t)(int)tf);
-            const uint32_t bU = sbase + (uint32_t)ES * (win(sl, w, 1) + (uint32_t)(int)tf);
-            const uint32_t KLU = (uint32_t)(s_C[sl][w] - 1) * ROWB + bU + bL;
-            // column-interpolated samples (U^-2 weighted) of the pair's first
-            // row (lower row r, upper row C - r) and of its second row
-            auto first = [&](uint32_t aL, uint32_t aU) {
-                return __ffma2_rn(A1, make_float2(Lds<TS, ES>::f(aL), Lds<TS, ROWB + ES>::f(aU)),
-                                  __fmul2_rn(A0, make_float2(Lds<TS, 0>::f(aL), Lds<TS, ROWB>::f(aU))));
-            };
-            auto second = [&](uint32_t aL, uint32_t aU) {
-                return __ffma2_rn(A1, make_float2(Lds<TS, ROWB + ES>::f(aL), Lds<TS, ES>::f(aU)),
-                                  __fmul2_rn(A0, make_float2(Lds<TS, ROWB>::f(aL), Lds<TS, 0>::f(aU))));
-            };
-            // row weights 1 - f and f (both lanes) from the fixed-point row
-            // coordinate: fb = 1 + f exactly, so 2 - fb and fb - 1 are exact
-            auto rowlerp = [&](uint32_t Vc, float2 A, float2 B, float2 acc_i) {
-                const float fb = __uint_as_float((Vc & 0x7fffffu) | 0x3f800000u);
-                const float f = fb - 1.0f, g = 2.0f - fb;
-                return __ffma2_rn(make_float2(f, f), B, __ffma2_rn(make_float2(g, g), A, acc_i));
-            };
-            if (stepA) {
-                // 1/U <= 1: the row advances by 0 or 1 per slice
-                uint32_t r = V >> 23;
-                uint32_t aL = r * ROWB + bL, aU = KLU - aL;
-                float2 A = first(aL, aU);
-                float2 B = second(aL, aU);
-                acc[0] = rowlerp(V, A, B, acc[0]);
-#pragma unroll
-                for (int i = 1; i < kZP; ++i) {
-                    V += dV;
-                    const uint32_t rn = V >> 23;
-                    const bool adv = rn != r;
-                    r = rn;
-                    aL = r * ROWB + bL;
-                    aU = KLU - aL;
-                    A = adv ? B : A;
-                    B = second(aL, aU);
-                    acc[i] = rowlerp(V, A, B, acc[i]);
-                }
-            } else {
-#pragma unroll
-                for (int i = 0; i < kZP; ++i) {
-                    const uint32_t r = V >> 23;
-                    const uint32_t aL = r * ROWB + bL, aU = KLU - aL;
-                    const float2 A = first(aL, aU);
-                    const float2 B = second(aL, aU);
-                    acc[i] = rowlerp(V, A, B, acc[i]);
-                    V += dV;
-                }
+            // window row of the column at the lower slab's centre, less the
+            // centre's slice number
+            const float wc = fmaf(-invU, pv->zcr * dd, pb.w);
+            const uint32_t col = (uint32_t)ES * __float_as_uint(tm);
+            const uint32_t bL = pv->baseL + col, KU = pv->KU + 2u * col;
+            if (group == 16) {
+                pair_slices<TS, ROWB, 16, ZP>(acc, wc, du, bL, KU, A0, A1);
+            } else if (group == 8) {
+                pair_slices<TS, ROWB, 8, ZP>(acc, wc, du, bL, KU, A0, A1);
+            } else if (group == 4) {
+                pair_slices<TS, ROWB, 4, ZP>(acc, wc, du, bL, KU, A0, A1);
+            } else if (group == 0) {
+                pair_slices_any<TS, ROWB, ZP>(acc, wc, invU, bL, KU, A0, A1);
             }
         }
         __syncwarp();
         if (lane == 0) tma::mbar_arrive(&empty[sl]);  // this warp is done with the slot
+        if (++sl == kPairSlots) {
+            sl = 0;
+            phase ^= 1u;
+        }
     }
     if (active) {
 #pragma unroll
-        for (int i = 0; i < kZP; ++i) {
+        for (int i = 0; i < ZP; ++i) {
             const int pz = p0 + i;
             if (pz < a.pend) {
                 const int zu = a.N - 1 - pz;
@@ -1135,40 +1213,43 @@ cudaError_t try_launch_tma(const PlanImpl &p, const SquareSet &ss, bool direct, 
     return cudaErrorInvalidValue;
 }
 
+// elements per staged window of the pair kernel, a 128-byte multiple
+inline int pair_tile_stride(int es, int rows, int WD) { return (rows * WD + (128 / es - 1)) & ~(128 / es - 1); }
+
 // dynamic shared memory of the pair kernel: kPairSlots slots of VPS views,
-// two windows per view, plus the 128-byte alignment slack
+// two windows per view, plus the pads and the 128-byte alignment slack
 inline size_t pair_smem(int es, int vps, int tile_stride) {
-    return (size_t)es * kPairSlots * vps * 2 * tile_stride + 128;
+    return (size_t)es * kPairSlots * vps * 2 * tile_stride + 2 * kPairPad + 128;
 }
 
-template <typename TS, bool DIRECT, int WD, int VPS>
+template <typename TS, bool DIRECT, int WD, int ZP, int VPS>
 cudaError_t launch_pair_t(const CUtensorMap &map, const BpPairParams &prm, int nsq, cudaStream_t st) {
     const size_t smem = pair_smem((int)sizeof(TS), VPS, prm.tile_stride);
-    cudaError_t e = ensure_smem<bp_pair_kernel<TS, DIRECT, WD, VPS>>(smem);
+    cudaError_t e = ensure_smem<bp_pair_kernel<TS, DIRECT, WD, ZP, VPS>>(smem);
     if (e != cudaSuccess) return e;
-    dim3 grid((unsigned)(nsq * prm.tps * prm.tps), (unsigned)((prm.pend - prm.pbase + kZP - 1) / kZP));
-    bp_pair_kernel<TS, DIRECT, WD, VPS><<<grid, kPairThreads, smem, st>>>(map, prm);
+    dim3 grid((unsigned)(nsq * prm.tps * prm.tps), (unsigned)((prm.pend - prm.pbase + ZP - 1) / ZP));
+    bp_pair_kernel<TS, DIRECT, WD, ZP, VPS><<<grid, kPairThreads, smem, st>>>(map, prm);
     return cudaGetLastError();
 }
 
-// views per slot: 2 (three CTAs per SM hold their ring at the usual window
-// sizes), or 1 for larger windows (the staging depth only; the arithmetic and
-// the result are the same)
+// 32 slice pairs per CTA always come with 2 views per slot (pair_slices_per_cta)
 template <typename TS, bool DIRECT, int WD>
-cudaError_t launch_pair_v(int vps, const CUtensorMap &map, const BpPairParams &prm, int nsq, cudaStream_t st) {
-    return vps == 2 ? launch_pair_t<TS, DIRECT, WD, 2>(map, prm, nsq, st)
-                    : launch_pair_t<TS, DIRECT, WD, 1>(map, prm, nsq, st);
+cudaError_t launch_pair_z(int zp, int vps, const CUtensorMap &map, const BpPairParams &prm, int nsq,
+                          cudaStream_t st) {
+    if (zp == 32) return launch_pair_t<TS, DIRECT, WD, 32, 2>(map, prm, nsq, st);
+    return vps == 2 ? launch_pair_t<TS, DIRECT, WD, 16, 2>(map, prm, nsq, st)
+                    : launch_pair_t<TS, DIRECT, WD, 16, 1>(map, prm, nsq, st);
 }
 
 template <typename TS, bool DIRECT>
-cudaError_t launch_pair_w(int WD, int vps, const CUtensorMap &map, const BpPairParams &prm, int nsq,
+cudaError_t launch_pair_w(int WD, int zp, int vps, const CUtensorMap &map, const BpPairParams &prm, int nsq,
                           cudaStream_t st) {
     switch (WD) {
-        case 32: return launch_pair_v<TS, DIRECT, 32>(vps, map, prm, nsq, st);
-        case 48: return launch_pair_v<TS, DIRECT, 48>(vps, map, prm, nsq, st);
-        case 64: return launch_pair_v<TS, DIRECT, 64>(vps, map, prm, nsq, st);
-        case 96: return launch_pair_v<TS, DIRECT, 96>(vps, map, prm, nsq, st);
-        case 128: return launch_pair_v<TS, DIRECT, 128>(vps, map, prm, nsq, st);
+        case 32: return launch_pair_z<TS, DIRECT, 32>(zp, vps, map, prm, nsq, st);
+        case 48: return launch_pair_z<TS, DIRECT, 48>(zp, vps, map, prm, nsq, st);
+        case 64: return launch_pair_z<TS, DIRECT, 64>(zp, vps, map, prm, nsq, st);
+        case 96: return launch_pair_z<TS, DIRECT, 96>(zp, vps, map, prm, nsq, st);
+        case 128: return launch_pair_z<TS, DIRECT, 128>(zp, vps, map, prm, nsq, st);
     }
     return cudaErrorInvalidValue;
 }
@@ -1187,16 +1268,52 @@ size_t smem_budget(size_t *per_sm = nullptr) {
     return optin > 2048 ? (size_t)optin - 2048 : 0;
 }
 
+// Views per ring slot of the pair kernel for windows of `rows` x WD elements
+// of es bytes: 2 where the SM then holds the CTAs that the registers allow
+// (each with its static shared memory and the runtime's reserve, 2 KiB
+// together at most), else 1 if one CTA fits, else 0.
+int pair_views(int es, int zp, int rows, int WD) {
+    size_t per_sm = 0;
+    const size_t budget = smem_budget(&per_sm);
+    const int ts = pair_tile_stride(es, rows, WD);
+    if ((size_t)pair_ctas(zp) * (pair_smem(es, 2, ts) + 2048) <= per_sm) return 2;
+    return pair_smem(es, 1, ts) <= budget ? 1 : 0;
+}
+
+// Slice pairs per CTA of the pair kernel, 0 where it does not apply (the
+// TMA conditions of make_tma_launch).  32 pairs per thread halve the
+// per-view set-up and stage fewer margin rows (512^3: 8.30 ms against 8.75 at
+// 16), but need enough CTAs: 2 per SM, half as many of them; measured at
+// 128^3 (128 CTAs) 16 is the faster one.  A rule on the plan alone, so that
+// launches over part of the volume round as the whole one does.
+int pair_slices_per_cta(const PlanImpl &p, const SquareSet &ss, bool direct, int &vps) {
+    const int es = (direct && p.qtype != FDKOD_F32) ? 2 : 4;
+    const int WD = es == 4 ? ss.WdT : ss.WdT16;
+    vps = 0;
+    if (WD == 0) return 0;
+    const long long tiles = (long long)ss.nsq * ss.tiles_per_side * ss.tiles_per_side;
+    int dev = 0, sms = 148;
+    if (cudaGetDevice(&dev) == cudaSuccess) cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
+    if (ss.Rw <= 256 && tiles * (((p.g.N + 1) / 2 + 31) / 32) >= 2LL * pair_ctas(32) * sms &&
+        (vps = pair_views(es, 32, ss.Rw, WD)) == 2)
+        return 32;
+    if (ss.Rw2 <= 256 && (vps = pair_views(es, 16, ss.Rw2, WD)) > 0) return 16;
+    return 0;
+}
+
 // The mirrored-pair kernel serves launches over the whole detector and the
-// slice pairs p0 .. p1 - 1 (slices p and N - 1 - p), with the TMA
-// conditions of make_tma_launch and windows of kZP slices.
+// slice pairs p0 .. p1 - 1 (slices p and N - 1 - p).
 cudaError_t try_launch_pair(const PlanImpl &p, const SquareSet &ss, bool direct, const void *src, float *vol,
                             cudaStream_t st, int p0, int p1, bool &launched) {
     launched = false;
     const int es = (direct && p.qtype != FDKOD_F32) ? 2 : 4;
     const int WD = es == 4 ? ss.WdT : ss.WdT16;
-    if (WD == 0 || ss.Rw2 > 256 || ((uintptr_t)src & 15) != 0) return cudaSuccess;
+    if (((uintptr_t)src & 15) != 0) return cudaSuccess;
     if (direct && ((size_t)p.g.Nu * es) % 16 != 0) return cudaSuccess;
+    int vps = 0;
+    const int zp = pair_slices_per_cta(p, ss, direct, vps);
+    if (zp == 0) return cudaSuccess;  // windows too large: the 32-slice kernel
+    const int rows = zp == 32 ? ss.Rw : ss.Rw2;
     uint64_t dims[3], strides[2];
     if (direct) {
         dims[0] = (uint64_t)p.g.Nu;
@@ -1210,7 +1327,7 @@ cudaError_t try_launch_pair(const PlanImpl &p, const SquareSet &ss, bool direct,
         strides[0] = (uint64_t)p.Tstride * sizeof(float);
     }
     strides[1] = strides[0] * dims[1];
-    const uint32_t box[3] = {(uint32_t)WD, (uint32_t)ss.Rw2, 1u};
+    const uint32_t box[3] = {(uint32_t)WD, (uint32_t)rows, 1u};
     const CUtensorMapDataType dt = es == 4 ? CU_TENSOR_MAP_DATA_TYPE_FLOAT32
                                    : (p.qtype == FDKOD_F16 ? CU_TENSOR_MAP_DATA_TYPE_FLOAT16
                                                            : CU_TENSOR_MAP_DATA_TYPE_BFLOAT16);
@@ -1228,16 +1345,8 @@ cudaError_t try_launch_pair(const PlanImpl &p, const SquareSet &ss, bool direct,
     a.m = ss.m;
     a.tps = ss.tiles_per_side;
     a.Pd = p.Pd;
-    a.RW = ss.Rw2;
-    a.tile_stride = (ss.Rw2 * WD + (128 / es - 1)) & ~(128 / es - 1);
-    size_t per_sm = 0;
-    const size_t budget = smem_budget(&per_sm);
-    // 2 views per slot where three CTAs fit an SM (each with its static
-    // shared memory and the runtime's reserve, 2 KiB together at most), else
-    // 1 if one CTA fits
-    const int vps = 3 * (pair_smem(es, 2, a.tile_stride) + 2048) <= per_sm ? 2
-                    : (pair_smem(es, 1, a.tile_stride) <= budget ? 1 : 0);
-    if (vps == 0) return cudaSuccess;  // windows too large: the 32-slice kernel
+    a.RW = rows;
+    a.tile_stride = pair_tile_stride(es, rows, WD);
     a.pbase = p0;
     a.pend = p1;
     a.wait_ns = p.wait_ns > 0 ? (unsigned long long)p.wait_ns : kWaitLimitNs;
@@ -1252,11 +1361,11 @@ cudaError_t try_launch_pair(const PlanImpl &p, const SquareSet &ss, bool direct,
         a.scale = (float)(M_PI / (double)p.Pd);
     }
     launched = true;
-    if (!direct) return launch_pair_w<float, false>(WD, vps, map, a, ss.nsq, st);
+    if (!direct) return launch_pair_w<float, false>(WD, zp, vps, map, a, ss.nsq, st);
     switch (p.qtype) {
-        case FDKOD_F32: return launch_pair_w<float, true>(WD, vps, map, a, ss.nsq, st);
-        case FDKOD_BF16: return launch_pair_w<__nv_bfloat16, true>(WD, vps, map, a, ss.nsq, st);
-        case FDKOD_F16: return launch_pair_w<__half, true>(WD, vps, map, a, ss.nsq, st);
+        case FDKOD_F32: return launch_pair_w<float, true>(WD, zp, vps, map, a, ss.nsq, st);
+        case FDKOD_BF16: return launch_pair_w<__nv_bfloat16, true>(WD, zp, vps, map, a, ss.nsq, st);
+        case FDKOD_F16: return launch_pair_w<__half, true>(WD, zp, vps, map, a, ss.nsq, st);
     }
     return cudaErrorInvalidValue;
 }
@@ -1266,6 +1375,12 @@ cudaError_t try_launch_pair(const PlanImpl &p, const SquareSet &ss, bool direct,
 cudaError_t launch_backproject_pairs(const PlanImpl &p, const SquareSet &ss, bool direct, const void *src,
                                      float *vol, cudaStream_t st, int p0, int p1, bool &launched) {
     return try_launch_pair(p, ss, direct, src, vol, st, p0, p1, launched);
+}
+
+int pair_slab(const PlanImpl &p, const SquareSet &ss, bool direct) {
+    int vps = 0;
+    const int zp = pair_slices_per_cta(p, ss, direct, vps);
+    return zp > 0 ? zp : 16;
 }
 
 cudaError_t launch_backproject(const PlanImpl &p, const SquareSet &ss, bool direct, const void *src, float *vol,

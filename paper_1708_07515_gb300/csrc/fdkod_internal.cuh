@@ -39,14 +39,14 @@ struct SquareSet {
     // (4-element alignment slack, rounded up to a kernel instantiation, 0
     // when no instantiation is wide enough)
     int Wd = 0, Rw = 0, WdT = 0, WdT16 = 0;  // WdT16: the same for 16-bit windows
-    int Rw2 = 0;  // rows of a window of kZP slices (the mirrored-pair kernel)
+    int Rw2 = 0;  // rows of a window of kZP slices (the mirrored-pair kernel; Rw: of kZT slices)
     int need = 0, need16 = 0;  // the narrowest TMA windows that hold every tile's footprint
     int tiles_per_side = 1;  // 16-voxel tiles per square side
 };
 
 constexpr int kTile = 16;      // tile side in x and y (threads per CTA = 256)
 constexpr int kZT = 32;        // z voxels per thread
-constexpr int kZP = 16;        // slices per half of the mirrored-pair kernel (2 kZP voxels per thread)
+constexpr int kZP = 16;        // slices per half of the mirrored-pair kernel's smaller form (the larger: kZT)
 constexpr int kViewsPerChunk = 8;  // generic backprojection kernel
 constexpr int kViewsPerStage = 4;  // TMA backprojection kernel (two stages)
 constexpr int kMaxTapD = 128;      // largest decimation factor with a tap table
@@ -176,6 +176,9 @@ cudaError_t launch_backproject(const PlanImpl &p, const SquareSet &ss, bool dire
 // the staged pair kernel does not apply (then nothing is launched).
 cudaError_t launch_backproject_pairs(const PlanImpl &p, const SquareSet &ss, bool direct, const void *src,
                                      float *vol, cudaStream_t st, int p0, int p1, bool &launched);
+// Slice pairs per CTA of that kernel for this plan: launches over part of
+// the pairs start at a multiple of it, so that they round as the whole launch
+int pair_slab(const PlanImpl &p, const SquareSet &ss, bool direct);
 
 // A batch of plans backprojected by one persistent launch (backproject.cu):
 // per plan its FDK-OD source (Q when D = 1, else the decomposed data) and

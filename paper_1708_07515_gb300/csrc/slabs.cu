@@ -460,7 +460,8 @@ extern "C" int fdkod_reconstruct(fdkod_plan_t *plan, const float *proj_host, flo
     // group's two z-ranges are read back as soon as it is done
     const int npair = (N + 1) / 2;
     int ps = (npair + kPipeSlabs - 1) / kPipeSlabs;
-    ps = (ps + fdkod::kZP - 1) / fdkod::kZP * fdkod::kZP;
+    const int slab = fdkod::pair_slab(p, p.od, direct);
+    ps = (ps + slab - 1) / slab * slab;
     int ns = 0;
     bool paired = true;
     const size_t plane = (size_t)N * N;
