@@ -881,7 +881,10 @@ bp_pair_kernel(const __grid_constant__ CUtensorMap tmap, BpPairParams a) {
             const float4 pa = pv->a;
             const float4 pb = pv->b;
             const float dd = fmaf(pa.x, dx, pa.y * dy);
-            const float invU = pb.y * rcp_approx(fmaf(pa.z, dd, 1.0f));
+            // one Newton step on the reciprocal: its error scales with the
+            // distance from the slab's centre, which 32 pairs double
+            const float den = fmaf(pa.z, dd, 1.0f), r0 = rcp_approx(den);
+            const float invU = pb.y * fmaf(r0, fmaf(-den, r0, 1.0f), r0);
             const float du = invU - 1.0f;
             const float t = fmaf(invU, fmaf(pa.w, dx, pb.x * dy), pb.z);
             const float tm = floor_biased(t);
