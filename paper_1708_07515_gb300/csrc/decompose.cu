@@ -14,11 +14,10 @@
 #include <cuda_bf16.h>
 #include <cuda_fp16.h>
 
+#include <algorithm>
 #include <type_traits>
-#include <utility>
 
 #include "fdkod_internal.cuh"
-#include "packed.cuh"
 #include "tma.cuh"
 
 namespace fdkod {
@@ -90,227 +89,207 @@ decompose_kernel(const TQ *__restrict__ Q, float *__restrict__ Sp, const int32_t
 
 
 // ---------------------------------------------------------------------------
-// TMA path: one CTA per (square q, band of VB detector rows), warp
-// specialised.  The producer warp's lane 0 brings each view's crop box
-// (VB rows x Wc columns starting at the 16-byte aligned column below
-// crop[q][k]) into a ring of kStages slots of kG views (Ring<TQ>) with 3D
-// bulk-tensor copies (zero fill outside the detector); slot n is full when
-// its bytes have landed (mbarrier full[n]) and free again when all consumer
-// warps have arrived on empty[n].  No block-wide barrier inside the view loop.
+// TMA path: one CTA per (square q, band of detector rows, range of decimated
+// views), warp specialised.  The producer warp's lane 0 brings each view's
+// crop box (the band's rows x Wc columns from the 16-byte aligned column
+// below crop[q][k]) into a ring of slots of kG views with 3D bulk-tensor copies
+// (zero fill outside the detector); slot n is full when its bytes have landed
+// (mbarrier full[n]) and free again when all consumer warps have arrived on
+// empty[n].  No block-wide barrier inside the view loop.
 //
-// Consumers: the 32 lanes of a warp share its rows (rows_per_lane adjacent
-// detector rows) and lane l owns the columns l, l + 32, ... (C of them), so
-// per view and column a lane makes two scalar shared loads at the crop's
-// offset inside its aligned box plus compile-time offsets -- consecutive
-// lanes read consecutive elements, free of bank conflicts for every offset
-// -- one lerp and the 2H tap FMAs; the per-view bookkeeping is shared by the
-// lane's rows and columns.  (Lanes that owned C consecutive columns loaded
-// them as aligned vectors and picked the offset's code path per view: about
-// 20 instructions per shifted sample, issue-bound.)  Everything else
-// a view needs -- shift fraction, which tap weights apply and whether a
-// decimated view is complete -- is one 8-byte entry of a per-CTA table in
-// stream order, built once from crop[q][.] and frac[q][.], plus the weights
-// w[r] of its block offset r (one 16-byte entry per r).
+// Consumers: lane = detector row, and each warp owns kCW consecutive shifted
+// columns of its 32 rows, so a sample is loaded once and serves as the right
+// neighbour of one column and the left one of the next: kCW + 1 samples per
+// kCW columns, in aligned 16-byte loads.  The box's rows are an odd number
+// of 16-byte units long, which keeps those loads free of bank conflicts; the
+// crop's offset inside its aligned box is the same for all rows, so it picks
+// one of the unrolled bodies (a uniform branch).  Per view and lane: 5 (16-bit
+// Q: 3) loads, kCW lerps and kCW 2H tap FMAs.  A finished decimated view goes
+// through a per-warp transpose buffer, so that its rows leave in 64-byte runs.
+//
+// What bounds it: instruction issue, with the L2 -> shared traffic of the
+// crops (~14 |Q|) close behind.  The form before had lanes along the columns:
+// two scalar loads per sample, and columns in steps of 32 lanes (128 computed
+// for ~100 used).
+//
+// Everything else a view needs -- shift fraction, tap weights, crop offset --
+// is one 16-byte entry of a per-CTA table in stream order (H = 2: 8 more bytes
+// of weights), built once.  Views go block by block (D views): a block's end
+// completes a decimated view and moves the running sums on.
 
-constexpr int kConsumerWarps = 8;
-// adjacent detector rows per lane (the per-view bookkeeping -- table loads,
-// slot waits, decimated-view stores -- is shared by them): four with the
-// triangle's two running sums, two with the four of 2D-tap filters
-// (registers; measured: 2 -> 4 rows took 1.63 -> 1.48 ms at 512^3); half of
-// that where the launch would not fill two waves of the GPU (short row bands)
-__host__ __device__ constexpr int rows_per_lane(int H, bool wide = true) {
-    return (H == 1 ? 4 : 2) / (wide ? 1 : 2);
-}
-// ring shape per element type (measured): slots of kG views, kStages slots
+constexpr int kCW = 16;       // shifted columns per warp
+constexpr int kTP = kCW + 4;  // row pitch of the transpose buffer (floats; 5 16-byte units: no conflicts)
+constexpr int kDecMaxSegs = 8;  // column segments (consumer warps) per CTA; wider squares take several CTAs
+// ring shape per element type (measured at 512^3 f32 and 2000^3 bf16: slots of
+// one view 1.11 and 5.62 ms, of two views 1.40 and 5.37 ms; what counts most is
+// that three CTAs fit an SM)
 template <typename TQ>
 struct Ring {
-    static constexpr int kG = sizeof(TQ) == 4 ? 2 : 4;
-    static constexpr int kStages = 3;
+    static constexpr int kG = sizeof(TQ) == 4 ? 1 : 2, kStages = sizeof(TQ) == 4 ? 3 : 2;
 };
-constexpr int kDecThreads = 32 * (kConsumerWarps + 1);
-// bytes after the ring: a lane's columns run up to 32 C + 1 elements (plus
-// the crop's offset, < 16 bytes) past its row's start, beyond the last row's
-// Wc columns; rounded up to 128 bytes so the tables behind it (float4 and
-// float2 entries) stay aligned
-__host__ __device__ constexpr int kColSlack(int C) { return (4 * (32 * C + 1) + 16 + 127) & ~127; }
-static_assert(kColSlack(1) % 16 == 0 && kColSlack(8) % 16 == 0, "table alignment");
+constexpr int kRingSlack = 128;  // the last segment's loads run up to 16 bytes past a row's end
 constexpr uint64_t kDecWaitNs = 2000000000ull;
 
-// code word of a table entry: bits 0-2 the crop's offset inside its aligned
-// box, bit 3 "last view of a decimated block" (rotate the running sums),
-// bits 4-11 the block offset r (its weights), bits 12.. the decimated view
-// to store plus one (0: none, a view before view 0).  D <= 128.
-constexpr int kCodeRotate = 8, kCodeTapShift = 4, kCodeStoreShift = 12;
-
-// Per-CTA tables over the stream positions pos = 0 .. P + (2H - 1) D - 2
-// (view k' = pos - (H D - 1), taken mod P): s_fc[pos] = {shift fraction of
-// square q, code word}, s_c[pos] = crop column, and s_taps[r] = the 2H
-// running-sum weights of block offset r (tapw, r < D).
-template <int kAl>
-__device__ __forceinline__ void build_stream_table(float2 *s_fc, int *s_c, float4 *s_taps,
+// Per-CTA tables over the stream of decimated views j0 .. j1 - 1: position
+// pos is view k' = j0 D - (H D - 1) + pos (taken mod P), s_v[pos] = {shift
+// fraction, the crop's offset inside its aligned box, weights 0 and 1}, s_w2[pos] = weights 2 and 3 (H = 2),
+// s_c[pos] = crop column.
+template <int kAl, int H>
+__device__ __forceinline__ void build_stream_table(float4 *s_v, float2 *s_w2, int *s_c,
                                                    const int32_t *__restrict__ crop,
                                                    const GeomEntry *__restrict__ geo,
-                                                   const float4 *__restrict__ tapw, int q, int P, int D, int Pd,
-                                                   int H) {
-    const int nstream = P + (2 * H - 1) * D - 1;
+                                                   const float4 *__restrict__ tapw, int q, int P, int D, int j0,
+                                                   int nstream) {
     for (int pos = threadIdx.x; pos < nstream; pos += blockDim.x) {
-        const int kp = pos - (H * D - 1);
+        const int kp = j0 * D + pos - (H * D - 1);
         const int kk = ((kp % P) + P) % P;
         const int c = crop[(size_t)q * P + kk];
         const int jb = floor_div(kp, D);
         const int r = kp - jb * D;
-        int code = (c & (kAl - 1)) | (r << kCodeTapShift);
-        const int jst = jb - H + 1;  // decimated view whose support ends here
-        if (r == D - 1) code |= kCodeRotate | (jst >= 0 && jst < Pd ? (jst + 1) << kCodeStoreShift : 0);
-        s_fc[pos] = make_float2(geo[(size_t)q * P + kk].frac, __int_as_float(code));
+        const float4 w = tapw[r];
+        s_v[pos] = make_float4(geo[(size_t)q * P + kk].frac, __int_as_float(c & (kAl - 1)), w.x, w.y);
+        if (H == 2) s_w2[pos] = make_float2(w.z, w.w);
         s_c[pos] = c;
     }
-    for (int r = threadIdx.x; r < D; r += blockDim.x) s_taps[r] = tapw[r];
 }
 
-// One element at a compile-time byte offset from 32-bit shared address a,
-// widened to float.
-template <typename TQ, int OFF>
-struct Ld1;
-template <int OFF>
-struct Ld1<float, OFF> {
-    static __device__ __forceinline__ float f(uint32_t a) {
-        float v;
-        asm volatile("ld.shared.f32 %0, [%1+%2];" : "=f"(v) : "r"(a), "n"(OFF) : "memory");
-        return v;
+// 16 bytes of a row, as floats
+template <typename TQ>
+struct Row16;
+template <>
+struct Row16<float> {
+    static constexpr int kN = 4;
+    static __device__ __forceinline__ void load(uint32_t a, float *v) {
+        asm volatile("ld.shared.v4.f32 {%0, %1, %2, %3}, [%4];"
+                     : "=f"(v[0]), "=f"(v[1]), "=f"(v[2]), "=f"(v[3])
+                     : "r"(a)
+                     : "memory");
     }
 };
-template <int OFF>
-struct Ld1<__nv_bfloat16, OFF> {
-    static __device__ __forceinline__ float f(uint32_t a) {
-        uint32_t u;
-        asm volatile("ld.shared.u16 %0, [%1+%2];" : "=r"(u) : "r"(a), "n"(OFF) : "memory");
-        return __uint_as_float(u << 16);  // bfloat16 is the top half of a float32
-    }
-};
-template <int OFF>
-struct Ld1<__half, OFF> {
-    static __device__ __forceinline__ float f(uint32_t a) {
-        unsigned short h;
-        asm volatile("ld.shared.u16 %0, [%1+%2];" : "=h"(h) : "r"(a), "n"(OFF) : "memory");
-        return __half2float(__ushort_as_half(h));
-    }
-};
-
-// One view for one lane: in each of its RPL rows (row stride rs bytes), the
-// columns t = lane + 32 i (i < C, t < T) sample the row at box column
-// off + t (+ the shift fraction f) and feed that row's 2H running sums with
-// weights w.  a is the byte address of box column off + lane of the lane's
-// first row, so consecutive lanes read consecutive elements (no bank
-// conflicts) whatever the crop's offset off inside its aligned box.
-// Columns past T are computed too (no branch; their sums are never stored):
-// their loads stay inside the CTA's shared memory, within the next row, the
-// next slot or the ring's tail slack of kColSlack(C) bytes.
-//
-// Rows are taken in pairs (r, r + 1) where the lane has an even number of
-// them: the two rows share the shift fraction and the tap weights, so one
-// packed two-lane FP32 instruction (each lane rounded as the scalar
-// operation would be) does the work of two.  acc[rp][m][i] holds running
-// sum m of column i for rows 2 rp (x) and 2 rp + 1 (y); a lane with one row
-// uses x only.
-template <typename TQ, int I, int C, int H>
-__device__ __forceinline__ void col_step(uint32_t ar, float f, float4 w, float2 (&acc)[2 * H][C]) {
-    constexpr int ES = (int)sizeof(TQ);
-    const float a0 = Ld1<TQ, ES * 32 * I>::f(ar), a1 = Ld1<TQ, ES * (32 * I + 1)>::f(ar);
-    const float smp = fmaf(f, a1 - a0, a0);
-    acc[0][I].x = fmaf(w.x, smp, acc[0][I].x);
-    acc[1][I].x = fmaf(w.y, smp, acc[1][I].x);
-    if (H == 2) {
-        acc[2][I].x = fmaf(w.z, smp, acc[2][I].x);
-        acc[3][I].x = fmaf(w.w, smp, acc[3][I].x);
-    }
+__device__ __forceinline__ uint4 lds128(uint32_t a) {
+    uint4 u;
+    asm volatile("ld.shared.v4.u32 {%0, %1, %2, %3}, [%4];"
+                 : "=r"(u.x), "=r"(u.y), "=r"(u.z), "=r"(u.w)
+                 : "r"(a)
+                 : "memory");
+    return u;
 }
-
-template <typename TQ, int I, int C, int H>
-__device__ __forceinline__ void col_step2(uint32_t ar, uint32_t ar2, float2 f2, const float2 (&w2)[2 * H],
-                                          float2 (&acc)[2 * H][C]) {
-    constexpr int ES = (int)sizeof(TQ);
-    const float2 a0 = make_float2(Ld1<TQ, ES * 32 * I>::f(ar), Ld1<TQ, ES * 32 * I>::f(ar2));
-    const float2 a1 = make_float2(Ld1<TQ, ES * (32 * I + 1)>::f(ar), Ld1<TQ, ES * (32 * I + 1)>::f(ar2));
-    // a0 + f (a1 - a0)
-    const float2 smp = __ffma2_rn(f2, fsub2(a1, a0), a0);
+template <>
+struct Row16<__nv_bfloat16> {
+    static constexpr int kN = 8;
+    static __device__ __forceinline__ void load(uint32_t a, float *v) {
+        const uint4 u = lds128(a);
+        const uint32_t w[4] = {u.x, u.y, u.z, u.w};
 #pragma unroll
-    for (int m = 0; m < 2 * H; ++m) acc[m][I] = __ffma2_rn(w2[m], smp, acc[m][I]);
-}
-
-template <typename TQ, int C, int H, int... I>
-__device__ __forceinline__ void row_cols(uint32_t ar, float f, float4 w, float2 (&acc)[2 * H][C],
-                                         std::integer_sequence<int, I...>) {
-    (col_step<TQ, I, C, H>(ar, f, w, acc), ...);
-}
-
-template <typename TQ, int C, int H, int... I>
-__device__ __forceinline__ void row_pair_cols(uint32_t ar, uint32_t ar2, float2 f2, const float2 (&w2)[2 * H],
-                                              float2 (&acc)[2 * H][C], std::integer_sequence<int, I...>) {
-    (col_step2<TQ, I, C, H>(ar, ar2, f2, w2, acc), ...);
-}
-
-template <typename TQ, int C, int H, int RPL>
-__device__ __forceinline__ void view_cols(uint32_t a, uint32_t rs, float f, float4 w,
-                                          float2 (&acc)[(RPL + 1) / 2][2 * H][C]) {
-    if constexpr (RPL % 2 == 0) {
-        const float2 f2 = make_float2(f, f);
-        float2 w2[2 * H];
-        w2[0] = make_float2(w.x, w.x);
-        w2[1] = make_float2(w.y, w.y);
-        if constexpr (H == 2) {
-            w2[2] = make_float2(w.z, w.z);
-            w2[3] = make_float2(w.w, w.w);
+        for (int i = 0; i < 4; ++i) {  // bfloat16 is the top half of a float32
+            v[2 * i] = __uint_as_float(w[i] << 16);
+            v[2 * i + 1] = __uint_as_float(w[i] & 0xffff0000u);
         }
+    }
+};
+template <>
+struct Row16<__half> {
+    static constexpr int kN = 8;
+    static __device__ __forceinline__ void load(uint32_t a, float *v) {
+        const uint4 u = lds128(a);
+        const uint32_t w[4] = {u.x, u.y, u.z, u.w};
 #pragma unroll
-        for (int rp = 0; rp < RPL / 2; ++rp) {
-            const uint32_t ar = a + rs * (uint32_t)(2 * rp);
-            row_pair_cols<TQ, C, H>(ar, ar + rs, f2, w2, acc[rp], std::make_integer_sequence<int, C>{});
+        for (int i = 0; i < 4; ++i) {
+            const float2 f = __half22float2(*reinterpret_cast<const __half2 *>(&w[i]));
+            v[2 * i] = f.x;
+            v[2 * i + 1] = f.y;
         }
-    } else {
-        static_assert(RPL == 1, "an odd number of rows per lane is one row");
-        row_cols<TQ, C, H>(a, f, w, acc[0], std::make_integer_sequence<int, C>{});
+    }
+};
+
+// One view for one lane: its row's samples at columns OFF .. OFF + kCW of the
+// 16-byte aligned address a feed the 2H running sums of its kCW columns.
+template <typename TQ, int H, int OFF>
+__device__ __forceinline__ void view_step(uint32_t a, float f, const float (&w)[2 * H], float (&acc)[2 * H][kCW]) {
+    constexpr int kN = Row16<TQ>::kN;
+    constexpr int kL = (OFF + kCW + 1 + kN - 1) / kN;
+    float v[kL * kN];
+#pragma unroll
+    for (int i = 0; i < kL; ++i) Row16<TQ>::load(a + 16u * (uint32_t)i, v + i * kN);
+#pragma unroll
+    for (int i = 0; i < kCW; ++i) {
+        const float smp = fmaf(f, v[OFF + i + 1] - v[OFF + i], v[OFF + i]);
+#pragma unroll
+        for (int m = 0; m < 2 * H; ++m) acc[m][i] = fmaf(w[m], smp, acc[m][i]);
     }
 }
 
-template <typename TQ, int C, int H, int RPL>
-__global__ void __launch_bounds__(kDecThreads)
-decompose_tma_kernel(const __grid_constant__ CUtensorMap tmap, float *__restrict__ Sp,
-                     const int32_t *__restrict__ crop, const GeomEntry *__restrict__ geo,
-                     const int32_t *__restrict__ Tq, const float4 *__restrict__ tapw, int *status, int Tstride, int P,
-                     int D, int Pd, int Nv, int Wc, int tile_stride, int rowoff, int rowend) {
+template <typename TQ, int H>
+__device__ __forceinline__ void view_any(int off, uint32_t a, float f, const float (&w)[2 * H],
+                                         float (&acc)[2 * H][kCW]) {
+    switch (off) {
+        case 0: view_step<TQ, H, 0>(a, f, w, acc); break;
+        case 1: view_step<TQ, H, 1>(a, f, w, acc); break;
+        case 2: view_step<TQ, H, 2>(a, f, w, acc); break;
+        case 3: view_step<TQ, H, 3>(a, f, w, acc); break;
+        default:
+            if constexpr (sizeof(TQ) == 2) {
+                switch (off) {
+                    case 4: view_step<TQ, H, 4>(a, f, w, acc); break;
+                    case 5: view_step<TQ, H, 5>(a, f, w, acc); break;
+                    case 6: view_step<TQ, H, 6>(a, f, w, acc); break;
+                    default: view_step<TQ, H, 7>(a, f, w, acc); break;
+                }
+            }
+    }
+}
+
+// dynamic shared memory: ring, transpose buffers, tables
+__host__ __device__ inline size_t dec_smem(int es, int stages, int tile_stride, int warps, int nstream, int H) {
+    return 128 + (size_t)es * stages * tile_stride + kRingSlack + (size_t)warps * 32 * kTP * sizeof(float) +
+           (size_t)nstream * (16 + (H == 2 ? 8 : 0) + 4);
+}
+
+// the thread bound only sets the register limit: 80 (24 warps per SM) for the
+// two running sums of the triangle, 128 (16 warps) for the four of 2D-tap filters
+template <typename TQ, int H>
+__global__ void __launch_bounds__(H == 1 ? 768 : 512, 1)
+decompose_rows_kernel(const __grid_constant__ CUtensorMap tmap, float *__restrict__ Sp,
+                      const int32_t *__restrict__ crop, const GeomEntry *__restrict__ geo,
+                      const int32_t *__restrict__ Tq, const float4 *__restrict__ tapw, int *status, int Tstride,
+                      int P, int D, int Pd, int Nv, int Wc, int tile_stride, int segs, int chunks, int rowoff, int rowend,
+                      int jrange) {
     constexpr int ES = (int)sizeof(TQ);
     constexpr int kAlign = 16 / ES;
     constexpr int kG = Ring<TQ>::kG, kStages = Ring<TQ>::kStages;
-    constexpr int VB = kConsumerWarps * RPL;   // rows per CTA (box height)
     extern __shared__ __align__(128) unsigned char smem_raw[];
     unsigned char *ring = smem_raw + ((128u - (tma::smem_u32(smem_raw) & 127u)) & 127u);
     const uint32_t tile_bytes = (uint32_t)(ES * tile_stride);
-    // views streamed: k' = -(H D - 1) .. P - 1 + (H - 1) D (view k' mod P)
-    const int nstream = P + (2 * H - 1) * D - 1;
+    const int j0 = blockIdx.z * jrange, j1 = min(j0 + jrange, Pd);
+    // views streamed: k' = j0 D - (H D - 1) .. (j1 - 1) D + H D - 1 (view k' mod P)
+    const int nstream = (j1 - j0) * D + (2 * H - 1) * D - 1;
     const int nstage = (nstream + kG - 1) / kG;
-    float4 *s_taps = (float4 *)(ring + (size_t)tile_bytes * kStages * kG + kColSlack(C));
-    float2 *s_fc = (float2 *)(s_taps + D);
-    int *s_c = (int *)(s_fc + nstream);
+    const int warps = (int)(blockDim.x >> 5) - 1;  // consumer warps
+    float *tbuf = (float *)(ring + (size_t)tile_bytes * kStages * kG + kRingSlack);
+    float4 *s_v = (float4 *)(tbuf + (size_t)warps * 32 * kTP);
+    float2 *s_w2 = (float2 *)(s_v + nstream);
+    int *s_c = (int *)(s_w2 + (H == 2 ? nstream : 0));
     __shared__ __align__(8) uint64_t full[kStages], empty[kStages];
 
-    const int q = blockIdx.x;
-    const int v0 = rowoff + blockIdx.y * VB;
-    const int tx = threadIdx.x & 31, ty = threadIdx.x >> 5;
+    const int q = blockIdx.x / chunks;
+    const int tc = (blockIdx.x - q * chunks) * (segs * kCW);  // first column of the CTA's segments
+    const int band = 32 * (warps / segs);                     // rows per CTA
+    const int v0 = rowoff + blockIdx.y * band;
+    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
 
-    build_stream_table<kAlign>(s_fc, s_c, s_taps, crop, geo, tapw, q, P, D, Pd, H);
+    build_stream_table<kAlign, H>(s_v, s_w2, s_c, crop, geo, tapw, q, P, D, j0, nstream);
     if (threadIdx.x == 0) {
         for (int i = 0; i < kStages; ++i) {
             tma::mbar_init(&full[i], 1);
-            tma::mbar_init(&empty[i], kConsumerWarps);
+            tma::mbar_init(&empty[i], warps);
         }
         tma::fence_mbar_init();
     }
     __syncthreads();
 
-    if (ty == kConsumerWarps) {  // producer
-        if (tx != 0) return;
-        int kk = ((-(H * D - 1)) % P + P) % P, n = 0, slot = 0;
+    if (warp == warps) {  // producer
+        if (lane != 0) return;
+        int kk = ((j0 * D - (H * D - 1)) % P + P) % P, n = 0, slot = 0;
         uint32_t phase = 0;  // parity of the slot's current round
         for (; n < nstage; ++n) {
             // round r of a slot may start once its round r - 1 was consumed
@@ -320,10 +299,10 @@ decompose_tma_kernel(const __grid_constant__ CUtensorMap tmap, float *__restrict
             }
             const int nv = min(kG, nstream - n * kG);
             tma::fence_proxy_async();
-            tma::mbar_arrive_expect_tx(&full[slot], (uint32_t)(nv * VB * Wc * ES));
+            tma::mbar_arrive_expect_tx(&full[slot], (uint32_t)(nv * band * Wc * ES));
             for (int w = 0; w < nv; ++w) {
                 tma::load_3d(ring + (size_t)tile_bytes * (slot * kG + w), &tmap, &full[slot],
-                             s_c[n * kG + w] & ~(kAlign - 1), v0, kk);
+                             (s_c[n * kG + w] & ~(kAlign - 1)) + tc, v0, kk);
                 if (++kk == P) kk = 0;
             }
             if (++slot == kStages) {
@@ -337,77 +316,84 @@ decompose_tma_kernel(const __grid_constant__ CUtensorMap tmap, float *__restrict
         return;
     }
 
-    const int rib = ty * RPL;  // first of the warp's rows in the band
-    const int v = v0 + rib;
+    const int grp = warp / segs, seg = warp - grp * segs;
+    const int rib = 32 * grp;  // first of the warp's rows in the band
+    const int t0 = tc + seg * kCW;  // first of its columns
     const int T = Tq[q];
-    constexpr int RP = (RPL + 1) / 2;  // row pairs
-    float2 acc[RP][2 * H][C];
+    float acc[2 * H][kCW];
 #pragma unroll
-    for (int r = 0; r < RP; ++r)
+    for (int m = 0; m < 2 * H; ++m)
 #pragma unroll
-        for (int m = 0; m < 2 * H; ++m)
-#pragma unroll
-            for (int i = 0; i < C; ++i) acc[r][m][i] = make_float2(0.f, 0.f);
+        for (int i = 0; i < kCW; ++i) acc[m][i] = 0.f;
+    // coalesced store: lane writes 16 bytes at row rib + lane / 4 (+ 8, 16, 24), column t0 + 4 (lane % 4)
     const size_t vstride = (size_t)Nv * Tstride;
-    float *out = Sp + ((size_t)q * Pd * Nv + v) * Tstride + tx;  // row v; row v + r is r Tstride further
-    const uint32_t lane_addr = tma::smem_u32(ring) + (uint32_t)(ES * (rib * Wc + tx));
-    const uint32_t row_bytes = (uint32_t)(ES * Wc);
+    const int srow = v0 + rib + (lane >> 2), scol = t0 + 4 * (lane & 3);
+    float *out = Sp + ((size_t)q * Pd * Nv + srow) * Tstride + scol;
+    float *tb = tbuf + (size_t)warp * 32 * kTP;
+    const uint32_t lane_addr = tma::smem_u32(ring) + (uint32_t)(ES * ((rib + lane) * Wc + seg * kCW));
     int slot = 0;
     uint32_t phase = 0;
 
-    for (int n = 0; n < nstage; ++n) {
-        const bool ok = tma::mbar_wait_bounded(&full[slot], phase, kDecWaitNs);
-        if (!__all_sync(0xffffffffu, ok)) {
-            if (tx == 0) atomicOr(status, 2);
-            return;
-        }
-        const int nv = min(kG, nstream - n * kG);
-        const uint32_t sa = lane_addr + tile_bytes * (uint32_t)(slot * kG);
-#pragma unroll
-        for (int w = 0; w < kG; ++w) {
-            if (w < nv) {
-                const float2 fc = s_fc[n * kG + w];
-                const int code = __float_as_int(fc.y);
-                const float4 tp = s_taps[(code >> kCodeTapShift) & 255];
-                view_cols<TQ, C, H, RPL>(sa + tile_bytes * (uint32_t)w + (uint32_t)(ES * (code & (kAlign - 1))),
-                                         row_bytes, fc.x, tp, acc);
-                if (code & kCodeRotate) {
-                    const int jst = (code >> kCodeStoreShift) - 1;
-                    if (jst >= 0) {
-#pragma unroll
-                        for (int r = 0; r < RPL; ++r) {
-                            if (v + r < rowend) {
-                                float *dst = out + (size_t)jst * vstride + (size_t)r * Tstride;
-#pragma unroll
-                                for (int i = 0; i < C; ++i) {
-                                    const float val = (r & 1) ? acc[r / 2][0][i].y : acc[r / 2][0][i].x;
-                                    if (tx + 32 * i < Tstride) dst[32 * i] = tx + 32 * i < T ? val : 0.f;
-                                }
-                            }
-                        }
-                    }
-#pragma unroll
-                    for (int r = 0; r < RP; ++r)
-#pragma unroll
-                        for (int i = 0; i < C; ++i) {
-#pragma unroll
-                            for (int m = 0; m < 2 * H - 1; ++m) acc[r][m][i] = acc[r][m + 1][i];
-                            acc[r][2 * H - 1][i] = make_float2(0.f, 0.f);
-                        }
+    // the stream starts at the second view of block j0 - H, whose end completes view j0 - 2 H + 1
+    int left = D - 1, w = 0;
+    const float4 *pe = s_v;
+    const float2 *pe2 = s_w2;
+    uint32_t a = lane_addr;
+    for (int jst = j0 - 2 * H + 1; jst < j1; ++jst, left = D) {
+#pragma unroll 1
+        for (; left > 0; --left) {
+            if (w == 0) {
+                const bool ok = tma::mbar_wait_bounded(&full[slot], phase, kDecWaitNs);
+                if (!__all_sync(0xffffffffu, ok)) {
+                    if (lane == 0) atomicOr(status, 2);
+                    return;
+                }
+            }
+            const float4 e = *pe++;
+            float wt[2 * H];
+            wt[0] = e.z;
+            wt[1] = e.w;
+            if constexpr (H == 2) {
+                const float2 e2 = *pe2++;
+                wt[2] = e2.x;
+                wt[3] = e2.y;
+            }
+            view_any<TQ, H>(__float_as_int(e.y), a, e.x, wt, acc);
+            a += tile_bytes;
+            if (++w == kG) {
+                w = 0;
+                __syncwarp();
+                if (lane == 0) tma::mbar_arrive(&empty[slot]);
+                if (++slot == kStages) {
+                    slot = 0;
+                    phase ^= 1u;
+                    a = lane_addr;
                 }
             }
         }
-        __syncwarp();
-        if (tx == 0) tma::mbar_arrive(&empty[slot]);
-        if (++slot == kStages) {
-            slot = 0;
-            phase ^= 1u;
+        if (jst >= j0) {  // decimated view jst is complete
+            float4 *dst = (float4 *)(tb + lane * kTP);
+#pragma unroll
+            for (int i = 0; i < kCW; i += 4)
+                dst[i / 4] = make_float4(t0 + i < T ? acc[0][i] : 0.f, t0 + i + 1 < T ? acc[0][i + 1] : 0.f,
+                                         t0 + i + 2 < T ? acc[0][i + 2] : 0.f, t0 + i + 3 < T ? acc[0][i + 3] : 0.f);
+            __syncwarp();
+            float *o = out + (size_t)jst * vstride;
+#pragma unroll
+            for (int i = 0; i < 4; ++i) {
+                const float4 val = *(const float4 *)(tb + (8 * i + (lane >> 2)) * kTP + 4 * (lane & 3));
+                if (srow + 8 * i < rowend && scol < Tstride) *(float4 *)(o + (size_t)(8 * i) * Tstride) = val;
+            }
+            __syncwarp();
+        }
+#pragma unroll
+        for (int i = 0; i < kCW; ++i) {
+#pragma unroll
+            for (int m = 0; m < 2 * H - 1; ++m) acc[m][i] = acc[m + 1][i];
+            acc[2 * H - 1][i] = 0.f;
         }
     }
 }
-
-// columns per lane C (lane t takes t, t + 32, ...) from the decomposed row length
-inline int dec_cols(int Tstride) { return Tstride <= 32 ? 1 : Tstride <= 64 ? 2 : Tstride <= 128 ? 4 : 8; }
 
 // Rows of a launch: the arrays hold `layout` rows per view (S' included)
 // and the launch covers rows rowoff .. rowend - 1 of them.
@@ -415,84 +401,77 @@ struct Rows {
     int layout, rowoff, rowend;
 };
 
-template <typename TQ, int C, int H, int RPL>
-cudaError_t launch_tma_shape(const PlanImpl &p, const CUtensorMap &map, float *out, int Wc, cudaStream_t st,
-                             Rows rw, size_t smem, int tile_stride) {
-    cudaError_t e = ensure_smem<decompose_tma_kernel<TQ, C, H, RPL>>(smem);
-    if (e != cudaSuccess) return e;
-    constexpr int VB = kConsumerWarps * RPL;
-    dim3 grid(p.od.nsq, (rw.rowend - rw.rowoff + VB - 1) / VB);
-    decompose_tma_kernel<TQ, C, H, RPL><<<grid, kDecThreads, smem, st>>>(
-        map, out, p.od.crop, p.od.geo, p.od.T, p.tapw, p.status, p.Tstride, p.g.P, p.D, p.Pd, rw.layout, Wc,
-        tile_stride, rw.rowoff, rw.rowend);
-    return cudaGetLastError();
-}
-
-template <typename TQ, int H, int RPL>
-cudaError_t launch_tma_c(const PlanImpl &p, const CUtensorMap &map, float *out, int Wc, cudaStream_t st, Rows rw,
-                         size_t smem, int tile_stride) {
-    switch (dec_cols(p.Tstride)) {
-        case 1: return launch_tma_shape<TQ, 1, H, RPL>(p, map, out, Wc, st, rw, smem, tile_stride);
-        case 2: return launch_tma_shape<TQ, 2, H, RPL>(p, map, out, Wc, st, rw, smem, tile_stride);
-        case 4: return launch_tma_shape<TQ, 4, H, RPL>(p, map, out, Wc, st, rw, smem, tile_stride);
-        default: return launch_tma_shape<TQ, 8, H, RPL>(p, map, out, Wc, st, rw, smem, tile_stride);
-    }
-}
-
-template <typename TQ, int H>
-cudaError_t launch_tma_h(const PlanImpl &p, const CUtensorMap &map, float *out, int Wc, cudaStream_t st, Rows rw,
-                         size_t smem, int tile_stride, bool wide) {
-    return wide ? launch_tma_c<TQ, H, rows_per_lane(H, true)>(p, map, out, Wc, st, rw, smem, tile_stride)
-                : launch_tma_c<TQ, H, rows_per_lane(H, false)>(p, map, out, Wc, st, rw, smem, tile_stride);
-}
-
-// the wide rows-per-lane shape unless its grid would not fill two waves
-bool wide_rows(const PlanImpl &p, int H, int nrows) {
-    int dev = 0, sms = 148;
-    if (cudaGetDevice(&dev) == cudaSuccess) cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
-    const int vb = kConsumerWarps * rows_per_lane(H, true);
-    return (long long)p.od.nsq * ((nrows + vb - 1) / vb) >= 2LL * sms;
-}
-
 // TMA applies when Q's rows are whole 16-byte units, Q and S' are 16-byte
-// aligned (vector stores), a crop box (T_max + one interpolation neighbour +
-// alignment) fits 256 columns, D <= 128 and the ring plus the stream tables
-// fit in shared memory.
-template <typename TQ>
-cudaError_t try_tma(const PlanImpl &p, const TQ *Q, float *out, cudaStream_t st, Rows rw, bool &launched) {
-    const int nrows = rw.layout;
+// aligned (vector stores), D <= 128 and the ring plus the stream tables fit
+// in shared memory.
+template <typename TQ, int H>
+cudaError_t try_rows(const PlanImpl &p, const TQ *Q, float *out, cudaStream_t st, Rows rw, bool &launched) {
     launched = false;
     constexpr int kAlign = 16 / (int)sizeof(TQ);
     if ((p.g.Nu % kAlign) != 0 || ((uintptr_t)Q & 15) != 0 || ((uintptr_t)out & 15) != 0) return cudaSuccess;
-    const int Wc = (p.od.Tmax + 1 + (kAlign - 1) + (kAlign - 1)) & ~(kAlign - 1);
-    if (Wc > 256 || p.Tstride > 256 || p.D > kMaxTapD) return cudaSuccess;  // block offset: 8 bits of the code
-    const bool wide = wide_rows(p, p.tap_blocks, rw.rowend - rw.rowoff);
-    const int VB = kConsumerWarps * rows_per_lane(p.tap_blocks, wide);
-    const int tile_stride = (VB * Wc + 63) & ~63;  // elements; 128-byte multiple for every type
-    const int nstream = p.g.P + (2 * p.tap_blocks - 1) * p.D - 1;
-    const size_t smem = 128 + sizeof(TQ) * (size_t)Ring<TQ>::kStages * Ring<TQ>::kG * tile_stride +
-                        kColSlack(dec_cols(p.Tstride)) +
-                        16 * (size_t)p.D +
-                        12 * (size_t)nstream;
-    if (smem > 200 * 1024) return cudaSuccess;
+    if (p.D > kMaxTapD) return cudaSuccess;
+    const int all = (p.Tstride + kCW - 1) / kCW;  // column segments of a square
+    const int chunks = (all + kDecMaxSegs - 1) / kDecMaxSegs, segs = (all + chunks - 1) / chunks;
+    // the segments' columns + neighbour + crop offset, whole 16-byte units, an odd number of them
+    int Wc = (std::min(p.od.Tmax, segs * kCW) + 1 + (kAlign - 1) + (kAlign - 1)) & ~(kAlign - 1);
+    if ((Wc / kAlign) % 2 == 0) Wc += kAlign;
+    const int nrows = rw.rowend - rw.rowoff;
+    // narrow squares: several row groups per CTA, at least four consumer warps
+    const int groups = std::max(1, std::min((nrows + 31) / 32, 4 / segs));
+    const int warps = segs * groups, band = 32 * groups;
+    const int bands = (nrows + band - 1) / band;
+    const int tile_stride = (band * Wc + 63) & ~63;  // elements; 128-byte multiple for every type
+    int dev = 0, sms = 148;
+    if (cudaGetDevice(&dev) == cudaSuccess) cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
+    constexpr int kLead = 2 * H - 1;  // a range streams kLead D - 1 views besides its own
+    auto smem_of = [&](int jr) {
+        return dec_smem((int)sizeof(TQ), Ring<TQ>::kStages * Ring<TQ>::kG, tile_stride, warps, (jr + kLead) * p.D - 1, H);
+    };
+    // The decimated views are split into ranges (the same sums in the same
+    // order, so the same result) where (square, band) CTAs would not fill the
+    // GPU twice -- a range then keeps at least 4 kLead decimated views -- and
+    // where a shorter table lets the CTAs that the registers allow share an SM
+    // (512^3 f32: 1.29 ms with two CTAs per SM, 1.11 with three)
+    const long long ctas = (long long)p.od.nsq * chunks * bands;
+    int ranges = (int)std::min<long long>(p.Pd, (4LL * sms + ctas - 1) / ctas);
+    int jrange = std::max((p.Pd + ranges - 1) / ranges, std::min(p.Pd, 4 * kLead));
+    int per_sm = 0;
+    if (cudaDeviceGetAttribute(&per_sm, cudaDevAttrMaxSharedMemoryPerMultiprocessor, dev) != cudaSuccess) per_sm = 0;
+    const size_t share = (size_t)per_sm / (H == 1 ? 3 : 2);
+    for (ranges = 1; (p.Pd + ranges - 1) / ranges >= std::min(p.Pd, 4 * kLead); ++ranges) {
+        const int jr = std::min(jrange, (p.Pd + ranges - 1) / ranges);
+        if (smem_of(jr) + 2048 <= share) {
+            jrange = jr;
+            break;
+        }
+        if (ranges == p.Pd) break;
+    }
+    const size_t smem = smem_of(jrange);
+    if (smem > 200 * 1024 || bands > 65535) return cudaSuccess;
     CUtensorMap map;
-    const uint64_t dims[3] = {(uint64_t)p.g.Nu, (uint64_t)nrows, (uint64_t)p.g.P};
-    const uint64_t strides[2] = {(uint64_t)p.g.Nu * sizeof(TQ), (uint64_t)p.g.Nu * nrows * sizeof(TQ)};
-    const uint32_t box[3] = {(uint32_t)Wc, (uint32_t)VB, 1u};
+    const uint64_t dims[3] = {(uint64_t)p.g.Nu, (uint64_t)rw.layout, (uint64_t)p.g.P};
+    const uint64_t strides[2] = {(uint64_t)p.g.Nu * sizeof(TQ), (uint64_t)p.g.Nu * rw.layout * sizeof(TQ)};
+    const uint32_t box[3] = {(uint32_t)Wc, (uint32_t)band, 1u};
     const CUtensorMapDataType dt = sizeof(TQ) == 4 ? CU_TENSOR_MAP_DATA_TYPE_FLOAT32
                                    : (std::is_same<TQ, __half>::value ? CU_TENSOR_MAP_DATA_TYPE_FLOAT16
                                                                       : CU_TENSOR_MAP_DATA_TYPE_BFLOAT16);
     if (encode_map_3d(&map, dt, Q, dims, strides, box) != cudaSuccess) return cudaSuccess;
     launched = true;
-    if (p.tap_blocks == 2) return launch_tma_h<TQ, 2>(p, map, out, Wc, st, rw, smem, tile_stride, wide);
-    return launch_tma_h<TQ, 1>(p, map, out, Wc, st, rw, smem, tile_stride, wide);
+    cudaError_t e = ensure_smem<decompose_rows_kernel<TQ, H>>(smem);
+    if (e != cudaSuccess) return e;
+    dim3 grid(p.od.nsq * chunks, bands, (p.Pd + jrange - 1) / jrange);
+    decompose_rows_kernel<TQ, H><<<grid, 32 * (warps + 1), smem, st>>>(
+        map, out, p.od.crop, p.od.geo, p.od.T, p.tapw, p.status, p.Tstride, p.g.P, p.D, p.Pd, rw.layout, Wc,
+        tile_stride, segs, chunks, rw.rowoff, rw.rowend, jrange);
+    return cudaGetLastError();
 }
 
 template <typename TQ>
 cudaError_t launch_t(const PlanImpl &p, const TQ *Q, float *out, cudaStream_t st, Rows rw) {
     if (p.tap_blocks != 1 && p.tap_blocks != 2) return cudaErrorInvalidValue;
     bool launched = false;
-    cudaError_t te = try_tma(p, Q, out, st, rw, launched);
+    cudaError_t te = p.tap_blocks == 2 ? try_rows<TQ, 2>(p, Q, out, st, rw, launched)
+                                       : try_rows<TQ, 1>(p, Q, out, st, rw, launched);
     if (launched || te != cudaSuccess) return te;
     dim3 grid((p.Tstride + kTX - 1) / kTX, (rw.rowend - rw.rowoff + kTY - 1) / kTY, p.od.nsq);
     if (p.tap_blocks == 2)
