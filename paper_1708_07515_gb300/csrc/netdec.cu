@@ -493,138 +493,284 @@ net_adjoint_kernel(const float *__restrict__ vol, const float *__restrict__ ref,
 // x, a1, a2 in FP32 with the FP32 weights w, take dS[q][j][v][t] as the
 // gradient of the decimated views, and accumulate the weight gradient
 // (layout of the C interface) into dW.  The plain low-pass has no weights.
+//
+// Three products make the work, 1280 multiply-adds each per view and column:
+// z2 = W2 * a1, dz1 = W2^T * dz2 and dW2 = dz2 a1^T.  FP32 CUDA cores, so the
+// floor is the FMA rate; what has to be avoided is a shared-memory operand
+// per multiply-add (the form before: 31 ms for the 256^3 training step, 12 %
+// of the FMA peak).  Each thread therefore holds a tile of results: for z2
+// and dz1 8 channels x 4 views of one column (18 loads per 160 FMAs, the
+// weights by broadcast 16-byte loads from a copy in the tile's order), for dW2
+// 2 x 4 channel pairs x 5 taps with the four a1 rows' taps sliding through
+// registers (6 loads per 40 FMAs).  Both run as packed two-lane FMAs.  Views are stored 8 columns apart with 8
+// words of padding after every fourth, so a warp's 4 view groups x 8 columns
+// touch 32 banks.  The next chunk's samples are loaded to registers before the
+// products and stored after them.
 constexpr int kBG = 8;                         // columns per CTA
 constexpr int kBThreads = 256;
-constexpr int kBA1 = kNA1 * kBG + 1;           // channel stride of a1 (padded)
-constexpr int kBA2 = kKA * kBG + 1;            // channel stride of a2
+constexpr int kTV = 4, kTC = kC / 2;           // tile: views x channels of a thread
+constexpr int kXV = kNA1 + kK - 1;             // x views per chunk the net reads
+constexpr int kMarg = 4;                       // zero views before dz2's first (and after its last)
+// word of view v of an array of views x kBG columns
+__host__ __device__ constexpr int vpos(int v) { return kBG * (v + v / 4); }
+constexpr int kBA1 = vpos(kNA1) + 2;           // channel stride of a1, then dz1 (2 mod 8: see dW2)
+constexpr int kBA2 = vpos(kNA1 + kMarg) + 2;   // channel stride of a2, then dz2
+static_assert(kNA1 % kTV == 0 && kKA % kTV == 0 && kNA1 / kTV * kBG * 2 == kBThreads, "tiles cover a chunk");
+static_assert(kKA % 20 == 0 && kKA + kMarg == kNA1, "dW2 unrolls 20 views; margin views");
+static_assert(kBA1 % 8 == 2 && kBA2 % 8 == 2, "four channel groups of four fall on distinct banks");
 __host__ __device__ inline size_t net_bwd_smem(const NetChunk &c) {
-    return sizeof(float) * ((size_t)kNetSize + (size_t)c.NX * kBG + (size_t)c.J * kBG + (size_t)kC * kBA1 +
-                            (size_t)kC * kBA2);
+    return sizeof(float) * ((size_t)2 * kC * kC * kK + 2 * kC * kK + (size_t)vpos(kXV + 3) + (size_t)c.J * kBG +
+                            (size_t)kC * kBA1 + (size_t)kC * kBA2);
 }
 
+// acc[c / 2][v] += sum_m w[m][c] s[v + m] (FLIP: s[v - m + 4]) for a tile,
+// two channels per packed FMA; w4: [kK][kTC]
+template <bool FLIP>
+__device__ __forceinline__ void tile_fma(float2 (&acc)[kTC / 2][kTV], const float4 *__restrict__ w4,
+                                         const float (&s)[2 * kTV]) {
+#pragma unroll
+    for (int m = 0; m < kK; ++m) {
+        float2 w[kTC / 2];
+#pragma unroll
+        for (int c = 0; c < kTC / 2; c += 2) {
+            const float4 f = w4[m * kTC / 4 + c / 2];
+            w[c] = make_float2(f.x, f.y);
+            w[c + 1] = make_float2(f.z, f.w);
+        }
+#pragma unroll
+        for (int c = 0; c < kTC / 2; ++c)
+#pragma unroll
+            for (int v = 0; v < kTV; ++v) {
+                const float x = s[FLIP ? v - m + kK - 1 : v + m];
+                acc[c][v] = __ffma2_rn(w[c], make_float2(x, x), acc[c][v]);
+            }
+    }
+}
+__device__ __forceinline__ float lane_of(float2 a, int i) { return i ? a.y : a.x; }
+
 template <typename TQ>
-__global__ void __launch_bounds__(kBThreads)
+__global__ void __launch_bounds__(kBThreads, 2)
 net_backward_kernel(const TQ *__restrict__ Q, const float *__restrict__ wts, const float *__restrict__ dS,
                     float *__restrict__ dW, const int32_t *__restrict__ crop, const GeomEntry *__restrict__ geo,
                     const int32_t *__restrict__ Tq, int Tstride, int P, int D, int Pd, int HD, int Nv, int Nu,
                     int ngroups, int row_lo) {
     extern __shared__ __align__(16) float fsm[];
     const NetChunk ch = net_chunk(D, HD);
-    float *W = fsm;                                  // W1 [80] W2 [1280] W3 [80]
-    float *xs = W + kNetSize;                        // [NX][kBG]
-    float *dy = xs + (size_t)ch.NX * kBG;            // [J][kBG]
+    float *Wf = fsm;                                 // W2 by (c', half of c): [16][2][5 m][8 c]
+    float *Wb = Wf + kC * kC * kK;                   // W2 by (c, half of c'): [16][2][5 m][8 c']
+    float *W1 = Wb + kC * kC * kK, *W3 = W1 + kC * kK;
+    float *xs = W3 + kC * kK;                        // x, view i = view j0 D - 6 + i
+    float *dy = xs + vpos(kXV + 3);                  // [J][kBG]
     float *a1 = dy + (size_t)ch.J * kBG;             // [kC][kBA1]: a1, then dz1
-    float *a2 = a1 + (size_t)kC * kBA1;              // [kC][kBA2]: a2, then dz2
-    const float *W1 = W, *W2 = W + kC * kK, *W3 = W + kC * kK + kC * kC * kK;
+    float *a2 = a1 + (size_t)kC * kBA1;              // [kC][kBA2]: a2, then dz2, kMarg views in
     const int q = blockIdx.x / ngroups, grp = blockIdx.x - q * ngroups;
     const int v = row_lo + blockIdx.y;
     const int t0 = grp * kBG;
     const int T = Tq[q];
     if (t0 >= T) return;
     const int tid = threadIdx.x;
-    for (int i = tid; i < kNetSize; i += kBThreads) W[i] = wts[i];
-    float g1 = 0.f, g3 = 0.f, g2[kK] = {0.f, 0.f, 0.f, 0.f, 0.f};
-    const int cw = tid >> 4, cv = tid & 15;        // (c, c') of this thread's W2 gradients
+    for (int i = tid; i < kC * kC * kK; i += kBThreads) {
+        const int m = i % kK, ci = i / kK % kC, c = i / (kK * kC);
+        const float w = wts[kC * kK + i];
+        Wf[((ci * 2 + c / kTC) * kK + m) * kTC + c % kTC] = w;
+        Wb[((c * 2 + ci / kTC) * kK + m) * kTC + ci % kTC] = w;
+    }
+    for (int i = tid; i < kC * kK; i += kBThreads) {
+        W1[(i / kK / kTC * kK + i % kK) * kTC + i / kK % kTC] = wts[i];  // [2][kK][kTC]
+        W3[i] = wts[kC * kK + kC * kC * kK + i];
+    }
+    for (int i = tid; i < kC * 2 * kMarg * kBG; i += kBThreads) {  // dz2's zero views
+        const int c = i / (2 * kMarg * kBG), r = i - c * (2 * kMarg * kBG), k = r / kBG;
+        a2[c * kBA2 + vpos(k < kMarg ? k : kKA + k) + r % kBG] = 0.f;
+    }
+    // tile of this thread: column tg, views kTV tv .., channels kTC th ..
+    const int tg = tid & (kBG - 1), tv = tid / kBG % (kNA1 / kTV), th = tid / (kBThreads / 2);
+    const float *xt = xs + vpos(kTV) * tv + tg;      // (vpos(4 n) = n vpos(4))
+    // dW2: channels c = 2 wc, 2 wc + 1 and c' = 4 wi .. 4 wi + 3 of column tg
+    const int wi = tid / kBG & 3, wc = tid / 32;
+    float2 g2[2][2][kK] = {};  // [c][pair of c'][tap]
+    // dW1, dW3: channel sc, column tg, one of two halves of the views
+    const int sc = tid / 16, sh = tid / kBG & 1;
+    float g1[kK] = {0.f, 0.f, 0.f, 0.f, 0.f}, g3[kK] = {0.f, 0.f, 0.f, 0.f, 0.f};
     const int nchunks = (Pd + ch.J - 1) / ch.J;
-    __syncthreads();
-    for (int cc = 0; cc < nchunks; ++cc) {
-        const int j0 = cc * ch.J, Jc = min(ch.J, Pd - j0);
-        const int kx0 = j0 * D - ch.XL;
-        for (int i = tid; i < ch.NX * kBG; i += kBThreads) {
-            const int ix = i / kBG, g = i - ix * kBG;
-            xs[i] = shifted_sample(Q, crop, geo, q, wrap(kx0 + ix, P), t0 + g, T, v, Nv, P, Nu);
-        }
-        for (int i = tid; i < ch.J * kBG; i += kBThreads) {
-            const int jl = i / kBG, t = t0 + (i - jl * kBG);
-            dy[i] = (jl < Jc && t < T) ? dS[(((size_t)q * Pd + j0 + jl) * Nv + v) * Tstride + t] : 0.f;
-        }
-        __syncthreads();
-        // layer 1 (a1 view ka = view j0 D - 4 + ka)
-        for (int i = tid; i < kC * kNA1 * kBG; i += kBThreads) {
-            const int c = i / (kNA1 * kBG), p = i - c * (kNA1 * kBG);
-            const float *xp = xs + (size_t)(p / kBG + ch.XL - 6) * kBG + (p % kBG);
-            float z = 0.f;
+
+    // x and dS of a chunk: this thread's elements to registers, then to shared memory
+    constexpr int kXN = (kXV * kBG + kBThreads - 1) / kBThreads;
+    float px[kXN], pd = 0.f;
+    auto load = [&](int cc) {
+        const int j0 = cc * ch.J;
 #pragma unroll
-            for (int m = 0; m < kK; ++m) z = fmaf(W1[c * kK + m], xp[m * kBG], z);
-            a1[c * kBA1 + p] = fmaxf(z, 0.f);
+        for (int n = 0; n < kXN; ++n) {
+            const int i = tid + n * kBThreads;
+            px[n] = i < kXV * kBG ? shifted_sample(Q, crop, geo, q, wrap(j0 * D - 6 + i / kBG, P), t0 + i % kBG, T, v,
+                                                   Nv, P, Nu)
+                                  : 0.f;
+        }
+        const int jl = tid / kBG, t = t0 + tid % kBG;
+        pd = (jl < ch.J && j0 + jl < Pd && t < T) ? dS[(((size_t)q * Pd + j0 + jl) * Nv + v) * Tstride + t] : 0.f;
+    };
+    static_assert((kKA - 5) / 2 + 1 <= kBThreads / kBG, "one dS element per thread (D >= 2)");
+
+    load(0);
+    for (int cc = 0; cc < nchunks; ++cc) {
+        const int Jc = min(ch.J, Pd - cc * ch.J);
+#pragma unroll
+        for (int n = 0; n < kXN; ++n) {
+            const int i = tid + n * kBThreads;
+            if (i < kXV * kBG) xs[vpos(i / kBG) + i % kBG] = px[n];
+        }
+        if (tid < ch.J * kBG) dy[tid] = pd;
+        __syncthreads();
+        if (cc + 1 < nchunks) load(cc + 1);
+        // layer 1 (a1 view ka = view j0 D - 4 + ka reads x views ka .. ka + 4)
+        {
+            float2 acc[kTC / 2][kTV] = {};
+            float s[2 * kTV];
+#pragma unroll
+            for (int i = 0; i < 2 * kTV; ++i) s[i] = xt[vpos(i)];
+            tile_fma<false>(acc, (const float4 *)(W1 + th * kTC * kK), s);
+#pragma unroll
+            for (int c = 0; c < kTC; ++c)
+#pragma unroll
+                for (int k = 0; k < kTV; ++k)
+                    a1[(th * kTC + c) * kBA1 + vpos(kTV) * tv + vpos(k) + tg] = fmaxf(lane_of(acc[c / 2][k], c & 1), 0.f);
         }
         __syncthreads();
         // layer 2 (a2 view ka2 = view j0 D - 2 + ka2 reads a1 views ka2 .. ka2 + 4)
-        for (int i = tid; i < kC * kKA * kBG; i += kBThreads) {
-            const int c = i / (kKA * kBG), p = i - c * (kKA * kBG);
-            float z = 0.f;
+        if (tv < kKA / kTV) {
+            float2 acc[kTC / 2][kTV] = {};
+#pragma unroll 1
             for (int ci = 0; ci < kC; ++ci) {
-                const float *w = W2 + (c * kC + ci) * kK;
-                const float *ap = a1 + ci * kBA1 + p;
+                const float *ap = a1 + ci * kBA1 + vpos(kTV) * tv + tg;
+                float s[2 * kTV];
 #pragma unroll
-                for (int m = 0; m < kK; ++m) z = fmaf(w[m], ap[m * kBG], z);
+                for (int i = 0; i < 2 * kTV; ++i) s[i] = ap[vpos(i)];
+                tile_fma<false>(acc, (const float4 *)(Wf + (ci * 2 + th) * kTC * kK), s);
             }
-            a2[c * kBA2 + p] = fmaxf(z, 0.f);
+#pragma unroll
+            for (int c = 0; c < kTC; ++c)
+#pragma unroll
+                for (int k = 0; k < kTV; ++k)
+                    a2[(th * kTC + c) * kBA2 + vpos(kTV) * (tv + 1) + vpos(k) + tg] = fmaxf(lane_of(acc[c / 2][k], c & 1), 0.f);
         }
         __syncthreads();
         // layer 3 weights: dW3[c][m] = sum_{jl, g} dy[jl][g] a2[c][jl D + m][g]
-        if (tid < kC * kK) {
-            const int c = tid / kK, m = tid - c * kK;
-            for (int jl = 0; jl < Jc; ++jl)
-                for (int g = 0; g < kBG; ++g) g3 = fmaf(dy[jl * kBG + g], a2[c * kBA2 + (jl * D + m) * kBG + g], g3);
+        for (int jl = sh; jl < Jc; jl += 2) {
+            const float d = dy[jl * kBG + tg];
+#pragma unroll
+            for (int m = 0; m < kK; ++m) g3[m] = fmaf(d, a2[sc * kBA2 + vpos(jl * D + m + kMarg) + tg], g3[m]);
         }
         __syncthreads();
         // dz2 in place of a2: relu'(z2) sum_jl W3[c][ka2 - jl D] dy[jl]
-        for (int i = tid; i < kC * kKA * kBG; i += kBThreads) {
-            const int c = i / (kKA * kBG), p = i - c * (kKA * kBG);
-            const int ka2 = p / kBG, g = p - ka2 * kBG;
+        for (int k = sh, j0 = 0; k < kKA; k += 2) {
+            while (j0 * D < k - (kK - 1)) ++j0;  // first output view whose taps reach k
+            float *z = a2 + sc * kBA2 + vpos(k + kMarg) + tg;
             float d = 0.f;
-            if (a2[c * kBA2 + p] > 0.f) {
-                int jl = ka2 >= 4 ? (ka2 - 4 + D - 1) / D : 0;
-                for (; jl * D <= ka2 && jl < Jc; ++jl) d = fmaf(W3[c * kK + ka2 - jl * D], dy[jl * kBG + g], d);
-            }
-            a2[c * kBA2 + p] = d;
+            for (int jl = j0; jl * D <= k && jl < Jc; ++jl) d = fmaf(W3[sc * kK + k - jl * D], dy[jl * kBG + tg], d);
+            *z = *z > 0.f ? d : 0.f;
         }
         __syncthreads();
-        // layer 2 weights: dW2[cw][cv][m] = sum_p dz2[cw][p] a1[cv][p + m kBG]
+        // layer 2 weights: dW2[c][c'][m] = sum_p dz2[c][p] a1[c'][view + m]
         {
-            const float *dz = a2 + cw * kBA2;
-            const float *ap = a1 + cv * kBA1;
-            for (int p = 0; p < kKA * kBG; ++p) {
-                const float d = dz[p];
+            const float *zp = a2 + 2 * wc * kBA2 + vpos(kMarg) + tg;
+            const float *ap = a1 + 4 * wi * kBA1 + tg;
+            float2 s[2][kK];
+            auto tap = [&](int j, int k) {
+                return make_float2(ap[2 * j * kBA1 + vpos(k)], ap[(2 * j + 1) * kBA1 + vpos(k)]);
+            };
 #pragma unroll
-                for (int m = 0; m < kK; ++m) g2[m] = fmaf(d, ap[p + m * kBG], g2[m]);
+            for (int j = 0; j < 2; ++j)
+#pragma unroll
+                for (int m = 0; m < kK - 1; ++m) s[j][m] = tap(j, m);
+#pragma unroll 1
+            for (int k0 = 0; k0 < kKA; k0 += 20, zp += vpos(20), ap += vpos(20)) {
+#pragma unroll
+                for (int k = 0; k < 20; ++k) {
+                    const float d0 = zp[vpos(k)], d1 = zp[kBA2 + vpos(k)];
+                    const float2 e0 = make_float2(d0, d0), e1 = make_float2(d1, d1);
+#pragma unroll
+                    for (int j = 0; j < 2; ++j) s[j][(k + kK - 1) % kK] = tap(j, k + kK - 1);
+#pragma unroll
+                    for (int j = 0; j < 2; ++j)
+#pragma unroll
+                        for (int m = 0; m < kK; ++m) {
+                            g2[0][j][m] = __ffma2_rn(e0, s[j][(k + m) % kK], g2[0][j][m]);
+                            g2[1][j][m] = __ffma2_rn(e1, s[j][(k + m) % kK], g2[1][j][m]);
+                        }
+                }
             }
         }
         __syncthreads();
         // dz1 in place of a1: relu'(z1) sum_{c, m} W2[c][c'][m] dz2[c][ka - m]
-        for (int i = tid; i < kC * kNA1 * kBG; i += kBThreads) {
-            const int ci = i / (kNA1 * kBG), p = i - ci * (kNA1 * kBG);
-            const int ka = p / kBG, g = p - ka * kBG;
-            float d = 0.f;
-            if (a1[ci * kBA1 + p] > 0.f) {
-                for (int c = 0; c < kC; ++c) {
-                    const float *w = W2 + (c * kC + ci) * kK;
-                    const float *dz = a2 + c * kBA2 + g;
+        {
+            float2 acc[kTC / 2][kTV] = {};
+#pragma unroll 1
+            for (int c = 0; c < kC; ++c) {
+                const float *zp = a2 + c * kBA2 + vpos(kTV) * tv + tg;  // views kTV tv - 4 ..
+                float s[2 * kTV];
 #pragma unroll
-                    for (int m = 0; m < kK; ++m) {
-                        const int k2 = ka - m;
-                        if (k2 >= 0 && k2 < kKA) d = fmaf(w[m], dz[k2 * kBG], d);
-                    }
-                }
+                for (int i = 0; i < 2 * kTV; ++i) s[i] = zp[vpos(i)];
+                tile_fma<true>(acc, (const float4 *)(Wb + (c * 2 + th) * kTC * kK), s);
             }
-            a1[ci * kBA1 + p] = d;
+#pragma unroll
+            for (int c = 0; c < kTC; ++c)
+#pragma unroll
+                for (int k = 0; k < kTV; ++k) {
+                    float *z = a1 + (th * kTC + c) * kBA1 + vpos(kTV) * tv + vpos(k) + tg;
+                    *z = *z > 0.f ? lane_of(acc[c / 2][k], c & 1) : 0.f;
+                }
         }
         __syncthreads();
         // layer 1 weights: dW1[c][m] = sum_p dz1[c][p] x[p + m]
-        if (tid < kC * kK) {
-            const int c = tid / kK, m = tid - c * kK;
-            for (int p = 0; p < kNA1 * kBG; ++p)
-                g1 = fmaf(a1[c * kBA1 + p], xs[(size_t)(p / kBG + ch.XL - 6 + m) * kBG + (p % kBG)], g1);
+        {
+            const float *zp = a1 + sc * kBA1 + vpos(kNA1 / 2) * sh + tg, *xp = xs + vpos(kNA1 / 2) * sh + tg;
+            float s[kK];
+#pragma unroll
+            for (int m = 0; m < kK - 1; ++m) s[m] = xp[vpos(m)];
+#pragma unroll
+            for (int k = 0; k < kNA1 / 2; ++k) {
+                s[(k + kK - 1) % kK] = xp[vpos(k + kK - 1)];
+                const float d = zp[vpos(k)];
+#pragma unroll
+                for (int m = 0; m < kK; ++m) g1[m] = fmaf(d, s[(k + m) % kK], g1[m]);
+            }
         }
         __syncthreads();
     }
-    if (tid < kC * kK) {
-        atomicAdd(dW + tid, g1);
-        atomicAdd(dW + kC * kK + kC * kC * kK + tid, g3);
-    }
+    // sums over the columns (lanes tg), and for dW1, dW3 over the two halves
 #pragma unroll
-    for (int m = 0; m < kK; ++m) atomicAdd(dW + kC * kK + (cw * kC + cv) * kK + m, g2[m]);
+    for (int o = 1; o < kBG; o <<= 1)
+#pragma unroll
+        for (int m = 0; m < kK; ++m) {
+#pragma unroll
+            for (int i = 0; i < 2; ++i)
+#pragma unroll
+                for (int j = 0; j < 2; ++j) {
+                    g2[i][j][m].x += __shfl_xor_sync(0xffffffffu, g2[i][j][m].x, o);
+                    g2[i][j][m].y += __shfl_xor_sync(0xffffffffu, g2[i][j][m].y, o);
+                }
+            g1[m] += __shfl_xor_sync(0xffffffffu, g1[m], o);
+            g3[m] += __shfl_xor_sync(0xffffffffu, g3[m], o);
+        }
+#pragma unroll
+    for (int m = 0; m < kK; ++m) {
+        g1[m] += __shfl_xor_sync(0xffffffffu, g1[m], kBG);
+        g3[m] += __shfl_xor_sync(0xffffffffu, g3[m], kBG);
+    }
+    if (tg == 0) {
+#pragma unroll
+        for (int m = 0; m < kK; ++m) {
+#pragma unroll
+            for (int i = 0; i < 2; ++i)
+#pragma unroll
+                for (int j = 0; j < 4; ++j)
+                    atomicAdd(dW + kC * kK + ((2 * wc + i) * kC + 4 * wi + j) * kK + m, lane_of(g2[i][j / 2][m], j & 1));
+            if (sh == 0) {
+                atomicAdd(dW + sc * kK + m, g1[m]);
+                atomicAdd(dW + kC * kK + kC * kC * kK + sc * kK + m, g3[m]);
+            }
+        }
+    }
 }
 
 template <typename TQ>
