@@ -28,13 +28,13 @@
 #include <utility>
 #include <vector>
 
+#include "bp_pair.cuh"
 #include "fdkod_internal.cuh"
 #include "tma.cuh"
 
 namespace fdkod {
 namespace {
 
-constexpr int kThreads = kTile * kTile;
 constexpr int kWarps = kThreads / 32;
 
 struct BpParams {
@@ -57,11 +57,6 @@ struct BpParams {
 __device__ __forceinline__ float ld_s(const float *p) { return __ldg(p); }
 __device__ __forceinline__ float ld_s(const __nv_bfloat16 *p) { return __bfloat162float(__ldg(p)); }
 __device__ __forceinline__ float ld_s(const __half *p) { return __half2float(__ldg(p)); }
-
-__device__ __forceinline__ void square_range(int q, int m, int N, int &i0, int &i1) {
-    i0 = (int)(((long long)q * N + m - 1) / m);
-    i1 = (int)((((long long)q + 1) * N + m - 1) / m) - 1;
-}
 
 template <typename TS, bool DIRECT>
 __global__ void __launch_bounds__(kThreads)
@@ -303,17 +298,7 @@ cudaError_t launch_t(BpParams prm, int nsq, cudaStream_t st) {
 }
 
 
-// ---------------------------------------------------------------------------
-// TMA path.  Same tiling and arithmetic as the generic kernel, but each
-// view's window is one 3D bulk-tensor copy (zero fill outside the source),
-// two stages of kViewsPerStage views are in flight (copy of stage c+1
-// overlaps the gather of stage c), the per-view set-up is FP32 only, and the
-// inner loop is
-//   v = fma(1/U, i, v0);  fl = floor(v);  fv = v - fl;  one multiply-add for
-//   the row address;  four shared loads at compile-time offsets;  two column
-//   lerps pre-weighted by U^-2;  row lerp (about 18.7 instructions/update).
-// Waits on the copies are bounded (FDKOD_ERR_TIMEOUT, then drain and exit).
-
+// Parameters of one plan in the batch's persistent launch.
 struct BpTmaParams {
     float *vol;
     const GeomEntry *geo;
@@ -330,610 +315,22 @@ struct BpTmaParams {
     int fault;                   // test hook (kTestFault*), 0 = none
 };
 
-// shared-memory load of one window element at a compile-time byte offset
-// from a 32-bit address, widened to float32
-template <typename TS, int OFF>
-struct Lds;
-template <int OFF>
-struct Lds<float, OFF> {
-    static __device__ __forceinline__ float f(uint32_t addr) {
-        float v;
-        asm volatile("ld.shared.f32 %0, [%1+%2];" : "=f"(v) : "r"(addr), "n"(OFF) : "memory");
-        return v;
-    }
-};
-template <int OFF>
-struct Lds<__nv_bfloat16, OFF> {
-    static __device__ __forceinline__ float f(uint32_t addr) {
-        uint32_t u;
-        asm volatile("ld.shared.u16 %0, [%1+%2];" : "=r"(u) : "r"(addr), "n"(OFF) : "memory");
-        return __uint_as_float(u << 16);  // bfloat16 is the top half of a float32
-    }
-};
-template <int OFF>
-struct Lds<__half, OFF> {
-    static __device__ __forceinline__ float f(uint32_t addr) {
-        unsigned short h;
-        asm volatile("ld.shared.u16 %0, [%1+%2];" : "=h"(h) : "r"(addr), "n"(OFF) : "memory");
-        return __half2float(__ushort_as_half(h));
-    }
-};
-
-// 1 / x for normal x, to an ulp (one MUFU instruction)
-__device__ __forceinline__ float rcp_approx(float x) {
-    float y;
-    asm("rcp.approx.ftz.f32 %0, %1;" : "=f"(y) : "f"(x));
-    return y;
-}
-
 // address bias: (row + kMagicBits) * 4 WD wraps to row * 4 WD in 32 bits once
 // tbase absorbs -kMagicBits * 4 WD (keeps the unsigned arithmetic explicit)
 constexpr int kMagicBits = 0x4B400000;
-constexpr uint64_t kWaitLimitNs = 2000000000ull;
-// test hooks of the failure paths (fdkod_set_test_fault)
-constexpr int kTestFaultSkipCopy = 1;    // CTA 0 leaves out one copy of its chunk 1
-constexpr int kTestFaultSmallWindow = 2; // every window counts as too small
-
-// three CTAs per SM (the shared-memory limit): up to 80 registers per thread
-template <typename TS, bool DIRECT, int WD>
-__global__ void __launch_bounds__(kThreads, 3)
-bp_tma_kernel(const __grid_constant__ CUtensorMap tmap, BpTmaParams a) {
-    constexpr int ES = (int)sizeof(TS);      // window element size (bytes)
-    constexpr int kAl = 16 / ES;             // copy start alignment (elements)
-    extern __shared__ __align__(128) unsigned char smem_raw[];
-    // 128-byte aligned staging area (offset from the shared array itself so
-    // the compiler keeps shared-memory addressing)
-    TS *sm = (TS *)(smem_raw + ((128u - (tma::smem_u32(smem_raw) & 127u)) & 127u));
-    const uint32_t sbase = tma::smem_u32(sm);
-    __shared__ __align__(8) uint64_t bars[2];
-    __shared__ float4 s_pa[2][kViewsPerStage];  // cos, sin, 1/d_c, alpha
-    __shared__ float4 s_pb[2][kViewsPerStage];  // gamma, g, column offset, row offset
-    __shared__ float s_zcr[2][kViewsPerStage];  // z_c / d_c
-    __shared__ int s_tx[2][kViewsPerStage], s_ty[2][kViewsPerStage], s_tz[2][kViewsPerStage];
-    __shared__ int s_skip[2][kViewsPerStage];
-
-    const int tiles = a.tps * a.tps;
-    const int q = blockIdx.x / tiles;
-    const int tt = blockIdx.x - q * tiles;
-    const int qy = q / a.m, qx = q - qy * a.m;
-    int ix0, ix1, iy0, iy1;
-    square_range(qx, a.m, a.N, ix0, ix1);
-    square_range(qy, a.m, a.N, iy0, iy1);
-    const int x0 = ix0 + (tt % a.tps) * kTile;
-    const int y0 = iy0 + (tt / a.tps) * kTile;
-    if (x0 > ix1 || y0 > iy1) return;  // ragged square: empty tile (uniform per CTA)
-    const int xe = min(x0 + kTile - 1, ix1), ye = min(y0 + kTile - 1, iy1);
-    const int z0 = a.zoff + blockIdx.y * kZT;
-    const int z1 = min(z0 + kZT - 1, a.zoff + a.nz - 1);
-
-    const float half_n = 0.5f * (float)(a.N - 1);
-    const float xc = 0.5f * ((float)ix0 + (float)ix1) - half_n;
-    const float yc = 0.5f * ((float)iy0 + (float)iy1) - half_n;
-    // centre of the full kZT-slice slab (also past the volume's end, so the
-    // window always covers every slice the loop evaluates)
-    const float zc = (float)z0 + 0.5f * (float)(kZT - 1) - half_n;
-    const float vcd = 0.5f * (float)(a.Nv - 1);
-
-    const int lx = threadIdx.x % kTile, ly = threadIdx.x / kTile;
-    const int x = x0 + lx, y = y0 + ly;
-    const bool active = x <= xe && y <= ye;
-    const float dx = (float)x - half_n - xc, dy = (float)y - half_n - yc;
-    const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-    const int32_t w0q = a.w0[q];
-    const int nch = (a.nviews + kViewsPerStage - 1) / kViewsPerStage;
-
-    // per-view window and coefficients of chunk c into stage st (warp w = view)
-    auto setup = [&](int c, int st) {
-        const int nj = min(kViewsPerStage, a.nviews - c * kViewsPerStage);
-        if (warp < nj) {
-            const int j = c * kViewsPerStage + warp;
-            const int k = j * a.vstep;
-            const size_t o = (size_t)q * a.P + k;
-            const GeomEntry ge = a.geo[o];
-            const int cbase = DIRECT ? a.crop[o] : 0;
-            const float toff = DIRECT ? ge.frac - (float)w0q : -(float)w0q;
-            const int cc = lane & 7;
-            const float cx = (float)((cc & 1) ? xe : x0) - half_n - xc;
-            const float cy = (float)((cc & 2) ? ye : y0) - half_n - yc;
-            const float cz = (cc & 4) ? 0.5f * (float)(kZT - 1) : -0.5f * (float)(kZT - 1);
-            const float dd = fmaf(ge.cb, cx, ge.sb * cy);
-            const float invU = __fdividef(ge.g_hi, fmaf(ge.r, dd, 1.0f));
-            const float t = fmaf(invU, fmaf(ge.alpha, cx, ge.gamma * cy), toff);
-            const float zcr = zc * ge.r;
-            // z_c g as hi + lo (exact product error by FMA)
-            const float ph = zc * ge.g_hi;
-            const float pl = fmaf(zc, ge.g_lo, fmaf(zc, ge.g_hi, -ph));
-            const float v = (ph + vcd) + (pl + invU * (cz - zcr * dd));
-            float tmin = t, tmax = t, vmin = v, vmax = v;
-#pragma unroll
-            for (int off = 4; off > 0; off >>= 1) {
-                tmin = fminf(tmin, __shfl_xor_sync(0xffffffffu, tmin, off));
-                tmax = fmaxf(tmax, __shfl_xor_sync(0xffffffffu, tmax, off));
-                vmin = fminf(vmin, __shfl_xor_sync(0xffffffffu, vmin, off));
-                vmax = fmaxf(vmax, __shfl_xor_sync(0xffffffffu, vmax, off));
-            }
-            if (lane == 0) {
-                // columns read: floor(t) .. floor(t) + 1 over the tile, with one
-                // sample of slack each side for FP32 rounding
-                const int clo = cbase + (int)floorf(tmin) - 1;
-                const int chi = cbase + (int)floorf(tmax) + 2;
-                const int xs = clo & ~(kAl - 1);  // 16-byte aligned start of the copy
-                const int vlo = (int)floorf(vmin) - 1;
-                const int vhi = (int)floorf(vmax) + 2;
-                const int skip =
-                    (chi - xs > WD - 1) || (vhi - vlo > a.RW - 1) || a.fault == kTestFaultSmallWindow;
-                if (skip) atomicOr(a.status, 1);
-                s_pa[st][warp] = make_float4(ge.cb, ge.sb, ge.r, ge.alpha);
-                s_pb[st][warp] = make_float4(ge.gamma, ge.g_hi, toff - (float)(xs - cbase),
-                                             (ph - ((float)vlo - vcd)) + pl);
-                s_zcr[st][warp] = zcr;
-                s_tx[st][warp] = xs;
-                s_ty[st][warp] = vlo - a.row0;  // row of the source (out of range: zero fill)
-                s_tz[st][warp] = DIRECT ? k : q * a.Pd + j;
-                s_skip[st][warp] = skip;
-            }
-        }
-    };
-    auto issue = [&](int c, int st) {
-        const int nj = min(kViewsPerStage, a.nviews - c * kViewsPerStage);
-        tma::fence_proxy_async();
-        tma::mbar_arrive_expect_tx(&bars[st], (uint32_t)(nj * a.RW * WD * ES));
-        for (int w = 0; w < nj; ++w) {
-            // test hook: the stage's bytes never all arrive, its wait runs out
-            if (a.fault == kTestFaultSkipCopy && c == 1 && w == 0 && blockIdx.x == 0 && blockIdx.y == 0) continue;
-            tma::load_3d(sm + (size_t)(st * kViewsPerStage + w) * a.tile_stride, &tmap, &bars[st], s_tx[st][w],
-                         s_ty[st][w], s_tz[st][w]);
-        }
-    };
-
-    if (threadIdx.x == 0) {
-        tma::mbar_init(&bars[0], 1);
-        tma::mbar_init(&bars[1], 1);
-        tma::fence_mbar_init();
-    }
-    __syncthreads();
-    setup(0, 0);
-    __syncthreads();
-    if (threadIdx.x == 0) issue(0, 0);
-
-    float acc[kZT];
-#pragma unroll
-    for (int i = 0; i < kZT; ++i) acc[i] = 0.f;
-
-    for (int c = 0; c < nch; ++c) {
-        const int st = c & 1;
-        if (c + 1 < nch) setup(c + 1, st ^ 1);
-        __syncthreads();
-        if (c + 1 < nch && threadIdx.x == 0) issue(c + 1, st ^ 1);
-        const bool ok = tma::mbar_wait_bounded(&bars[st], (uint32_t)((c >> 1) & 1), a.wait_ns);
-        if (!__syncthreads_and(ok)) {
-            // a copy never completed: report, let copies in flight land, leave
-            if (threadIdx.x == 0) atomicOr(a.status, 2);
-            tma::mbar_wait_bounded(&bars[st], (uint32_t)((c >> 1) & 1), a.wait_ns);
-            if (c + 1 < nch) tma::mbar_wait_bounded(&bars[st ^ 1], (uint32_t)(((c + 1) >> 1) & 1), a.wait_ns);
-            return;
-        }
-        if (active) {
-            const int nj = min(kViewsPerStage, a.nviews - c * kViewsPerStage);
-            for (int w = 0; w < nj; ++w) {
-                if (s_skip[st][w]) continue;
-                const float4 pa = s_pa[st][w];
-                const float4 pb = s_pb[st][w];
-                const float dd = fmaf(pa.x, dx, pa.y * dy);
-                const float invU = __fdividef(pb.y, fmaf(pa.z, dd, 1.0f));
-                const float t = fmaf(invU, fmaf(pa.w, dx, pb.x * dy), pb.z);
-                const float tf = floorf(t);
-                const float wgt = invU * invU;
-                const float a1 = wgt * (t - tf);
-                const float a0 = wgt - a1;
-                const float vb0 = fmaf(invU, -0.5f * (float)(kZT - 1) - s_zcr[st][w] * dd, pb.w);
-                // 32-bit shared address of sample (row 0, column floor(t));
-                // the row offset folds into one multiply-add per slice
-                const uint32_t tbase = sbase + (uint32_t)ES * ((uint32_t)(st * kViewsPerStage + w) *
-                                                                    (uint32_t)a.tile_stride + (uint32_t)(int)tf) -
-                                       (uint32_t)kMagicBits * (uint32_t)(ES * WD);
-#pragma unroll
-                for (int i = 0; i < kZT; ++i) {
-                    const float v = fmaf(invU, (float)i, vb0);
-                    const float fl = floorf(v);
-                    const float fv = v - fl;
-                    const uint32_t ad = (uint32_t)((int)fl + kMagicBits) * (uint32_t)(ES * WD) + tbase;
-                    const float c0 = fmaf(a1, Lds<TS, ES>::f(ad), a0 * Lds<TS, 0>::f(ad));
-                    const float c1 = fmaf(a1, Lds<TS, ES * WD + ES>::f(ad), a0 * Lds<TS, ES * WD>::f(ad));
-                    acc[i] = fmaf(fv, c1 - c0, acc[i] + c0);
-                }
-            }
-        }
-        __syncthreads();
-    }
-    if (active) {
-#pragma unroll
-        for (int i = 0; i < kZT; ++i)
-            if (z0 + i <= z1) a.vol[((size_t)(z0 + i - a.zoff) * a.N + y) * a.N + x] = acc[i] * a.scale;
-    }
-}
-
-// ---------------------------------------------------------------------------
-// Mirrored-pair form of the staged backprojection (whole volumes).  Each
-// thread owns ZP slices p0 .. p0 + ZP - 1 of the lower half of its (x, y)
-// column and their mirror images N - 1 - p about the mid-plane z = 0.  A
-// voxel and its mirror read the same column (Eq. 1 does not involve z) and
-// mirrored rows: z/U + (Nv-1)/2 and -z/U + (Nv-1)/2 add up to Nv - 1.  So
-// the column weights, the row fraction and the per-view set-up are shared
-// by the pair, and with the two windows of a view staged at row origins vlo
-// and vlo', the mirror's window row is C - v for C = Nv - 1 - vlo - vlo'.
-//
-// What bounds it is instruction issue (a packed two-lane FP32 instruction
-// reads its operands over two issue slots) together with the shared-memory
-// path.  So slices go in groups that read consecutive rows at compile-time
-// offsets from one address (pair_slices): no address, row or fraction
-// arithmetic in integers per slice, and each row is loaded and
-// column-interpolated once per group, also where 1/U > 1 (before: both rows
-// of every such slice).  ncu, 256^3 x 90 views: 28.7 -> 22.4 warp instructions
-// and 6.5 -> 5.0 shared loads per slice pair.  A warp covers 8 x 4 columns (16 x 2:
-// 5 % bank conflicts, now none).  Backprojection of 512^3 x 180 views:
-// 10.80 ms before, 8.77 ms with ZP = 16, 8.30 ms with ZP = 32.
-struct BpPairParams {
-    float *vol;
-    const GeomEntry *geo;
-    const int32_t *crop;
-    const int32_t *w0;
-    int *status;
-    int N, P, Nv, m, tps;
-    int nviews, vstep, Pd;
-    int RW, tile_stride;  // rows of a ZP-slice window; elements per staged window
-    int pbase, pend;      // slice pairs pbase .. pend - 1 (pair p: slices p and N - 1 - p)
-    float scale;
-    unsigned long long wait_ns;
-    int fault;
-};
-
-// Column-interpolated samples (U^-2 weighted) of the pair's row r + K: lower
-// window row r + K at aL + K ROWB, upper window row C - r - K at aU - K ROWB.
-template <typename TS, uint32_t ROWB, int K>
-__device__ __forceinline__ float2 pair_row(uint32_t aL, uint32_t aU, float2 A0, float2 A1) {
-    constexpr int ES = (int)sizeof(TS);
-    constexpr int OL = K * (int)ROWB, OU = -K * (int)ROWB;
-    return __ffma2_rn(A1, make_float2(Lds<TS, OL + ES>::f(aL), Lds<TS, OU + ES>::f(aU)),
-                      __fmul2_rn(A0, make_float2(Lds<TS, OL>::f(aL), Lds<TS, OU>::f(aU))));
-}
-
-// One slice of a group: with t in [-1, 1) the row coordinate relative to the
-// middle one of three consecutive rows c0, c1, c2, the row interpolation is
-// (1 - |t|) c1 + |t| (t < 0 ? c0 : c2): no row but the two around the sample
-// enters it (t itself scalar: a packed add of both lanes measured 3 % slower).
-template <typename TS, uint32_t ROWB, int G, int I>
-__device__ __forceinline__ void pair_group(float2 *acc, float2 c0, float2 c1, float t, float du, uint32_t aL,
-                                           uint32_t aU, float2 A0, float2 A1) {
-    if constexpr (I < G) {
-        const float2 c2 = pair_row<TS, ROWB, I + 2>(aL, aU, A0, A1);
-        const bool lo = t < 0.f;
-        const float2 y = make_float2(lo ? -c0.x : c2.x, lo ? -c0.y : c2.y);
-        const float w1 = 1.0f - fabsf(t);
-        acc[I] = __ffma2_rn(make_float2(t, t), y, __ffma2_rn(make_float2(w1, w1), c1, acc[I]));
-        pair_group<TS, ROWB, G, I + 1>(acc, c1, c2, t + du, du, aL, aU, A0, A1);
-    }
-}
-
-// floor of |x| < 2^22 through the float 1.5 2^23 + floor(x) (unit spacing,
-// rounded down): its bits are kFloorBits + floor(x), so an address takes one
-// multiply-add, and no conversion instruction is needed
-constexpr float kFloorBias = 12582912.0f;  // 1.5 * 2^23
-constexpr uint32_t kFloorBits = 0x4B400000u;
-__device__ __forceinline__ float floor_biased(float x) { return __fadd_rd(x, kFloorBias); }
-
-// The ZP slice pairs of one column in groups of G consecutive ones, for a
-// drift |1/U - 1| of at most 1 / (G - 1) rows per slice: then slice g + i of
-// a group reads two of the rows b + i, b + i + 1, b + i + 2 for one b, so a
-// group loads G + 2 rows at compile-time offsets from one address.  w is the
-// window row of the slab's centre less the centre's slice number: a number of
-// a few rows whatever ZP, so its rounding stays below a row coordinate's.
-template <typename TS, uint32_t ROWB, int G, int ZP>
-__device__ __forceinline__ void pair_slices(float2 (&acc)[ZP], float w, float du, uint32_t bL, uint32_t KU,
-                                            float2 A0, float2 A1) {
-#pragma unroll
-    for (int g = 0; g < ZP; g += G) {
-        // window row less slice number at the group's ends
-        const float first = fmaf((float)g - 0.5f * (float)(ZP - 1), du, w);
-        const float last = fmaf((float)(g + G - 1) - 0.5f * (float)(ZP - 1), du, w);
-        const float bm = floor_biased(fminf(first, last));
-        const float t0 = first - (bm - (kFloorBias - 1.0f));  // first - (b + 1), exact
-        const uint32_t aL = __float_as_uint(bm) * ROWB + (bL + ((uint32_t)g - kFloorBits) * ROWB), aU = KU - aL;
-        pair_group<TS, ROWB, G, 0>(acc + g, pair_row<TS, ROWB, 0>(aL, aU, A0, A1),
-                                   pair_row<TS, ROWB, 1>(aL, aU, A0, A1), t0, du, aL, aU, A0, A1);
-    }
-}
-
-// Any 1/U: both rows of every slice at an address of its own.  Row
-// coordinates in 9.23 fixed point: the row is V >> 23, the fraction's float
-// is V's mantissa bits under the exponent of 1.0.
-template <typename TS, uint32_t ROWB, int ZP>
-__device__ __forceinline__ void pair_slices_any(float2 (&acc)[ZP], float w, float invU, uint32_t bL, uint32_t KU,
-                                                float2 A0, float2 A1) {
-    constexpr float kFix = 8388608.0f;  // 2^23
-    uint32_t V = __float2uint_rn(fmaf(-0.5f * (float)(ZP - 1), invU - 1.0f, w) * kFix);
-    const uint32_t dV = __float2uint_rn(invU * kFix);
-#pragma unroll
-    for (int i = 0; i < ZP; ++i) {
-        const uint32_t aL = (V >> 23) * ROWB + bL, aU = KU - aL;
-        const float2 A = pair_row<TS, ROWB, 0>(aL, aU, A0, A1), B = pair_row<TS, ROWB, 1>(aL, aU, A0, A1);
-        // fb = 1 + f exactly, so 1 - f and f are exact
-        const float fb = __uint_as_float((V & 0x7fffffu) | 0x3f800000u);
-        const float f = fb - 1.0f, g = 2.0f - fb;
-        acc[i] = __ffma2_rn(make_float2(f, f), B, __ffma2_rn(make_float2(g, g), A, acc[i]));
-        V += dV;
-    }
-}
-
-// Warp-specialised: warp 8 is the producer (per chunk of VPS views it finds
-// the windows, writes the view parameters and issues the copies into a ring
-// of kPairSlots slots); warps 0-7 consume.  A slot is full when its copies
-// have landed (full[slot], which also publishes the producer's parameters)
-// and free again when all eight consumer warps have arrived on empty[slot]:
-// no block-wide barrier inside the view loop, so consumer warps drift within
-// the ring instead of waiting for the slowest.  Every wait is bounded
-// (FDKOD_ERR_TIMEOUT); a producer that gives up waits for its copies in
-// flight before it leaves.  The producer polls `empty` (mbarrier.test_wait):
-// suspended in mbarrier.try_wait it was measured to resume late (the whole
-// kernel 1.4x slower); the consumers' waits on `full` are mostly satisfied
-// at once and suspend (polling them measured no faster).
-struct PairView {
-    float4 a;   // cos, sin, 1/d_c, alpha
-    float4 b;   // gamma, g, column offset, window row of the lower slab's centre less its slice number
-    float zcr;  // z_c / d_c (lower slab)
-    int group;  // slices per group (pair_slices), 0: any drift, -1: window too small, skip the view
-    // byte addresses of row 0, column -kFloorBits of the lower window, and of
-    // row C of the upper one plus the former (row r of the lower window at
-    // aL = baseL + r ROWB + ..., row C - r of the upper one at KU - aL)
-    uint32_t baseL, KU;
-};
-constexpr int kPairSlots = 3;
-// a group's first or last row may lie one row outside its window (such a row
-// never enters a sum): one row of the widest window before and after the ring
-constexpr int kPairPad = 512;
-constexpr int kPairViews = 2;                      // views per slot, at most (16 producer lanes each)
-constexpr int kPairConsumers = kThreads / 32;      // 8
-constexpr int kPairThreads = kThreads + 32;        // plus the producer warp
-// CTAs per SM: registers decide (2 ZP accumulators per thread)
-constexpr int pair_ctas(int ZP) { return ZP == 32 ? 2 : 3; }
-
-template <typename TS, bool DIRECT, int WD, int ZP, int VPS>
-__global__ void __launch_bounds__(kPairThreads, pair_ctas(ZP))
-bp_pair_kernel(const __grid_constant__ CUtensorMap tmap, BpPairParams a) {
-    constexpr int ES = (int)sizeof(TS);
-    constexpr int kAl = 16 / ES;
-    constexpr uint32_t ROWB = (uint32_t)(ES * WD);  // bytes per window row
-    static_assert(VPS <= kPairViews, "the producer warp sets up a view on 16 lanes");
-    extern __shared__ __align__(128) unsigned char smem_raw[];
-    TS *sm = (TS *)(smem_raw + ((128u - (tma::smem_u32(smem_raw) & 127u)) & 127u) + kPairPad);
-    const uint32_t sbase = tma::smem_u32(sm);
-    __shared__ __align__(8) uint64_t full[kPairSlots], empty[kPairSlots];
-    __shared__ PairView s_view[kPairSlots * VPS];
-
-    const int tiles = a.tps * a.tps;
-    const int q = blockIdx.x / tiles;
-    const int tt = blockIdx.x - q * tiles;
-    const int qy = q / a.m, qx = q - qy * a.m;
-    int ix0, ix1, iy0, iy1;
-    square_range(qx, a.m, a.N, ix0, ix1);
-    square_range(qy, a.m, a.N, iy0, iy1);
-    const int x0 = ix0 + (tt % a.tps) * kTile;
-    const int y0 = iy0 + (tt / a.tps) * kTile;
-    if (x0 > ix1 || y0 > iy1) return;  // ragged square: empty tile (uniform per CTA)
-    const int xe = min(x0 + kTile - 1, ix1), ye = min(y0 + kTile - 1, iy1);
-    const int p0 = a.pbase + blockIdx.y * ZP;  // first slice pair
-
-    const float half_n = 0.5f * (float)(a.N - 1);
-    const float xc = 0.5f * ((float)ix0 + (float)ix1) - half_n;
-    const float yc = 0.5f * ((float)iy0 + (float)iy1) - half_n;
-    // centre of the lower slab (the upper one is centred at -zc)
-    const float zc = (float)p0 + 0.5f * (float)(ZP - 1) - half_n;
-    const float vcd = 0.5f * (float)(a.Nv - 1);
-    const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-    const int nch = (a.nviews + VPS - 1) / VPS;
-    // window of view w of slot sl, lower (h = 0) or upper (h = 1) slab
-    auto win = [&](int sl, int w, int h) { return (uint32_t)((sl * VPS + w) * 2 + h) * (uint32_t)a.tile_stride; };
-
-    if (threadIdx.x == 0) {
-        for (int i = 0; i < kPairSlots; ++i) {
-            tma::mbar_init(&full[i], 1);
-            tma::mbar_init(&empty[i], kPairConsumers);
-        }
-        tma::fence_mbar_init();
-    }
-    __syncthreads();
-
-    if (warp == kPairConsumers) {
-        // ---- producer: lanes 16 w .. 16 w + 15 set up view w of the chunk,
-        // 0-7 of them at the corners of the lower slab, 8-15 of the upper
-        const int32_t w0q = a.w0[q];
-        const int w = lane >> 4, cc = lane & 7;
-        const float zcl = (lane & 8) ? -zc : zc;
-        const float cx = (float)((cc & 1) ? xe : x0) - half_n - xc;
-        const float cy = (float)((cc & 2) ? ye : y0) - half_n - yc;
-        const float cz = (cc & 4) ? 0.5f * (float)(ZP - 1) : -0.5f * (float)(ZP - 1);
-        int c = 0;
-        for (; c < nch; ++c) {
-            const int sl = c % kPairSlots;
-            const int nj = min(VPS, a.nviews - c * VPS);
-            const int j = c * VPS + min(w, nj - 1);  // lanes past the chunk repeat its last view
-            const int k = j * a.vstep;
-            const size_t o = (size_t)q * a.P + k;
-            const GeomEntry ge = a.geo[o];
-            const int cbase = DIRECT ? a.crop[o] : 0;
-            const float toff = DIRECT ? ge.frac - (float)w0q : -(float)w0q;
-            const float dd = fmaf(ge.cb, cx, ge.sb * cy);
-            const float invU = __fdividef(ge.g_hi, fmaf(ge.r, dd, 1.0f));
-            const float t = fmaf(invU, fmaf(ge.alpha, cx, ge.gamma * cy), toff);
-            const float zcr = zcl * ge.r;
-            // z_c g as hi + lo (exact product error by FMA)
-            const float ph = zcl * ge.g_hi;
-            const float pl = fmaf(zcl, ge.g_lo, fmaf(zcl, ge.g_hi, -ph));
-            const float v = (ph + vcd) + (pl + invU * (cz - zcr * dd));
-            float tmin = t, tmax = t, vmin = v, vmax = v;
-#pragma unroll
-            for (int off = 4; off > 0; off >>= 1) {  // within each half's 8 corners
-                vmin = fminf(vmin, __shfl_xor_sync(0xffffffffu, vmin, off));
-                vmax = fmaxf(vmax, __shfl_xor_sync(0xffffffffu, vmax, off));
-            }
-#pragma unroll
-            for (int off = 8; off > 0; off >>= 1) {  // columns: both halves
-                tmin = fminf(tmin, __shfl_xor_sync(0xffffffffu, tmin, off));
-                tmax = fmaxf(tmax, __shfl_xor_sync(0xffffffffu, tmax, off));
-            }
-            const float vmin2 = __shfl_down_sync(0xffffffffu, vmin, 8);
-            const float vmax2 = __shfl_down_sync(0xffffffffu, vmax, 8);
-            // lane 16 w: columns read floor(t) .. floor(t) + 1 over the tile,
-            // one sample of slack each side for FP32 rounding
-            const int clo = cbase + (int)floorf(tmin) - 1;
-            const int chi = cbase + (int)floorf(tmax) + 2;
-            const int xs = clo & ~(kAl - 1);  // 16-byte aligned start of the copy
-            const int vlo = (int)floorf(vmin) - 1, vhi = (int)floorf(vmax) + 2;
-            const int vlo2 = (int)floorf(vmin2) - 1, vhi2 = (int)floorf(vmax2) + 2;
-            // largest drift per slice over the tile (1/U is monotone in x
-            // and y), with a margin for rounding
-            float drift = fabsf(invU - 1.0f);
-#pragma unroll
-            for (int off = 2; off > 0; off >>= 1) drift = fmaxf(drift, __shfl_xor_sync(0xffffffffu, drift, off));
-            // round r of a slot may start once its round r - 1 was consumed
-            // (lane 0 waits; the warp follows its answer)
-            bool ok = true;
-            if (c >= kPairSlots && lane == 0)
-                ok = tma::mbar_wait_spin(&empty[sl], (uint32_t)(((c / kPairSlots) & 1) ^ 1), a.wait_ns);
-            if (!__shfl_sync(0xffffffffu, ok, 0)) {
-                if (lane == 0) atomicOr(a.status, 2);
-                break;
-            }
-            const bool lead = (lane & 15) == 0 && w < nj;
-            if (lead) {
-                const bool skip = (chi - xs > WD - 1) || (vhi - vlo > a.RW - 1) || (vhi2 - vlo2 > a.RW - 1) ||
-                                  a.fault == kTestFaultSmallWindow;
-                if (skip) atomicOr(a.status, 1);
-                PairView &pv = s_view[sl * VPS + w];
-                pv.a = make_float4(ge.cb, ge.sb, ge.r, ge.alpha);
-                pv.b = make_float4(ge.gamma, ge.g_hi, toff - (float)(xs - cbase),
-                                   (ph - ((float)vlo - vcd + 0.5f * (float)(ZP - 1))) + pl);
-                pv.zcr = zcr;
-                pv.group = skip ? -1
-                           : drift * 15.f < 0.999f ? 16
-                           : drift * 7.f < 0.999f  ? 8
-                           : drift * 3.f < 0.999f  ? 4
-                                                   : 0;
-                const uint32_t bL = sbase + (uint32_t)ES * (win(sl, w, 0) - kFloorBits);
-                const uint32_t bU = sbase + (uint32_t)ES * (win(sl, w, 1) - kFloorBits);
-                pv.baseL = bL;
-                pv.KU = (uint32_t)((a.Nv - 1) - vlo - vlo2) * ROWB + bU + bL;
-            }
-            // the copies: lane 0 for every view of the chunk
-            const int xs0 = __shfl_sync(0xffffffffu, xs, 0), xs1 = __shfl_sync(0xffffffffu, xs, 16);
-            const int vl0 = __shfl_sync(0xffffffffu, vlo, 0), vl1 = __shfl_sync(0xffffffffu, vlo, 16);
-            const int vu0 = __shfl_sync(0xffffffffu, vlo2, 0), vu1 = __shfl_sync(0xffffffffu, vlo2, 16);
-            const int tz = DIRECT ? k : q * a.Pd + j;
-            const int tz0 = __shfl_sync(0xffffffffu, tz, 0), tz1 = __shfl_sync(0xffffffffu, tz, 16);
-            __syncwarp();  // the parameters are written before lane 0 publishes them
-            if (lane == 0) {
-                tma::fence_proxy_async();
-                tma::mbar_arrive_expect_tx(&full[sl], (uint32_t)(nj * 2 * a.RW * WD * ES));
-                for (int v2 = 0; v2 < nj; ++v2) {
-                    // test hook: the slot's bytes never all arrive, its wait runs out
-                    if (a.fault == kTestFaultSkipCopy && c == 1 && v2 == 0 && blockIdx.x == 0 && blockIdx.y == 0)
-                        continue;
-                    const int x = v2 == 0 ? xs0 : xs1, z = v2 == 0 ? tz0 : tz1;
-                    tma::load_3d(sm + win(sl, v2, 0), &tmap, &full[sl], x, v2 == 0 ? vl0 : vl1, z);
-                    tma::load_3d(sm + win(sl, v2, 1), &tmap, &full[sl], x, v2 == 0 ? vu0 : vu1, z);
-                }
-            }
-            __syncwarp();
-        }
-        // copies still in flight must land before the CTA may exit
-        if (lane == 0)
-            for (int m = max(0, c - kPairSlots); m < c; ++m)
-                tma::mbar_wait_bounded(&full[m % kPairSlots], (uint32_t)((m / kPairSlots) & 1), a.wait_ns);
-        return;
-    }
-
-    // ---- consumers.  A voxel and its mirror go through the same operations
-    // on different samples, so they share packed two-lane FP32 instructions
-    // (x: lower slab, y: upper slab; each lane rounds as the scalar
-    // operation would): half the arithmetic instructions of two scalar
-    // updates.
-    const int x = x0 + (warp & 1) * 8 + (lane & 7), y = y0 + (warp >> 1) * 4 + (lane >> 3);
-    const bool active = x <= xe && y <= ye;
-    // threads outside a ragged tile repeat its last column (inside the
-    // window) and store nothing
-    const float dx = (float)min(x, xe) - half_n - xc, dy = (float)min(y, ye) - half_n - yc;
-    float2 acc[ZP];  // (lower slab, upper mirrored slab)
-#pragma unroll
-    for (int i = 0; i < ZP; ++i) acc[i] = make_float2(0.f, 0.f);
-
-    int sl = 0, left = a.nviews;
-    uint32_t phase = 0;
-    for (; left > 0; left -= VPS) {
-        const bool ok = tma::mbar_wait_bounded(&full[sl], phase, a.wait_ns);
-        if (!__all_sync(0xffffffffu, ok)) {
-            if (lane == 0) atomicOr(a.status, 2);
-            return;  // the producer waits for the copies in flight
-        }
-        const PairView *pv = s_view + sl * VPS, *pe = pv + min(VPS, left);
-#pragma unroll 1
-        for (; pv != pe; ++pv) {
-            const int group = pv->group;  // uniform per CTA
-            const float4 pa = pv->a;
-            const float4 pb = pv->b;
-            const float dd = fmaf(pa.x, dx, pa.y * dy);
-            // one Newton step on the reciprocal: its error scales with the
-            // distance from the slab's centre, which 32 pairs double
-            const float den = fmaf(pa.z, dd, 1.0f), r0 = rcp_approx(den);
-            const float invU = pb.y * fmaf(r0, fmaf(-den, r0, 1.0f), r0);
-            const float du = invU - 1.0f;
-            const float t = fmaf(invU, fmaf(pa.w, dx, pb.x * dy), pb.z);
-            const float tm = floor_biased(t);
-            const float wgt = invU * invU;
-            const float a1 = wgt * (t - (tm - kFloorBias));
-            const float a0 = wgt - a1;
-            const float2 A1 = make_float2(a1, a1), A0 = make_float2(a0, a0);
-            // window row of the column at the lower slab's centre, less the
-            // centre's slice number
-            const float wc = fmaf(-invU, pv->zcr * dd, pb.w);
-            const uint32_t col = (uint32_t)ES * __float_as_uint(tm);
-            const uint32_t bL = pv->baseL + col, KU = pv->KU + 2u * col;
-            if (group == 16) {
-                pair_slices<TS, ROWB, 16, ZP>(acc, wc, du, bL, KU, A0, A1);
-            } else if (group == 8) {
-                pair_slices<TS, ROWB, 8, ZP>(acc, wc, du, bL, KU, A0, A1);
-            } else if (group == 4) {
-                pair_slices<TS, ROWB, 4, ZP>(acc, wc, du, bL, KU, A0, A1);
-            } else if (group == 0) {
-                pair_slices_any<TS, ROWB, ZP>(acc, wc, invU, bL, KU, A0, A1);
-            }
-        }
-        __syncwarp();
-        if (lane == 0) tma::mbar_arrive(&empty[sl]);  // this warp is done with the slot
-        if (++sl == kPairSlots) {
-            sl = 0;
-            phase ^= 1u;
-        }
-    }
-    if (active) {
-#pragma unroll
-        for (int i = 0; i < ZP; ++i) {
-            const int pz = p0 + i;
-            if (pz < a.pend) {
-                const int zu = a.N - 1 - pz;
-                a.vol[((size_t)pz * a.N + y) * a.N + x] = acc[i].x * a.scale;
-                if (zu != pz) a.vol[((size_t)zu * a.N + y) * a.N + x] = acc[i].y * a.scale;
-            }
-        }
-    }
-}
-
 // ---------------------------------------------------------------------------
 // Persistent form for a batch of plans (float32 windows): one launch, as
 // many CTAs as fit the GPU, each taking work items (plan, tile, z-slab) from
-// an atomic counter until the list is exhausted; per item the arithmetic of
-// bp_tma_kernel, with the plan's tensor map and parameters read from global
-// memory and the window width a run-time value (the second window row is one
-// add away).  The mbarrier stages continue from item to item.
+// an atomic counter until the list is exhausted.  Same tiling as the generic
+// kernel; each view's window is one 3D bulk-tensor copy (zero fill outside
+// the source), two stages of kViewsPerStage views are in flight (the copy of
+// stage c + 1 overlaps the gather of stage c), the per-view set-up is FP32
+// only, and per slice: v = fma(1/U, i, v0), floor, fraction, one multiply-add
+// for the row address, four shared loads, two column lerps pre-weighted by
+// U^-2, row lerp.  The plan's tensor map and parameters are read from global
+// memory and the window width is a run-time value (the second window row is
+// one add away).  The mbarrier stages continue from item to item; waits on
+// the copies are bounded (FDKOD_ERR_TIMEOUT, then drain and exit).
 struct BatchInst {
     BpTmaParams a;
     int direct, WD;
@@ -1116,57 +513,33 @@ bp_persistent_kernel(const CUtensorMap *__restrict__ maps, const BatchInst *__re
     }
 }
 
-template <typename TS, bool DIRECT, int WD>
-cudaError_t launch_tma_t(const CUtensorMap &map, const BpTmaParams &prm, int nsq, cudaStream_t st) {
-    const size_t smem = sizeof(TS) * (size_t)2 * kViewsPerStage * prm.tile_stride + 128;
-    cudaError_t e = ensure_smem<bp_tma_kernel<TS, DIRECT, WD>>(smem);
-    if (e != cudaSuccess) return e;
-    dim3 grid((unsigned)(nsq * prm.tps * prm.tps), (unsigned)((prm.nz + kZT - 1) / kZT));
-    bp_tma_kernel<TS, DIRECT, WD><<<grid, kThreads, smem, st>>>(map, prm);
-    return cudaGetLastError();
+// Tensor map of a source (Q itself, or the decomposed data, float32) that
+// holds `rows` detector rows, with boxes of WD columns x `box_rows` rows.
+// False where TMA cannot describe it: the source must be 16-byte aligned, its
+// rows whole 16-byte units, and the window must fit a box (WD != 0, <= 256
+// rows).
+bool source_map(const PlanImpl &p, const SquareSet &ss, bool direct, const void *src, int rows, int WD, int box_rows,
+                CUtensorMap &map) {
+    const int es = (direct && p.qtype != FDKOD_F32) ? 2 : 4;
+    if (WD == 0 || box_rows > 256 || ((uintptr_t)src & 15) != 0) return false;
+    if (direct && ((size_t)p.g.Nu * es) % 16 != 0) return false;
+    const uint64_t cols = direct ? (uint64_t)p.g.Nu : (uint64_t)p.Tstride;
+    const uint64_t dims[3] = {cols, (uint64_t)rows, direct ? (uint64_t)p.g.P : (uint64_t)ss.nsq * p.Pd};
+    const uint64_t strides[2] = {cols * es, cols * es * (uint64_t)rows};
+    const uint32_t box[3] = {(uint32_t)WD, (uint32_t)box_rows, 1u};
+    const CUtensorMapDataType dt = es == 4 ? CU_TENSOR_MAP_DATA_TYPE_FLOAT32
+                                   : (p.qtype == FDKOD_F16 ? CU_TENSOR_MAP_DATA_TYPE_FLOAT16
+                                                           : CU_TENSOR_MAP_DATA_TYPE_BFLOAT16);
+    return encode_map_3d(&map, dt, src, dims, strides, box) == cudaSuccess;
 }
 
-template <typename TS, bool DIRECT>
-cudaError_t launch_tma_w(int WD, const CUtensorMap &map, const BpTmaParams &prm, int nsq, cudaStream_t st) {
-    switch (WD) {
-        case 32: return launch_tma_t<TS, DIRECT, 32>(map, prm, nsq, st);
-        case 48: return launch_tma_t<TS, DIRECT, 48>(map, prm, nsq, st);
-        case 64: return launch_tma_t<TS, DIRECT, 64>(map, prm, nsq, st);
-        case 96: return launch_tma_t<TS, DIRECT, 96>(map, prm, nsq, st);
-        case 128: return launch_tma_t<TS, DIRECT, 128>(map, prm, nsq, st);
-    }
-    return cudaErrorInvalidValue;
-}
-
-// The TMA path applies when the source is 16-byte aligned, its rows are whole
-// 16-byte units, and the window fits a box (<= 256 rows, width an
-// instantiated WD).  The decomposed data is float32; Q may be 16-bit.
-// Fills the tensor map, the parameters and the window width; false when the
-// TMA path does not apply.
+// Tensor map, parameters and window width of a plan in the batch's persistent
+// launch; false when it cannot take it.
 bool make_tma_launch(const PlanImpl &p, const SquareSet &ss, bool direct, const void *src, float *vol,
                      const Band &b, CUtensorMap &map, BpTmaParams &a, int &WD) {
     const int es = (direct && p.qtype != FDKOD_F32) ? 2 : 4;
     WD = es == 4 ? ss.WdT : ss.WdT16;
-    if (WD == 0 || ss.Rw > 256 || ((uintptr_t)src & 15) != 0) return false;
-    if (direct && ((size_t)p.g.Nu * es) % 16 != 0) return false;
-    uint64_t dims[3], strides[2];
-    if (direct) {
-        dims[0] = (uint64_t)p.g.Nu;
-        dims[1] = (uint64_t)b.nrows;
-        dims[2] = (uint64_t)p.g.P;
-        strides[0] = (uint64_t)p.g.Nu * es;
-    } else {
-        dims[0] = (uint64_t)p.Tstride;
-        dims[1] = (uint64_t)b.nrows;
-        dims[2] = (uint64_t)ss.nsq * p.Pd;
-        strides[0] = (uint64_t)p.Tstride * sizeof(float);
-    }
-    strides[1] = strides[0] * dims[1];
-    const uint32_t box[3] = {(uint32_t)WD, (uint32_t)ss.Rw, 1u};
-    const CUtensorMapDataType dt = es == 4 ? CU_TENSOR_MAP_DATA_TYPE_FLOAT32
-                                   : (p.qtype == FDKOD_F16 ? CU_TENSOR_MAP_DATA_TYPE_FLOAT16
-                                                           : CU_TENSOR_MAP_DATA_TYPE_BFLOAT16);
-    if (encode_map_3d(&map, dt, src, dims, strides, box) != cudaSuccess) return false;  // generic path
+    if (!source_map(p, ss, direct, src, b.nrows, WD, ss.Rw, map)) return false;
     a = BpTmaParams{};
     a.vol = vol;
     a.geo = ss.geo;
@@ -1199,64 +572,6 @@ bool make_tma_launch(const PlanImpl &p, const SquareSet &ss, bool direct, const 
     return true;
 }
 
-cudaError_t try_launch_tma(const PlanImpl &p, const SquareSet &ss, bool direct, const void *src, float *vol,
-                           cudaStream_t st, const Band &b, bool &launched) {
-    launched = false;
-    CUtensorMap map;
-    BpTmaParams a;
-    int WD = 0;
-    if (!make_tma_launch(p, ss, direct, src, vol, b, map, a, WD)) return cudaSuccess;
-    launched = true;
-    if (!direct) return launch_tma_w<float, false>(WD, map, a, ss.nsq, st);
-    switch (p.qtype) {
-        case FDKOD_F32: return launch_tma_w<float, true>(WD, map, a, ss.nsq, st);
-        case FDKOD_BF16: return launch_tma_w<__nv_bfloat16, true>(WD, map, a, ss.nsq, st);
-        case FDKOD_F16: return launch_tma_w<__half, true>(WD, map, a, ss.nsq, st);
-    }
-    return cudaErrorInvalidValue;
-}
-
-// elements per staged window of the pair kernel, a 128-byte multiple
-inline int pair_tile_stride(int es, int rows, int WD) { return (rows * WD + (128 / es - 1)) & ~(128 / es - 1); }
-
-// dynamic shared memory of the pair kernel: kPairSlots slots of VPS views,
-// two windows per view, plus the pads and the 128-byte alignment slack
-inline size_t pair_smem(int es, int vps, int tile_stride) {
-    return (size_t)es * kPairSlots * vps * 2 * tile_stride + 2 * kPairPad + 128;
-}
-
-template <typename TS, bool DIRECT, int WD, int ZP, int VPS>
-cudaError_t launch_pair_t(const CUtensorMap &map, const BpPairParams &prm, int nsq, cudaStream_t st) {
-    const size_t smem = pair_smem((int)sizeof(TS), VPS, prm.tile_stride);
-    cudaError_t e = ensure_smem<bp_pair_kernel<TS, DIRECT, WD, ZP, VPS>>(smem);
-    if (e != cudaSuccess) return e;
-    dim3 grid((unsigned)(nsq * prm.tps * prm.tps), (unsigned)((prm.pend - prm.pbase + ZP - 1) / ZP));
-    bp_pair_kernel<TS, DIRECT, WD, ZP, VPS><<<grid, kPairThreads, smem, st>>>(map, prm);
-    return cudaGetLastError();
-}
-
-// 32 slice pairs per CTA always come with 2 views per slot (pair_slices_per_cta)
-template <typename TS, bool DIRECT, int WD>
-cudaError_t launch_pair_z(int zp, int vps, const CUtensorMap &map, const BpPairParams &prm, int nsq,
-                          cudaStream_t st) {
-    if (zp == 32) return launch_pair_t<TS, DIRECT, WD, 32, 2>(map, prm, nsq, st);
-    return vps == 2 ? launch_pair_t<TS, DIRECT, WD, 16, 2>(map, prm, nsq, st)
-                    : launch_pair_t<TS, DIRECT, WD, 16, 1>(map, prm, nsq, st);
-}
-
-template <typename TS, bool DIRECT>
-cudaError_t launch_pair_w(int WD, int zp, int vps, const CUtensorMap &map, const BpPairParams &prm, int nsq,
-                          cudaStream_t st) {
-    switch (WD) {
-        case 32: return launch_pair_z<TS, DIRECT, 32>(zp, vps, map, prm, nsq, st);
-        case 48: return launch_pair_z<TS, DIRECT, 48>(zp, vps, map, prm, nsq, st);
-        case 64: return launch_pair_z<TS, DIRECT, 64>(zp, vps, map, prm, nsq, st);
-        case 96: return launch_pair_z<TS, DIRECT, 96>(zp, vps, map, prm, nsq, st);
-        case 128: return launch_pair_z<TS, DIRECT, 128>(zp, vps, map, prm, nsq, st);
-    }
-    return cudaErrorInvalidValue;
-}
-
 // opt-in shared memory per block of the current device, less room for the
 // kernels' static shared memory; *per_sm: the SM's shared memory less what
 // the runtime reserves per block, shared by the CTAs of an SM
@@ -1283,59 +598,39 @@ int pair_views(int es, int zp, int rows, int WD) {
     return pair_smem(es, 1, ts) <= budget ? 1 : 0;
 }
 
-// Slice pairs per CTA of the pair kernel, 0 where it does not apply (the
-// TMA conditions of make_tma_launch).  32 pairs per thread halve the
-// per-view set-up and stage fewer margin rows (512^3: 8.30 ms against 8.75 at
-// 16), but need enough CTAs: 2 per SM, half as many of them; measured at
-// 128^3 (128 CTAs) 16 is the faster one.  A rule on the plan alone, so that
-// launches over part of the volume round as the whole one does.
-int pair_slices_per_cta(const PlanImpl &p, const SquareSet &ss, bool direct, int &vps) {
+// The pair kernel's shape for `pairs` pairs of slices per column; false where
+// it does not apply (no window width, or windows too large to stage).  32
+// pairs per thread halve the per-view set-up and stage fewer margin rows
+// (512^3: 8.30 ms against 8.75 at 16), but need enough CTAs: 2 per SM, half as
+// many of them (from 160^3 to 256^3 both take the same time within 4 %), and
+// they must not compute much more than they keep (the last slab's excess).
+bool pair_shape(const PlanImpl &p, const SquareSet &ss, bool direct, bool mirror, int pairs, PairShape &s) {
     const int es = (direct && p.qtype != FDKOD_F32) ? 2 : 4;
-    const int WD = es == 4 ? ss.WdT : ss.WdT16;
-    vps = 0;
-    if (WD == 0) return 0;
+    s.WD = es == 4 ? ss.WdT : ss.WdT16;
+    s.mirror = mirror;
+    if (s.WD == 0) return false;
     const long long tiles = (long long)ss.nsq * ss.tiles_per_side * ss.tiles_per_side;
     int dev = 0, sms = 148;
     if (cudaGetDevice(&dev) == cudaSuccess) cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
-    if (ss.Rw <= 256 && tiles * (((p.g.N + 1) / 2 + 31) / 32) >= 2LL * pair_ctas(32) * sms &&
-        (vps = pair_views(es, 32, ss.Rw, WD)) == 2)
-        return 32;
-    if (ss.Rw2 <= 256 && (vps = pair_views(es, 16, ss.Rw2, WD)) > 0) return 16;
-    return 0;
+    const int n32 = (pairs + 31) / 32, n16 = (pairs + 15) / 16;
+    s.zp = 32;
+    if (ss.Rw <= 256 && tiles * n32 >= 2LL * pair_ctas(32) * sms && 64 * n32 <= 34 * n16 &&
+        (s.vps = pair_views(es, 32, ss.Rw, s.WD)) == 2)
+        return true;
+    s.zp = 16;
+    return ss.Rw2 <= 256 && (s.vps = pair_views(es, 16, ss.Rw2, s.WD)) > 0;
 }
 
-// The mirrored-pair kernel serves launches over the whole detector and the
-// slice pairs p0 .. p1 - 1 (slices p and N - 1 - p).
+// The staged kernel over the slices of b (mirror: over the whole detector and
+// the slice pairs p0 .. p1 - 1, i.e. slices p and N - 1 - p, of the whole
+// volume, with the shape s of the whole launch).
 cudaError_t try_launch_pair(const PlanImpl &p, const SquareSet &ss, bool direct, const void *src, float *vol,
-                            cudaStream_t st, int p0, int p1, bool &launched) {
+                            cudaStream_t st, const PairShape &s, const Band &b, int p0, int p1, bool &launched) {
     launched = false;
     const int es = (direct && p.qtype != FDKOD_F32) ? 2 : 4;
-    const int WD = es == 4 ? ss.WdT : ss.WdT16;
-    if (((uintptr_t)src & 15) != 0) return cudaSuccess;
-    if (direct && ((size_t)p.g.Nu * es) % 16 != 0) return cudaSuccess;
-    int vps = 0;
-    const int zp = pair_slices_per_cta(p, ss, direct, vps);
-    if (zp == 0) return cudaSuccess;  // windows too large: the 32-slice kernel
-    const int rows = zp == 32 ? ss.Rw : ss.Rw2;
-    uint64_t dims[3], strides[2];
-    if (direct) {
-        dims[0] = (uint64_t)p.g.Nu;
-        dims[1] = (uint64_t)p.g.Nv;
-        dims[2] = (uint64_t)p.g.P;
-        strides[0] = (uint64_t)p.g.Nu * es;
-    } else {
-        dims[0] = (uint64_t)p.Tstride;
-        dims[1] = (uint64_t)p.g.Nv;
-        dims[2] = (uint64_t)ss.nsq * p.Pd;
-        strides[0] = (uint64_t)p.Tstride * sizeof(float);
-    }
-    strides[1] = strides[0] * dims[1];
-    const uint32_t box[3] = {(uint32_t)WD, (uint32_t)rows, 1u};
-    const CUtensorMapDataType dt = es == 4 ? CU_TENSOR_MAP_DATA_TYPE_FLOAT32
-                                   : (p.qtype == FDKOD_F16 ? CU_TENSOR_MAP_DATA_TYPE_FLOAT16
-                                                           : CU_TENSOR_MAP_DATA_TYPE_BFLOAT16);
+    const int rows = s.zp == 32 ? ss.Rw : ss.Rw2;
     CUtensorMap map;
-    if (encode_map_3d(&map, dt, src, dims, strides, box) != cudaSuccess) return cudaSuccess;
+    if (!source_map(p, ss, direct, src, b.nrows, s.WD, rows, map)) return cudaSuccess;
     BpPairParams a{};
     a.vol = vol;
     a.geo = ss.geo;
@@ -1349,9 +644,11 @@ cudaError_t try_launch_pair(const PlanImpl &p, const SquareSet &ss, bool direct,
     a.tps = ss.tiles_per_side;
     a.Pd = p.Pd;
     a.RW = rows;
-    a.tile_stride = pair_tile_stride(es, rows, WD);
+    a.tile_stride = pair_tile_stride(es, rows, s.WD);
     a.pbase = p0;
     a.pend = p1;
+    a.zoff = b.zoff;
+    a.row0 = b.row0;
     a.wait_ns = p.wait_ns > 0 ? (unsigned long long)p.wait_ns : kWaitLimitNs;
     a.fault = p.test_fault;
     if (direct) {
@@ -1364,26 +661,25 @@ cudaError_t try_launch_pair(const PlanImpl &p, const SquareSet &ss, bool direct,
         a.scale = (float)(M_PI / (double)p.Pd);
     }
     launched = true;
-    if (!direct) return launch_pair_w<float, false>(WD, zp, vps, map, a, ss.nsq, st);
-    switch (p.qtype) {
-        case FDKOD_F32: return launch_pair_w<float, true>(WD, zp, vps, map, a, ss.nsq, st);
-        case FDKOD_BF16: return launch_pair_w<__nv_bfloat16, true>(WD, zp, vps, map, a, ss.nsq, st);
-        case FDKOD_F16: return launch_pair_w<__half, true>(WD, zp, vps, map, a, ss.nsq, st);
-    }
-    return cudaErrorInvalidValue;
+    if (!direct || p.qtype == FDKOD_F32) return launch_pair_f32(direct, s, map, a, ss.nsq, st);
+    return p.qtype == FDKOD_BF16 ? launch_pair_bf16(s, map, a, ss.nsq, st) : launch_pair_f16(s, map, a, ss.nsq, st);
 }
 
 }  // namespace
 
 cudaError_t launch_backproject_pairs(const PlanImpl &p, const SquareSet &ss, bool direct, const void *src,
                                      float *vol, cudaStream_t st, int p0, int p1, bool &launched) {
-    return try_launch_pair(p, ss, direct, src, vol, st, p0, p1, launched);
+    launched = false;
+    PairShape s;
+    if (!pair_shape(p, ss, direct, true, (p.g.N + 1) / 2, s)) return cudaSuccess;
+    Band whole;
+    whole.nrows = p.g.Nv;
+    return try_launch_pair(p, ss, direct, src, vol, st, s, whole, p0, p1, launched);
 }
 
 int pair_slab(const PlanImpl &p, const SquareSet &ss, bool direct) {
-    int vps = 0;
-    const int zp = pair_slices_per_cta(p, ss, direct, vps);
-    return zp > 0 ? zp : 16;
+    PairShape s;
+    return pair_shape(p, ss, direct, true, (p.g.N + 1) / 2, s) ? s.zp : 16;
 }
 
 cudaError_t launch_backproject(const PlanImpl &p, const SquareSet &ss, bool direct, const void *src, float *vol,
@@ -1392,12 +688,13 @@ cudaError_t launch_backproject(const PlanImpl &p, const SquareSet &ss, bool dire
     if (b.nrows < 0) b.nrows = p.g.Nv;
     if (b.nz < 0) b.nz = p.g.N;
     bool launched = false;
-    if (whole) {
-        cudaError_t pe = try_launch_pair(p, ss, direct, src, vol, st, 0, (p.g.N + 1) / 2, launched);
-        if (launched || pe != cudaSuccess) return pe;
-    }
-    cudaError_t te = try_launch_tma(p, ss, direct, src, vol, st, b, launched);
-    if (launched || te != cudaSuccess) return te;
+    PairShape s;
+    cudaError_t pe = cudaSuccess;
+    if (whole)
+        pe = launch_backproject_pairs(p, ss, direct, src, vol, st, 0, (p.g.N + 1) / 2, launched);
+    else if (pair_shape(p, ss, direct, false, (b.nz + 1) / 2, s))
+        pe = try_launch_pair(p, ss, direct, src, vol, st, s, b, b.zoff, b.zoff + b.nz, launched);
+    if (launched || pe != cudaSuccess) return pe;
     BpParams a{};
     a.src = src;
     a.vol = vol;

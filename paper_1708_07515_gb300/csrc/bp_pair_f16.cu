@@ -1,0 +1,11 @@
+// bp_pair_kernel on Q stored as float16.
+#include "bp_pair.cuh"
+
+namespace fdkod {
+
+cudaError_t launch_pair_f16(const PairShape &s, const CUtensorMap &map, const BpPairParams &prm, int nsq,
+                             cudaStream_t st) {
+    return launch_pair<__half, true>(s, map, prm, nsq, st);
+}
+
+}  // namespace fdkod

@@ -71,3 +71,29 @@ def test_many_tiles_sampled_slices(fd, oracle_mod, qtype, ratio):
         assert plan.device_status() == 0
     _cmp(got, oracle_mod.fdkod_slices(Qr, R, N, s, D, zs), f"FDK-OD {qtype} R={ratio}N")
     _cmp(plain, oracle_mod.fdk_slices(Qr, R, N, zs), f"plain FDK {qtype} R={ratio}N")
+
+
+@pytest.mark.parametrize("ratio", [4.0, 1.6, 1.2])
+@pytest.mark.parametrize("N,s,D,z0,nz", [
+    (245, 2, 2, 30, 192),   # 32 slices per slab and thread
+    (245, 2, 1, 228, 17),   # the volume's last slices, a second slab wholly past the end
+    (61, 1, 3, 0, 33),      # one slice past a CTA's slabs
+    (61, 1, 1, 20, 1),
+])
+def test_slabs_equal_the_whole_volume(fd, N, s, D, z0, nz, ratio):
+    """Slabs (two slabs per CTA, not mirrored) from just the detector rows
+    they read, against the whole volume's mirrored pairs: float32 rounding of
+    the same sums (rel-RMSE 1e-5, as slabs against whole volumes elsewhere)."""
+    P, Nv = 24, N + 2
+    Nu = N + (-N) % 4
+    Q = torch.from_numpy(_smooth_q(np.random.default_rng(N + nz), P, Nv, Nu)).cuda()
+    with fd.Plan(ratio * N, N, Nu, Nv, P, s, D) as plan:
+        whole = plan.backproject(Q)
+        v0, nr = plan.slab_rows(z0, nz)
+        rows = Q[:, v0:v0 + nr].contiguous()
+        work = torch.empty(max(1, plan.slab_workspace_elems(nr)), device="cuda")
+        slab = plan.backproject_slab(rows, v0, work, z0, nz)
+        assert plan.device_status() == 0
+    want = whole[z0:z0 + nz]
+    err = (slab.double() - want.double()).norm() / want.double().norm()
+    assert float(err) <= 1e-5, float(err)
