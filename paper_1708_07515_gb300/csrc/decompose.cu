@@ -89,7 +89,7 @@ decompose_kernel(const TQ *__restrict__ Q, float *__restrict__ Sp, const int32_t
 
 
 // ---------------------------------------------------------------------------
-// TMA path: one CTA per (square q, band of detector rows, range of decimated
+// Staged path: one CTA per (square q, band of detector rows, range of decimated
 // views), warp specialised.  The producer warp's lane 0 brings each view's
 // crop box (the band's rows x Wc columns from the 16-byte aligned column
 // below crop[q][k]) into a ring of slots of kG views with 3D bulk-tensor copies
@@ -112,6 +112,14 @@ decompose_kernel(const TQ *__restrict__ Q, float *__restrict__ Sp, const int32_t
 // two scalar loads per sample, and columns in steps of 32 lanes (128 computed
 // for ~100 used).
 //
+// Where TMA cannot describe a float32 Q (its rows are not whole 16-byte units,
+// or it is not 16-byte aligned: odd detector widths), kLoaders warps copy the
+// crops with 4-byte asynchronous copies, starting at the crop's own column
+// (offset 0), into the same ring; the consumers are the same.  Bound by those
+// copies: 501^3 x 720 views 3.8 ms (windowed sinc 4.6 with 8 loader warps, 6.3
+// with 4) against 5.8 (6.0) with one thread per output, which 16-bit Q keeps
+// (staged by plain 2-byte loads it took 15 ms against 5.6).
+//
 // Everything else a view needs -- shift fraction, tap weights, crop offset --
 // is one 16-byte entry of a per-CTA table in stream order (H = 2: 8 more bytes
 // of weights), built once.  Views go block by block (D views): a block's end
@@ -127,6 +135,8 @@ template <typename TQ>
 struct Ring {
     static constexpr int kG = sizeof(TQ) == 4 ? 1 : 2, kStages = sizeof(TQ) == 4 ? 3 : 2;
 };
+template <int H>
+constexpr int kLoaders = H == 1 ? 4 : 8;  // loader warps of the form without TMA
 constexpr int kRingSlack = 128;  // the last segment's loads run up to 16 bytes past a row's end
 constexpr uint64_t kDecWaitNs = 2000000000ull;
 
@@ -245,18 +255,29 @@ __host__ __device__ inline size_t dec_smem(int es, int stages, int tile_stride, 
            (size_t)nstream * (16 + (H == 2 ? 8 : 0) + 4);
 }
 
+// 4-byte asynchronous copy global -> shared (zero where !in), and the arrival
+// of this thread's earlier ones on `bar`
+__device__ __forceinline__ void cp_async4(uint32_t dst, const float *src, bool in) {
+    asm volatile("cp.async.ca.shared.global [%0], [%1], 4, %2;" ::"r"(dst), "l"(src), "r"(in ? 4u : 0u) : "memory");
+}
+__device__ __forceinline__ void cp_async_arrive(uint64_t *bar) {
+    asm volatile("cp.async.mbarrier.arrive.noinc.shared::cta.b64 [%0];" ::"r"(tma::smem_u32(bar)) : "memory");
+}
+
 // the thread bound only sets the register limit: 80 (24 warps per SM) for the
 // two running sums of the triangle, 128 (16 warps) for the four of 2D-tap filters
-template <typename TQ, int H>
+template <typename TQ, int H, bool TMA>
 __global__ void __launch_bounds__(H == 1 ? 768 : 512, 1)
-decompose_rows_kernel(const __grid_constant__ CUtensorMap tmap, float *__restrict__ Sp,
+decompose_rows_kernel(const __grid_constant__ CUtensorMap tmap, const TQ *__restrict__ Q, float *__restrict__ Sp,
                       const int32_t *__restrict__ crop, const GeomEntry *__restrict__ geo,
                       const int32_t *__restrict__ Tq, const float4 *__restrict__ tapw, int *status, int Tstride,
                       int P, int D, int Pd, int Nv, int Wc, int tile_stride, int segs, int chunks, int rowoff, int rowend,
-                      int jrange) {
+                      int jrange, int Nu) {
+    static_assert(TMA || sizeof(TQ) == 4, "plain copies: float32 only");
     constexpr int ES = (int)sizeof(TQ);
-    constexpr int kAlign = 16 / ES;
+    constexpr int kAlign = TMA ? 16 / ES : 1;
     constexpr int kG = Ring<TQ>::kG, kStages = Ring<TQ>::kStages;
+    constexpr int kProducers = TMA ? 1 : kLoaders<H>;
     extern __shared__ __align__(128) unsigned char smem_raw[];
     unsigned char *ring = smem_raw + ((128u - (tma::smem_u32(smem_raw) & 127u)) & 127u);
     const uint32_t tile_bytes = (uint32_t)(ES * tile_stride);
@@ -264,7 +285,7 @@ decompose_rows_kernel(const __grid_constant__ CUtensorMap tmap, float *__restric
     // views streamed: k' = j0 D - (H D - 1) .. (j1 - 1) D + H D - 1 (view k' mod P)
     const int nstream = (j1 - j0) * D + (2 * H - 1) * D - 1;
     const int nstage = (nstream + kG - 1) / kG;
-    const int warps = (int)(blockDim.x >> 5) - 1;  // consumer warps
+    const int warps = (int)(blockDim.x >> 5) - kProducers;  // consumer warps
     float *tbuf = (float *)(ring + (size_t)tile_bytes * kStages * kG + kRingSlack);
     float4 *s_v = (float4 *)(tbuf + (size_t)warps * 32 * kTP);
     float2 *s_w2 = (float2 *)(s_v + nstream);
@@ -280,14 +301,52 @@ decompose_rows_kernel(const __grid_constant__ CUtensorMap tmap, float *__restric
     build_stream_table<kAlign, H>(s_v, s_w2, s_c, crop, geo, tapw, q, P, D, j0, nstream);
     if (threadIdx.x == 0) {
         for (int i = 0; i < kStages; ++i) {
-            tma::mbar_init(&full[i], 1);
+            tma::mbar_init(&full[i], TMA ? 1 : 32 * kProducers);
             tma::mbar_init(&empty[i], warps);
         }
         tma::fence_mbar_init();
     }
     __syncthreads();
 
-    if (warp == warps) {  // producer
+    if constexpr (!TMA) {
+        if (warp >= warps) {  // loader: rows lw, lw + kProducers, ... of the band
+            const int lw = warp - warps;
+            int kk = ((j0 * D - (H * D - 1)) % P + P) % P, slot = 0;
+            uint32_t phase = 0;
+            for (int n = 0; n < nstream; ++n) {
+                static_assert(TMA || kG == 1, "one view per slot");
+                if (n >= kStages && !tma::mbar_wait_bounded(&empty[slot], phase ^ 1u, kDecWaitNs)) {
+                    if (lane == 0) atomicOr(status, 2);
+                    asm volatile("cp.async.wait_all;" ::: "memory");
+                    return;
+                }
+                const int c0 = s_c[n] + tc;
+                const float *src = Q + (ptrdiff_t)kk * Nv * Nu + c0 + lane;
+                const uint32_t dst = tma::smem_u32(ring + (size_t)tile_bytes * slot) + 4u * (uint32_t)lane;
+                constexpr int kCols = (kDecMaxSegs * kCW + 4 + 31) / 32;  // 32-column steps of the widest box
+#pragma unroll 4
+                for (int r = lw; r < band; r += kProducers) {
+                    const int v = v0 + r;
+                    const float *row = src + (ptrdiff_t)v * Nu;
+#pragma unroll
+                    for (int i = 0; i < kCols; ++i) {
+                        const int c = 32 * i + lane;
+                        const bool in = v < Nv && c0 + c >= 0 && c0 + c < Nu;  // else zeros
+                        if (c < Wc) cp_async4(dst + 4u * (uint32_t)(r * Wc + 32 * i), in ? row + 32 * i : Q, in);
+                    }
+                }
+                cp_async_arrive(&full[slot]);  // once this lane's copies have landed
+                if (++kk == P) kk = 0;
+                if (++slot == kStages) {
+                    slot = 0;
+                    phase ^= 1u;
+                }
+            }
+            // copies still in flight must land before the CTA may exit
+            asm volatile("cp.async.wait_all;" ::: "memory");
+            return;
+        }
+    } else if (warp == warps) {  // producer
         if (lane != 0) return;
         int kk = ((j0 * D - (H * D - 1)) % P + P) % P, n = 0, slot = 0;
         uint32_t phase = 0;  // parity of the slot's current round
@@ -358,7 +417,8 @@ decompose_rows_kernel(const __grid_constant__ CUtensorMap tmap, float *__restric
                 wt[2] = e2.x;
                 wt[3] = e2.y;
             }
-            view_any<TQ, H>(__float_as_int(e.y), a, e.x, wt, acc);
+            if constexpr (TMA) view_any<TQ, H>(__float_as_int(e.y), a, e.x, wt, acc);
+            else view_step<TQ, H, 0>(a, e.x, wt, acc);
             a += tile_bytes;
             if (++w == kG) {
                 w = 0;
@@ -401,19 +461,19 @@ struct Rows {
     int layout, rowoff, rowend;
 };
 
-// TMA applies when Q's rows are whole 16-byte units, Q and S' are 16-byte
-// aligned (vector stores), D <= 128 and the ring plus the stream tables fit
-// in shared memory.
-template <typename TQ, int H>
+// Applies when S' is 16-byte aligned (vector stores), D <= 128 and the ring
+// plus the stream tables fit in shared memory; TMA: when Q is 16-byte aligned
+// and its rows are whole 16-byte units.
+template <typename TQ, int H, bool TMA>
 cudaError_t try_rows(const PlanImpl &p, const TQ *Q, float *out, cudaStream_t st, Rows rw, bool &launched) {
     launched = false;
     constexpr int kAlign = 16 / (int)sizeof(TQ);
-    if ((p.g.Nu % kAlign) != 0 || ((uintptr_t)Q & 15) != 0 || ((uintptr_t)out & 15) != 0) return cudaSuccess;
-    if (p.D > kMaxTapD) return cudaSuccess;
+    if (TMA && ((p.g.Nu % kAlign) != 0 || ((uintptr_t)Q & 15) != 0)) return cudaSuccess;
+    if (((uintptr_t)out & 15) != 0 || p.D > kMaxTapD) return cudaSuccess;
     const int all = (p.Tstride + kCW - 1) / kCW;  // column segments of a square
     const int chunks = (all + kDecMaxSegs - 1) / kDecMaxSegs, segs = (all + chunks - 1) / chunks;
     // the segments' columns + neighbour + crop offset, whole 16-byte units, an odd number of them
-    int Wc = (std::min(p.od.Tmax, segs * kCW) + 1 + (kAlign - 1) + (kAlign - 1)) & ~(kAlign - 1);
+    int Wc = (std::min(p.od.Tmax, segs * kCW) + 1 + (TMA ? kAlign - 1 : 0) + (kAlign - 1)) & ~(kAlign - 1);
     if ((Wc / kAlign) % 2 == 0) Wc += kAlign;
     const int nrows = rw.rowend - rw.rowoff;
     // narrow squares: several row groups per CTA, at least four consumer warps
@@ -448,30 +508,40 @@ cudaError_t try_rows(const PlanImpl &p, const TQ *Q, float *out, cudaStream_t st
     }
     const size_t smem = smem_of(jrange);
     if (smem > 200 * 1024 || bands > 65535) return cudaSuccess;
-    CUtensorMap map;
-    const uint64_t dims[3] = {(uint64_t)p.g.Nu, (uint64_t)rw.layout, (uint64_t)p.g.P};
-    const uint64_t strides[2] = {(uint64_t)p.g.Nu * sizeof(TQ), (uint64_t)p.g.Nu * rw.layout * sizeof(TQ)};
-    const uint32_t box[3] = {(uint32_t)Wc, (uint32_t)band, 1u};
-    const CUtensorMapDataType dt = sizeof(TQ) == 4 ? CU_TENSOR_MAP_DATA_TYPE_FLOAT32
-                                   : (std::is_same<TQ, __half>::value ? CU_TENSOR_MAP_DATA_TYPE_FLOAT16
-                                                                      : CU_TENSOR_MAP_DATA_TYPE_BFLOAT16);
-    if (encode_map_3d(&map, dt, Q, dims, strides, box) != cudaSuccess) return cudaSuccess;
+    CUtensorMap map{};
+    if constexpr (TMA) {
+        const uint64_t dims[3] = {(uint64_t)p.g.Nu, (uint64_t)rw.layout, (uint64_t)p.g.P};
+        const uint64_t strides[2] = {(uint64_t)p.g.Nu * sizeof(TQ), (uint64_t)p.g.Nu * rw.layout * sizeof(TQ)};
+        const uint32_t box[3] = {(uint32_t)Wc, (uint32_t)band, 1u};
+        const CUtensorMapDataType dt = sizeof(TQ) == 4 ? CU_TENSOR_MAP_DATA_TYPE_FLOAT32
+                                       : (std::is_same<TQ, __half>::value ? CU_TENSOR_MAP_DATA_TYPE_FLOAT16
+                                                                          : CU_TENSOR_MAP_DATA_TYPE_BFLOAT16);
+        if (encode_map_3d(&map, dt, Q, dims, strides, box) != cudaSuccess) return cudaSuccess;
+    }
     launched = true;
-    cudaError_t e = ensure_smem<decompose_rows_kernel<TQ, H>>(smem);
+    cudaError_t e = ensure_smem<decompose_rows_kernel<TQ, H, TMA>>(smem);
     if (e != cudaSuccess) return e;
     dim3 grid(p.od.nsq * chunks, bands, (p.Pd + jrange - 1) / jrange);
-    decompose_rows_kernel<TQ, H><<<grid, 32 * (warps + 1), smem, st>>>(
-        map, out, p.od.crop, p.od.geo, p.od.T, p.tapw, p.status, p.Tstride, p.g.P, p.D, p.Pd, rw.layout, Wc,
-        tile_stride, segs, chunks, rw.rowoff, rw.rowend, jrange);
+    decompose_rows_kernel<TQ, H, TMA><<<grid, 32 * (warps + (TMA ? 1 : kLoaders<H>)), smem, st>>>(
+        map, Q, out, p.od.crop, p.od.geo, p.od.T, p.tapw, p.status, p.Tstride, p.g.P, p.D, p.Pd, rw.layout, Wc,
+        tile_stride, segs, chunks, rw.rowoff, rw.rowend, jrange, p.g.Nu);
     return cudaGetLastError();
+}
+
+template <typename TQ, int H>
+cudaError_t try_staged(const PlanImpl &p, const TQ *Q, float *out, cudaStream_t st, Rows rw, bool &launched) {
+    cudaError_t e = try_rows<TQ, H, true>(p, Q, out, st, rw, launched);
+    if constexpr (sizeof(TQ) == 4)
+        if (!launched && e == cudaSuccess) e = try_rows<TQ, H, false>(p, Q, out, st, rw, launched);
+    return e;
 }
 
 template <typename TQ>
 cudaError_t launch_t(const PlanImpl &p, const TQ *Q, float *out, cudaStream_t st, Rows rw) {
     if (p.tap_blocks != 1 && p.tap_blocks != 2) return cudaErrorInvalidValue;
     bool launched = false;
-    cudaError_t te = p.tap_blocks == 2 ? try_rows<TQ, 2>(p, Q, out, st, rw, launched)
-                                       : try_rows<TQ, 1>(p, Q, out, st, rw, launched);
+    cudaError_t te = p.tap_blocks == 2 ? try_staged<TQ, 2>(p, Q, out, st, rw, launched)
+                                       : try_staged<TQ, 1>(p, Q, out, st, rw, launched);
     if (launched || te != cudaSuccess) return te;
     dim3 grid((p.Tstride + kTX - 1) / kTX, (rw.rowend - rw.rowoff + kTY - 1) / kTY, p.od.nsq);
     if (p.tap_blocks == 2)

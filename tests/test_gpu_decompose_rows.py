@@ -1,9 +1,11 @@
 """The staged decomposition (lane = detector row, 16 columns per warp) against
 the generic kernel, bit for bit.
 
-Both add the same products in the same order, so on the same Q they must
-agree exactly; the generic kernel runs when Q is not 16-byte aligned, and is
-itself checked against the FP64 oracle here.  Shapes: squares whose shifted
+All forms add the same products in the same order, so on the same Q they must
+agree exactly.  The staged kernel takes its crops by TMA, or (float32) by
+4-byte copies where Q is not 16-byte aligned or its rows are not whole 16-byte
+units; the generic kernel runs when the output is not 16-byte aligned, and is itself
+checked against the FP64 oracle here.  Shapes: squares whose shifted
 rows end on and beside a multiple of 16 columns, one to eight column segments,
 squares wider than 128 columns (several CTAs side by side), detectors of 1,
 31, 32, 33 and more rows, few and many views (ranges of decimated views), both
@@ -26,16 +28,19 @@ def fd():
     return fd
 
 
-def _both(fd, plan, Q):
-    """(staged, generic) decomposed data of the same Q."""
-    n = Q.numel()
-    buf = torch.empty(n + 1, dtype=Q.dtype, device="cuda")
-    off = buf[1:].view(Q.shape)          # one element past an aligned address
-    off.copy_(Q)
-    a = plan.decompose(Q)
-    b = plan.decompose(off)
+def _past_aligned(shape, dtype):
+    """A contiguous tensor one element past an aligned address."""
+    n = int(np.prod(shape))
+    return torch.empty(n + 1, dtype=dtype, device="cuda")[1:].view(shape)
+
+
+def _forms(plan, Q):
+    """Decomposed data of the same Q: staged, staged from a misaligned Q, generic."""
+    off = _past_aligned(Q.shape, Q.dtype).copy_(Q)
+    a, b = plan.decompose(Q), plan.decompose(off)
+    c = plan.decompose(Q, _past_aligned(plan.decomposed_shape, torch.float32))
     assert plan.device_status() == 0
-    return a, b
+    return a, b, c
 
 
 @pytest.mark.parametrize("qtype", ["f32", "bf16", "f16"])
@@ -49,21 +54,24 @@ def _both(fd, plan, Q):
     (250, 256, 35, 40, 0, 4, 3.0),   # three CTAs side by side
     (200, 200, 64, 400, 1, 2, 4.0),  # ranges of decimated views
     (61, 64, 70, 900, 3, 2, 1.6),    # many views, ragged squares, a near source
+    (61, 63, 45, 60, 1, 3, 2.5),     # odd detector: 4-byte copies
+    (150, 149, 40, 48, 0, 2, 4.0),   # and wider than 128 columns
 ])
 def test_staged_equals_generic(fd, qtype, taps, N, Nu, Nv, P, s, D, r):
     Q = torch.from_numpy(np.random.default_rng(N + P).standard_normal((P, Nv, Nu)).astype(np.float32))
     Q = Q.to(_TYPES[qtype]).cuda()
     with fd.Plan(r * N, N, Nu, Nv, P, s, D, qtype=qtype, taps=taps) as plan:
-        a, b = _both(fd, plan, Q)
-        assert torch.equal(a, b), (plan.info["T_stride"], float((a - b).abs().max()))
+        a, b, c = _forms(plan, Q)
+        assert torch.equal(a, c), (plan.info["T_stride"], float((a - c).abs().max()))
+        assert torch.equal(b, c), (plan.info["T_stride"], float((b - c).abs().max()))
 
 
 def test_generic_against_the_oracle(fd, oracle_mod):
     N, P, s, D = 40, 36, 1, 3
     Q = np.random.default_rng(5).standard_normal((P, 31, 40)).astype(np.float32)
     with fd.Plan(4.0 * N, N, 40, 31, P, s, D) as plan:
-        _, b = _both(fd, plan, torch.from_numpy(Q).cuda())
-        got, T = b.cpu().numpy(), plan.bounds()["T"]
+        c = _forms(plan, torch.from_numpy(Q).cuda())[2]
+        got, T = c.cpu().numpy(), plan.bounds()["T"]
     for q in range(4):
         want = oracle_mod.shift_decimate(Q, 4.0 * N, N, s, D, q)
         assert np.abs(got[q, :, :, :T[q]] - want).max() <= 1e-6 * np.abs(Q).max()
