@@ -608,6 +608,7 @@ bool pair_shape(const PlanImpl &p, const SquareSet &ss, bool direct, bool mirror
     const int es = (direct && p.qtype != FDKOD_F32) ? 2 : 4;
     s.WD = es == 4 ? ss.WdT : ss.WdT16;
     s.mirror = mirror;
+    s.nsplit = 1;
     if (s.WD == 0) return false;
     const long long tiles = (long long)ss.nsq * ss.tiles_per_side * ss.tiles_per_side;
     int dev = 0, sms = 148;
@@ -618,6 +619,21 @@ bool pair_shape(const PlanImpl &p, const SquareSet &ss, bool direct, bool mirror
         (s.vps = pair_views(es, 32, ss.Rw, s.WD)) == 2)
         return true;
     s.zp = 16;
+    // Clusters share the views where the tiles leave SMs idle: as many CTAs as
+    // fit the GPU at once, at least 5 views each (64^3 x 45 views, 32 CTAs: 36.4
+    // us alone, 16.8 in clusters of 8; 96^3 x 67, 108 CTAs: 51.7, 37.3 in 4,
+    // 44.9 in 8).  Up to two waves, smaller pieces still fill the last wave
+    // better where they are long enough (128^3 x 64, 256 CTAs: 74.3, 69.4 in 4;
+    // x 179: 196, 167; 160^3 x 55, 500 CTAs: 115, 109 in 2), but not beyond
+    // (192^3 x 67, 864 CTAs: 203, 211 in 2).
+    if (mirror) {
+        const int views = direct ? p.g.P : p.Pd;
+        const long long ctas = tiles * n16, slots = (long long)pair_ctas(16) * sms;
+        for (int n = 8; n >= 2 && s.nsplit == 1; n /= 2)
+            if (ctas * n <= slots && views >= 5 * n) s.nsplit = n;
+        if (s.nsplit == 1 && ctas * 4 <= 3 * slots && views >= 64) s.nsplit = 4;
+        if (s.nsplit == 1 && ctas * 4 <= 5 * slots && views >= 32) s.nsplit = 2;
+    }
     return ss.Rw2 <= 256 && (s.vps = pair_views(es, 16, ss.Rw2, s.WD)) > 0;
 }
 
@@ -649,6 +665,7 @@ cudaError_t try_launch_pair(const PlanImpl &p, const SquareSet &ss, bool direct,
     a.pend = p1;
     a.zoff = b.zoff;
     a.row0 = b.row0;
+    a.nsplit = s.nsplit;
     a.wait_ns = p.wait_ns > 0 ? (unsigned long long)p.wait_ns : kWaitLimitNs;
     a.fault = p.test_fault;
     if (direct) {

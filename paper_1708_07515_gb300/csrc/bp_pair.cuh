@@ -6,6 +6,8 @@
 #include <cuda_bf16.h>
 #include <cuda_fp16.h>
 
+#include <algorithm>
+
 #include "fdkod_internal.cuh"
 #include "tma.cuh"
 
@@ -60,15 +62,16 @@ struct BpPairParams {
     // otherwise slices pbase .. pend - 1, written to vol[z - zoff]
     int pbase, pend, zoff;
     int row0;             // detector row held in the source's row 0
+    int nsplit;           // SPLIT: CTAs of a cluster that share the views
     float scale;
     unsigned long long wait_ns;
     int fault;
 };
 
 // What a launch needs besides its parameters: the window width, slices per
-// slab and views per ring slot pick the instantiation.
+// slab, views per ring slot and CTAs per cluster pick the instantiation.
 struct PairShape {
-    int WD, zp, vps;
+    int WD, zp, vps, nsplit;
     bool mirror;
 };
 
@@ -120,6 +123,21 @@ __device__ __forceinline__ float rcp_approx(float x) {
     float y;
     asm("rcp.approx.ftz.f32 %0, %1;" : "=f"(y) : "f"(x));
     return y;
+}
+
+// barrier over all threads of the cluster, ordering their shared memory
+__device__ __forceinline__ void cluster_sync() {
+    asm volatile("barrier.cluster.arrive.release.aligned;\n\tbarrier.cluster.wait.acquire.aligned;" ::: "memory");
+}
+// two floats at this CTA's shared address a, of the cluster's CTA `rank`
+__device__ __forceinline__ float2 ld_cluster(uint32_t a, uint32_t rank) {
+    float2 v;
+    asm volatile("{\n\t.reg .u32 ra;\n\tmapa.shared::cluster.u32 ra, %2, %3;\n\t"
+                 "ld.shared::cluster.v2.f32 {%0, %1}, [ra];\n\t}"
+                 : "=f"(v.x), "=f"(v.y)
+                 : "r"(a), "r"(rank)
+                 : "memory");
+    return v;
 }
 
 // Column-interpolated samples (U^-2 weighted) of row r + K of the first slab's
@@ -250,7 +268,10 @@ constexpr int kPairThreads = kThreads + 32;        // plus the producer warp
 // CTAs per SM: registers decide (2 ZP accumulators per thread)
 constexpr int pair_ctas(int ZP) { return ZP == 32 ? 2 : 3; }
 
-template <typename TS, bool DIRECT, bool MIRROR, int WD, int ZP, int VPS>
+// SPLIT: the nsplit CTAs of a cluster (grid z) take a range of the views each
+// and add up their sums through distributed shared memory, CTA r every
+// nsplit-th slice from r on, in the order of the ranges (pair_shape says where).
+template <typename TS, bool DIRECT, bool MIRROR, int WD, int ZP, int VPS, bool SPLIT>
 __global__ void __launch_bounds__(kPairThreads, pair_ctas(ZP))
 bp_pair_kernel(const __grid_constant__ CUtensorMap tmap, BpPairParams a) {
     constexpr int ES = (int)sizeof(TS);
@@ -285,7 +306,10 @@ bp_pair_kernel(const __grid_constant__ CUtensorMap tmap, BpPairParams a) {
     const float zc2 = MIRROR ? -zc : (p0 + ZP < a.pend ? zc + (float)ZP : zc);
     const float vcd = 0.5f * (float)(a.Nv - 1);
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-    const int nch = (a.nviews + VPS - 1) / VPS;
+    // this CTA's views
+    const int j0 = SPLIT ? a.nviews * (int)blockIdx.z / a.nsplit : 0;
+    const int nviews = SPLIT ? a.nviews * ((int)blockIdx.z + 1) / a.nsplit - j0 : a.nviews;
+    const int nch = (nviews + VPS - 1) / VPS;
     // window of view w of slot sl, first (h = 0) or second (h = 1) slab
     auto win = [&](int sl, int w, int h) { return (uint32_t)((sl * VPS + w) * 2 + h) * (uint32_t)a.tile_stride; };
 
@@ -310,8 +334,8 @@ bp_pair_kernel(const __grid_constant__ CUtensorMap tmap, BpPairParams a) {
         int c = 0;
         for (; c < nch; ++c) {
             const int sl = c % kPairSlots;
-            const int nj = min(VPS, a.nviews - c * VPS);
-            const int j = c * VPS + min(w, nj - 1);  // lanes past the chunk repeat its last view
+            const int nj = min(VPS, nviews - c * VPS);
+            const int j = j0 + c * VPS + min(w, nj - 1);  // lanes past the chunk repeat its last view
             const int k = j * a.vstep;
             const size_t o = (size_t)q * a.P + k;
             const GeomEntry ge = a.geo[o];
@@ -396,7 +420,7 @@ bp_pair_kernel(const __grid_constant__ CUtensorMap tmap, BpPairParams a) {
                 tma::mbar_arrive_expect_tx(&full[sl], (uint32_t)(nj * 2 * a.RW * WD * ES));
                 for (int v2 = 0; v2 < nj; ++v2) {
                     // test hook: the slot's bytes never all arrive, its wait runs out
-                    if (a.fault == kTestFaultSkipCopy && c == 1 && v2 == 0 && blockIdx.x == 0 && blockIdx.y == 0)
+                    if (a.fault == kTestFaultSkipCopy && c == 1 && v2 == 0 && blockIdx.x + blockIdx.y + blockIdx.z == 0)
                         continue;
                     const int x = v2 == 0 ? xs0 : xs1, z = v2 == 0 ? tz0 : tz1;
                     // rows of the source (out of range: zero fill)
@@ -410,6 +434,11 @@ bp_pair_kernel(const __grid_constant__ CUtensorMap tmap, BpPairParams a) {
         if (lane == 0)
             for (int m = max(0, c - kPairSlots); m < c; ++m)
                 tma::mbar_wait_bounded(&full[m % kPairSlots], (uint32_t)((m / kPairSlots) & 1), a.wait_ns);
+        if constexpr (SPLIT) {
+            __syncwarp();
+            cluster_sync();
+            cluster_sync();
+        }
         return;
     }
 
@@ -426,13 +455,14 @@ bp_pair_kernel(const __grid_constant__ CUtensorMap tmap, BpPairParams a) {
 #pragma unroll
     for (int i = 0; i < ZP; ++i) acc[i] = make_float2(0.f, 0.f);
 
-    int sl = 0, left = a.nviews;
+    int sl = 0, left = nviews;
     uint32_t phase = 0;
     for (; left > 0; left -= VPS) {
         const bool ok = tma::mbar_wait_bounded(&full[sl], phase, a.wait_ns);
         if (!__all_sync(0xffffffffu, ok)) {
             if (lane == 0) atomicOr(a.status, 2);
-            return;  // the producer waits for the copies in flight
+            if constexpr (SPLIT) break;  // the cluster's barriers wait for this warp
+            return;                      // the producer waits for the copies in flight
         }
         const PairView *pv = s_view + sl * VPS, *pe = pv + min(VPS, left);
 #pragma unroll 1
@@ -475,6 +505,28 @@ bp_pair_kernel(const __grid_constant__ CUtensorMap tmap, BpPairParams a) {
             phase ^= 1u;
         }
     }
+    if constexpr (SPLIT) {
+        // every warp is done with the ring: it takes this CTA's sums [i][thread]
+        asm volatile("bar.sync 1, %0;" ::"n"(32 * kPairConsumers) : "memory");
+        float2 *part = (float2 *)sm + threadIdx.x;
+#pragma unroll
+        for (int i = 0; i < ZP; ++i) part[i * 32 * kPairConsumers] = acc[i];
+        cluster_sync();
+        for (int i = (int)blockIdx.z; i < ZP; i += a.nsplit) {
+            float2 sum = make_float2(0.f, 0.f);
+            for (int r = 0; r < a.nsplit; ++r)
+                sum = __fadd2_rn(sum, ld_cluster(tma::smem_u32(part + i * 32 * kPairConsumers), (uint32_t)r));
+            const int pz = p0 + i;
+            if (active && pz < a.pend) {
+                static_assert(!SPLIT || MIRROR, "whole volumes only");
+                const int zu = a.N - 1 - pz;
+                a.vol[((size_t)pz * a.N + y) * a.N + x] = sum.x * a.scale;
+                if (zu != pz) a.vol[((size_t)zu * a.N + y) * a.N + x] = sum.y * a.scale;
+            }
+        }
+        cluster_sync();  // the others may still be reading this CTA's sums
+        return;
+    }
     if (active) {
 #pragma unroll
         for (int i = 0; i < ZP; ++i) {
@@ -502,22 +554,40 @@ inline size_t pair_smem(int es, int vps, int tile_stride) {
     return (size_t)es * kPairSlots * vps * 2 * tile_stride + 2 * kPairPad + 128;
 }
 
-template <typename TS, bool DIRECT, bool MIRROR, int WD, int ZP, int VPS>
+template <typename TS, bool DIRECT, bool MIRROR, int WD, int ZP, int VPS, bool SPLIT = false>
 cudaError_t launch_pair_t(const CUtensorMap &map, const BpPairParams &prm, int nsq, cudaStream_t st) {
-    const size_t smem = pair_smem((int)sizeof(TS), VPS, prm.tile_stride);
-    cudaError_t e = ensure_smem<bp_pair_kernel<TS, DIRECT, MIRROR, WD, ZP, VPS>>(smem);
+    size_t smem = pair_smem((int)sizeof(TS), VPS, prm.tile_stride);
+    // SPLIT: the ring also holds the CTA's sums
+    if (SPLIT) smem = std::max(smem, sizeof(float2) * ZP * 32 * kPairConsumers + 2 * (size_t)kPairPad + 128);
+    cudaError_t e = ensure_smem<bp_pair_kernel<TS, DIRECT, MIRROR, WD, ZP, VPS, SPLIT>>(smem);
     if (e != cudaSuccess) return e;
     constexpr int kSlices = MIRROR ? ZP : 2 * ZP;
-    dim3 grid((unsigned)(nsq * prm.tps * prm.tps), (unsigned)((prm.pend - prm.pbase + kSlices - 1) / kSlices));
-    bp_pair_kernel<TS, DIRECT, MIRROR, WD, ZP, VPS><<<grid, kPairThreads, smem, st>>>(map, prm);
-    return cudaGetLastError();
+    cudaLaunchConfig_t cfg{};
+    cfg.gridDim = dim3((unsigned)(nsq * prm.tps * prm.tps), (unsigned)((prm.pend - prm.pbase + kSlices - 1) / kSlices),
+                       SPLIT ? (unsigned)prm.nsplit : 1u);
+    cfg.blockDim = dim3(kPairThreads);
+    cfg.dynamicSmemBytes = smem;
+    cfg.stream = st;
+    cudaLaunchAttribute at{};
+    at.id = cudaLaunchAttributeClusterDimension;
+    at.val.clusterDim.x = at.val.clusterDim.y = 1;
+    at.val.clusterDim.z = SPLIT ? (unsigned)prm.nsplit : 1u;
+    cfg.attrs = &at;
+    cfg.numAttrs = SPLIT ? 1 : 0;
+    return cudaLaunchKernelEx(&cfg, bp_pair_kernel<TS, DIRECT, MIRROR, WD, ZP, VPS, SPLIT>, map, prm);
 }
 
-// 32 slices per slab always come with 2 views per slot (pair_shape)
+// 32 slices per slab always come with 2 views per slot and no split, a split
+// with whole volumes (pair_shape)
 template <typename TS, bool DIRECT, bool MIRROR, int WD>
 cudaError_t launch_pair_z(const PairShape &s, const CUtensorMap &map, const BpPairParams &prm, int nsq,
                           cudaStream_t st) {
     if (s.zp == 32) return launch_pair_t<TS, DIRECT, MIRROR, WD, 32, 2>(map, prm, nsq, st);
+    if constexpr (MIRROR) {
+        if (s.nsplit > 1)
+            return s.vps == 2 ? launch_pair_t<TS, DIRECT, MIRROR, WD, 16, 2, true>(map, prm, nsq, st)
+                              : launch_pair_t<TS, DIRECT, MIRROR, WD, 16, 1, true>(map, prm, nsq, st);
+    }
     return s.vps == 2 ? launch_pair_t<TS, DIRECT, MIRROR, WD, 16, 2>(map, prm, nsq, st)
                       : launch_pair_t<TS, DIRECT, MIRROR, WD, 16, 1>(map, prm, nsq, st);
 }

@@ -52,6 +52,27 @@ def test_every_group_size(fd, oracle_mod, N, P, s, D, ratio):
     _cmp(got, oracle_mod.fdkod(Q, R, N, s, D), f"N={N} R={ratio}N")
 
 
+@pytest.mark.parametrize("N,P,s,D,qtype", [
+    (16, 10, 0, 1, "f32"),     # clusters of 2 (5 views each)
+    (33, 43, 1, 1, "bf16"),    # of 8, uneven ranges of views
+    (96, 90, 1, 2, "f32"),     # of 4
+    (130, 128, 1, 2, "f32"),   # of 4 in two waves, ragged tiles
+    (131, 66, 0, 2, "f32"),    # of 2
+    (64, 45, 1, 1, "f16"),
+])
+def test_views_shared_by_a_cluster(fd, oracle_mod, N, P, s, D, qtype):
+    R = 3.0 * N
+    Q = _smooth_q(np.random.default_rng(P), P, N, N + (-N) % 8)
+    t = {"f32": torch.float32, "bf16": torch.bfloat16, "f16": torch.float16}[qtype]
+    Qd = torch.from_numpy(Q).to(t).cuda()
+    with fd.Plan(R, N, Q.shape[2], N, P, s, D, qtype=qtype) as plan:
+        got = plan.backproject(Qd)
+        again = plan.backproject(Qd)
+        assert plan.device_status() == 0
+    assert torch.equal(got, again)   # the ranges are added in a fixed order
+    _cmp(got.cpu().numpy(), oracle_mod.fdkod(Qd.float().cpu().numpy(), R, N, s, D), f"N={N} P={P}")
+
+
 @pytest.mark.parametrize("ratio", [4.0, 1.6])
 @pytest.mark.parametrize("qtype", ["f32", "f16"])
 def test_many_tiles_sampled_slices(fd, oracle_mod, qtype, ratio):
