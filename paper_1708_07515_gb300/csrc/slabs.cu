@@ -194,8 +194,8 @@ extern "C" int fdkod_reconstruct_slabs(fdkod_plan_t *plan, const float *proj_hos
 //     overlaps the next group's backprojection.
 namespace fdkod {
 
-// Row bands of the upload, outside in: two thin outer bands of Nv/8 rows
-// (the outermost slice pairs read only those, so their backprojection can
+// Row bands of the upload, outside in: two thin outer bands of Nv/8 rows or a
+// little more (the outermost slice pairs read only those, so their backprojection can
 // start early), then bands of Nv/4 rows.  The strided copy of a band (one
 // segment per view) keeps near the contiguous copy rate down to about
 // 256 KiB segments (measured: 211 GB/s for two bands of 512^2 x 720
@@ -379,6 +379,10 @@ extern "C" int fdkod_reconstruct(fdkod_plan_t *plan, const float *proj_host, flo
     // whole-detector launch does); an odd Nv, or a learned decimation (its
     // kernel takes every row at once), makes one band.
     const bool banded = (Nv % 2) == 0 && !p.net;
+    // slice pairs per backprojection group: a multiple of what a CTA takes
+    const bool direct = p.D == 1;
+    const int npair = (N + 1) / 2, slab = fdkod::pair_slab(p, p.od, direct);
+    const int group = ((npair + kPipeSlabs - 1) / kPipeSlabs + slab - 1) / slab * slab;
     // band i covers rows bv[i] .. bv[i + 1] - 1 (even bounds); upload order:
     // the two outer bands, then inwards, alternating bottom and top
     int bv[kPipeChunks + 1], nbands = 0;
@@ -387,7 +391,15 @@ extern "C" int fdkod_reconstruct(fdkod_plan_t *plan, const float *proj_host, flo
         bv[1] = Nv;
         nbands = 1;
     } else {
-        const int outer = std::max(2, (Nv / 8) & ~1), inner = std::max(2, (Nv / 4) & ~1);
+        // the outer bands hold what the first group of slice pairs reads, so
+        // that its backprojection starts while the others are on their way
+        // (512^3: 68 rows for 32 pairs; with 64 rows it waited for the second
+        // pair of bands: 12.99 against 12.20 ms a call)
+        int32_t first0 = 0, firstn = 0;
+        fdkod_slab_rows(plan, 0, std::min(group, N), &first0, &firstn);
+        const int need = first0 + firstn;
+        const int outer = std::max(2, (std::min(std::max(Nv / 8, need), Nv / 4) + 1) & ~1);
+        const int inner = std::max(2, (Nv / 4) & ~1);
         int lo = 0, hi = Nv, cuts_lo[kPipeChunks], cuts_hi[kPipeChunks], nl = 0, nh = 0;
         for (int step = outer; lo < hi; step = inner) {  // walk inwards from both ends
             if (nl + nh + 2 > kPipeChunks - 1 || hi - lo <= 2 * step) break;
@@ -452,16 +464,12 @@ extern "C" int fdkod_reconstruct(fdkod_plan_t *plan, const float *proj_host, flo
             if (bv[bi] < v0 + nr && bv[bi + 1] > v0) SLAB_TRY(cudaStreamWaitEvent(c, hp.ev_band[bi], 0));
         return FDKOD_OK;
     };
-    const bool direct = p.D == 1;
     const void *src = direct ? hp.Q : (const void *)p.Sp;
     // backprojection in groups of slice pairs (slices p and N - 1 - p, the
     // same tiles as one whole-volume launch), outermost first, alternating
     // between the two compute streams, each after the bands it reads; each
     // group's two z-ranges are read back as soon as it is done
-    const int npair = (N + 1) / 2;
-    int ps = (npair + kPipeSlabs - 1) / kPipeSlabs;
-    const int slab = fdkod::pair_slab(p, p.od, direct);
-    ps = (ps + slab - 1) / slab * slab;
+    const int ps = group;
     int ns = 0;
     bool paired = true;
     const size_t plane = (size_t)N * N;
