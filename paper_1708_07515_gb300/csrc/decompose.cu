@@ -128,12 +128,14 @@ decompose_kernel(const TQ *__restrict__ Q, float *__restrict__ Sp, const int32_t
 constexpr int kCW = 16;       // shifted columns per warp
 constexpr int kTP = kCW + 4;  // row pitch of the transpose buffer (floats; 5 16-byte units: no conflicts)
 constexpr int kDecMaxSegs = 8;  // column segments (consumer warps) per CTA; wider squares take several CTAs
-// ring shape per element type (measured at 512^3 f32 and 2000^3 bf16: slots of
-// one view 1.11 and 5.62 ms, of two views 1.40 and 5.37 ms; what counts most is
-// that three CTAs fit an SM)
-template <typename TQ>
+// ring shape per element type and tap length: slots of kG views, kStages slots.
+// float32, measured at 512^3: what counts is that the CTAs the registers allow
+// fit an SM (three with H = 1: 3 x 1 views 1.11 ms, 4 x 1 1.29; two with H = 2:
+// 4 x 1 1.61, 3 x 1 1.68).  16-bit, 2000^3: fewer waits, 2 x 3 views 5.1 ms, 3 x 2
+// 5.3, 2 x 2 5.4, 6 x 1 5.6.
+template <typename TQ, int H>
 struct Ring {
-    static constexpr int kG = sizeof(TQ) == 4 ? 1 : 2, kStages = sizeof(TQ) == 4 ? 3 : 2;
+    static constexpr int kG = sizeof(TQ) == 4 ? 1 : 3, kStages = sizeof(TQ) == 4 ? (H == 1 ? 3 : 4) : 2;
 };
 template <int H>
 constexpr int kLoaders = H == 1 ? 4 : 8;  // loader warps of the form without TMA
@@ -276,7 +278,7 @@ decompose_rows_kernel(const __grid_constant__ CUtensorMap tmap, const TQ *__rest
     static_assert(TMA || sizeof(TQ) == 4, "plain copies: float32 only");
     constexpr int ES = (int)sizeof(TQ);
     constexpr int kAlign = TMA ? 16 / ES : 1;
-    constexpr int kG = Ring<TQ>::kG, kStages = Ring<TQ>::kStages;
+    constexpr int kG = Ring<TQ, H>::kG, kStages = Ring<TQ, H>::kStages;
     constexpr int kProducers = TMA ? 1 : kLoaders<H>;
     extern __shared__ __align__(128) unsigned char smem_raw[];
     unsigned char *ring = smem_raw + ((128u - (tma::smem_u32(smem_raw) & 127u)) & 127u);
@@ -485,7 +487,7 @@ cudaError_t try_rows(const PlanImpl &p, const TQ *Q, float *out, cudaStream_t st
     if (cudaGetDevice(&dev) == cudaSuccess) cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
     constexpr int kLead = 2 * H - 1;  // a range streams kLead D - 1 views besides its own
     auto smem_of = [&](int jr) {
-        return dec_smem((int)sizeof(TQ), Ring<TQ>::kStages * Ring<TQ>::kG, tile_stride, warps, (jr + kLead) * p.D - 1, H);
+        return dec_smem((int)sizeof(TQ), Ring<TQ, H>::kStages * Ring<TQ, H>::kG, tile_stride, warps, (jr + kLead) * p.D - 1, H);
     };
     // The decimated views are split into ranges (the same sums in the same
     // order, so the same result) where (square, band) CTAs would not fill the
