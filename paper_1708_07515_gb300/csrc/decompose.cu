@@ -490,23 +490,28 @@ cudaError_t try_rows(const PlanImpl &p, const TQ *Q, float *out, cudaStream_t st
         return dec_smem((int)sizeof(TQ), Ring<TQ, H>::kStages * Ring<TQ, H>::kG, tile_stride, warps, (jr + kLead) * p.D - 1, H);
     };
     // The decimated views are split into ranges (the same sums in the same
-    // order, so the same result) where (square, band) CTAs would not fill the
-    // GPU twice -- a range then keeps at least 4 kLead decimated views -- and
-    // where a shorter table lets the CTAs that the registers allow share an SM
-    // (512^3 f32: 1.29 ms with two CTAs per SM, 1.11 with three)
+    // order, so the same result) of at least 4 kLead decimated views, by a
+    // model of the time: CTAs per SM times streamed views per CTA (8 more for
+    // its set-up) over the share of its rate that an SM reaches with 1, 2 or 3
+    // resident CTAs (512^3 f32: 1.88, 1.29, 1.11 ms; a shorter table can let one
+    // more fit).  352^3 x 514, 352 CTAs: 3 ranges 285 us, 2 362.
     const long long ctas = (long long)p.od.nsq * chunks * bands;
-    int ranges = (int)std::min<long long>(p.Pd, (4LL * sms + ctas - 1) / ctas);
-    int jrange = std::max((p.Pd + ranges - 1) / ranges, std::min(p.Pd, 4 * kLead));
     int per_sm = 0;
     if (cudaDeviceGetAttribute(&per_sm, cudaDevAttrMaxSharedMemoryPerMultiprocessor, dev) != cudaSuccess) per_sm = 0;
-    const size_t share = (size_t)per_sm / (H == 1 ? 3 : 2);
-    for (ranges = 1; (p.Pd + ranges - 1) / ranges >= std::min(p.Pd, 4 * kLead); ++ranges) {
-        const int jr = std::min(jrange, (p.Pd + ranges - 1) / ranges);
-        if (smem_of(jr) + 2048 <= share) {
+    const int producers = TMA ? 1 : kLoaders<H>;
+    int jrange = p.Pd;
+    double best = 0.0;
+    for (int r = 1; r <= 64; ++r) {
+        const int jr = (p.Pd + r - 1) / r;
+        if (r > 1 && jr < 4 * kLead) break;
+        const long long per = (ctas * ((p.Pd + jr - 1) / jr) + sms - 1) / sms;  // CTAs per SM
+        const long long fit = std::min<long long>(H == 1 ? 3 : 2, (long long)(per_sm / (smem_of(jr) + 2048)));
+        const double rate[] = {0.1, 0.59, 0.86, 1.0};
+        const double cost = (double)per * ((jr + kLead) * p.D + 8) / rate[std::max(0LL, std::min(fit, per))];
+        if (r == 1 || cost < best) {
+            best = cost;
             jrange = jr;
-            break;
         }
-        if (ranges == p.Pd) break;
     }
     const size_t smem = smem_of(jrange);
     if (smem > 200 * 1024 || bands > 65535) return cudaSuccess;
@@ -524,7 +529,7 @@ cudaError_t try_rows(const PlanImpl &p, const TQ *Q, float *out, cudaStream_t st
     cudaError_t e = ensure_smem<decompose_rows_kernel<TQ, H, TMA>>(smem);
     if (e != cudaSuccess) return e;
     dim3 grid(p.od.nsq * chunks, bands, (p.Pd + jrange - 1) / jrange);
-    decompose_rows_kernel<TQ, H, TMA><<<grid, 32 * (warps + (TMA ? 1 : kLoaders<H>)), smem, st>>>(
+    decompose_rows_kernel<TQ, H, TMA><<<grid, 32 * (warps + producers), smem, st>>>(
         map, Q, out, p.od.crop, p.od.geo, p.od.T, p.tapw, p.status, p.Tstride, p.g.P, p.D, p.Pd, rw.layout, Wc,
         tile_stride, segs, chunks, rw.rowoff, rw.rowend, jrange, p.g.Nu);
     return cudaGetLastError();
