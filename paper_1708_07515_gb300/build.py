@@ -20,8 +20,8 @@ INCLUDE = os.path.join(ROOT, "include")
 BUILD = os.path.join(HERE, "_build")
 LIB = os.path.join(HERE, "libfdkod.so")
 
-SOURCES = ["api.cu", "bounds.cu", "filter.cu", "decompose.cu", "backproject.cu", "bp_pair_f32.cu",
-           "bp_pair_bf16.cu", "bp_pair_f16.cu", "noalloc.cu", "slabs.cu",
+SOURCES = ["api.cu", "bounds.cu", "filter.cu", "decompose.cu", "backproject.cu", "bp_pair_od.cu",
+           "bp_pair_f32.cu", "bp_pair_bf16.cu", "bp_pair_f16.cu", "noalloc.cu", "slabs.cu",
            "netdec.cu"]
 ARCH = ["-gencode", "arch=compute_103a,code=sm_103a"]
 COMMON = ["-O3", "-std=c++17", "-lineinfo", "-Xcompiler", "-fPIC", "-I", INCLUDE]

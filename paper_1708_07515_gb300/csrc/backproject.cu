@@ -638,16 +638,22 @@ size_t smem_budget(size_t *per_sm = nullptr) {
     return optin > 2048 ? (size_t)optin - 2048 : 0;
 }
 
-// Views per ring slot of the pair kernel for windows of `rows` x WD elements
-// of es bytes: 2 where the SM then holds the CTAs that the registers allow
-// (each with its static shared memory and the runtime's reserve, 2 KiB
-// together at most), else 1 if one CTA fits, else 0.
-int pair_views(int es, int zp, int rows, int WD) {
+// Ring of the pair kernel for windows of `rows` x WD elements of es bytes: 3
+// slots of 2 views, or 2 of 2, where the SM then holds the CTAs that the
+// registers allow (each with its static shared memory and the runtime's
+// reserve, 2 KiB together at most), else 3 of 1 if one CTA fits; false if not.
+// (250^3, R = 2.5 N: 3 x 1 views 917 us, 2 x 2 846; 512^3: 3 x 2 8.35 ms, 2 x 2
+// 8.38.)
+bool pair_ring(int es, int zp, int rows, PairShape &s) {
     size_t per_sm = 0;
     const size_t budget = smem_budget(&per_sm);
-    const int ts = pair_tile_stride(es, rows, WD);
-    if ((size_t)pair_ctas(zp) * (pair_smem(es, 2, ts) + 2048) <= per_sm) return 2;
-    return pair_smem(es, 1, ts) <= budget ? 1 : 0;
+    const int ts = pair_tile_stride(es, rows, s.WD);
+    s.vps = 2;
+    for (s.slots = 3; s.slots >= 2; --s.slots)
+        if ((size_t)pair_ctas(zp) * (pair_smem(es, 2, s.slots, ts) + 2048) <= per_sm) return true;
+    s.vps = 1;
+    s.slots = 3;
+    return pair_smem(es, 1, 3, ts) <= budget;
 }
 
 // The pair kernel's shape for `pairs` pairs of slices per column; false where
@@ -668,7 +674,7 @@ bool pair_shape(const PlanImpl &p, const SquareSet &ss, bool direct, bool mirror
     const int n32 = (pairs + 31) / 32, n16 = (pairs + 15) / 16;
     s.zp = 32;
     if (ss.Rw <= 256 && tiles * n32 >= 2LL * pair_ctas(32) * sms && 64 * n32 <= 34 * n16 &&
-        (s.vps = pair_views(es, 32, ss.Rw, s.WD)) == 2)
+        pair_ring(es, 32, ss.Rw, s) && s.vps == 2)
         return true;
     s.zp = 16;
     // Clusters share the views where the tiles leave SMs idle: as many CTAs as
@@ -686,7 +692,7 @@ bool pair_shape(const PlanImpl &p, const SquareSet &ss, bool direct, bool mirror
         if (s.nsplit == 1 && ctas * 4 <= 3 * slots && views >= 64) s.nsplit = 4;
         if (s.nsplit == 1 && ctas * 4 <= 5 * slots && views >= 32) s.nsplit = 2;
     }
-    return ss.Rw2 <= 256 && (s.vps = pair_views(es, 16, ss.Rw2, s.WD)) > 0;
+    return ss.Rw2 <= 256 && pair_ring(es, 16, ss.Rw2, s);
 }
 
 // The staged kernel over the slices of b (mirror: over the whole detector and
@@ -730,8 +736,13 @@ cudaError_t try_launch_pair(const PlanImpl &p, const SquareSet &ss, bool direct,
         a.scale = (float)(M_PI / (double)p.Pd);
     }
     launched = true;
-    if (!direct || p.qtype == FDKOD_F32) return launch_pair_f32(direct, s, map, a, ss.nsq, st);
-    return p.qtype == FDKOD_BF16 ? launch_pair_bf16(s, map, a, ss.nsq, st) : launch_pair_f16(s, map, a, ss.nsq, st);
+    if (!direct) return launch_pair_od(s, map, a, ss.nsq, st);
+    switch (p.qtype) {
+        case FDKOD_F32: return launch_pair_f32(s, map, a, ss.nsq, st);
+        case FDKOD_BF16: return launch_pair_bf16(s, map, a, ss.nsq, st);
+        case FDKOD_F16: return launch_pair_f16(s, map, a, ss.nsq, st);
+    }
+    return cudaErrorInvalidValue;
 }
 
 }  // namespace

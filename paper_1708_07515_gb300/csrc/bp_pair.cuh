@@ -15,8 +15,10 @@ namespace fdkod {
 
 struct BpPairParams;
 struct PairShape;
-// one per source: decomposed data and float32 Q, bfloat16 Q, float16 Q
-cudaError_t launch_pair_f32(bool direct, const PairShape &s, const CUtensorMap &map, const BpPairParams &prm, int nsq,
+// one per source: decomposed data, float32 Q, bfloat16 Q, float16 Q
+cudaError_t launch_pair_od(const PairShape &s, const CUtensorMap &map, const BpPairParams &prm, int nsq,
+                           cudaStream_t st);
+cudaError_t launch_pair_f32(const PairShape &s, const CUtensorMap &map, const BpPairParams &prm, int nsq,
                             cudaStream_t st);
 cudaError_t launch_pair_bf16(const PairShape &s, const CUtensorMap &map, const BpPairParams &prm, int nsq,
                              cudaStream_t st);
@@ -69,9 +71,9 @@ struct BpPairParams {
 };
 
 // What a launch needs besides its parameters: the window width, slices per
-// slab, views per ring slot and CTAs per cluster pick the instantiation.
+// slab, views per ring slot, slots and CTAs per cluster pick the instantiation.
 struct PairShape {
-    int WD, zp, vps, nsplit;
+    int WD, zp, vps, slots, nsplit;
     bool mirror;
 };
 
@@ -235,7 +237,7 @@ __device__ __forceinline__ void pair_slices_any(float2 (&acc)[ZP], float w, floa
 
 // Warp-specialised: warp 8 is the producer (per chunk of VPS views it finds
 // the windows, writes the view parameters and issues the copies into a ring
-// of kPairSlots slots); warps 0-7 consume.  A slot is full when its copies
+// of SLOTS slots); warps 0-7 consume.  A slot is full when its copies
 // have landed (full[slot], which also publishes the producer's parameters)
 // and free again when all eight consumer warps have arrived on empty[slot]:
 // no block-wide barrier inside the view loop, so consumer warps drift within
@@ -258,7 +260,6 @@ struct PairView {
     float w2, zcr2;  // second slab: as b.w and zcr (not MIRROR)
     float pad[2];
 };
-constexpr int kPairSlots = 3;
 // a group's first or last row may lie one row outside its window (such a row
 // never enters a sum): one row of the widest window before and after the ring
 constexpr int kPairPad = 512;
@@ -271,7 +272,7 @@ constexpr int pair_ctas(int ZP) { return ZP == 32 ? 2 : 3; }
 // SPLIT: the nsplit CTAs of a cluster (grid z) take a range of the views each
 // and add up their sums through distributed shared memory, CTA r every
 // nsplit-th slice from r on, in the order of the ranges (pair_shape says where).
-template <typename TS, bool DIRECT, bool MIRROR, int WD, int ZP, int VPS, bool SPLIT>
+template <typename TS, bool DIRECT, bool MIRROR, int WD, int ZP, int VPS, int SLOTS, bool SPLIT>
 __global__ void __launch_bounds__(kPairThreads, pair_ctas(ZP))
 bp_pair_kernel(const __grid_constant__ CUtensorMap tmap, BpPairParams a) {
     constexpr int ES = (int)sizeof(TS);
@@ -281,8 +282,8 @@ bp_pair_kernel(const __grid_constant__ CUtensorMap tmap, BpPairParams a) {
     extern __shared__ __align__(128) unsigned char smem_raw[];
     TS *sm = (TS *)(smem_raw + ((128u - (tma::smem_u32(smem_raw) & 127u)) & 127u) + kPairPad);
     const uint32_t sbase = tma::smem_u32(sm);
-    __shared__ __align__(8) uint64_t full[kPairSlots], empty[kPairSlots];
-    __shared__ PairView s_view[kPairSlots * VPS];
+    __shared__ __align__(8) uint64_t full[SLOTS], empty[SLOTS];
+    __shared__ PairView s_view[SLOTS * VPS];
 
     const int tiles = a.tps * a.tps;
     const int q = blockIdx.x / tiles;
@@ -314,7 +315,7 @@ bp_pair_kernel(const __grid_constant__ CUtensorMap tmap, BpPairParams a) {
     auto win = [&](int sl, int w, int h) { return (uint32_t)((sl * VPS + w) * 2 + h) * (uint32_t)a.tile_stride; };
 
     if (threadIdx.x == 0) {
-        for (int i = 0; i < kPairSlots; ++i) {
+        for (int i = 0; i < SLOTS; ++i) {
             tma::mbar_init(&full[i], 1);
             tma::mbar_init(&empty[i], kPairConsumers);
         }
@@ -333,7 +334,7 @@ bp_pair_kernel(const __grid_constant__ CUtensorMap tmap, BpPairParams a) {
         const float cz = (cc & 4) ? 0.5f * (float)(ZP - 1) : -0.5f * (float)(ZP - 1);
         int c = 0;
         for (; c < nch; ++c) {
-            const int sl = c % kPairSlots;
+            const int sl = c % SLOTS;
             const int nj = min(VPS, nviews - c * VPS);
             const int j = j0 + c * VPS + min(w, nj - 1);  // lanes past the chunk repeat its last view
             const int k = j * a.vstep;
@@ -377,8 +378,8 @@ bp_pair_kernel(const __grid_constant__ CUtensorMap tmap, BpPairParams a) {
             // round r of a slot may start once its round r - 1 was consumed
             // (lane 0 waits; the warp follows its answer)
             bool ok = true;
-            if (c >= kPairSlots && lane == 0)
-                ok = tma::mbar_wait_spin(&empty[sl], (uint32_t)(((c / kPairSlots) & 1) ^ 1), a.wait_ns);
+            if (c >= SLOTS && lane == 0)
+                ok = tma::mbar_wait_spin(&empty[sl], (uint32_t)(((c / SLOTS) & 1) ^ 1), a.wait_ns);
             if (!__shfl_sync(0xffffffffu, ok, 0)) {
                 if (lane == 0) atomicOr(a.status, 2);
                 break;
@@ -432,8 +433,8 @@ bp_pair_kernel(const __grid_constant__ CUtensorMap tmap, BpPairParams a) {
         }
         // copies still in flight must land before the CTA may exit
         if (lane == 0)
-            for (int m = max(0, c - kPairSlots); m < c; ++m)
-                tma::mbar_wait_bounded(&full[m % kPairSlots], (uint32_t)((m / kPairSlots) & 1), a.wait_ns);
+            for (int m = max(0, c - SLOTS); m < c; ++m)
+                tma::mbar_wait_bounded(&full[m % SLOTS], (uint32_t)((m / SLOTS) & 1), a.wait_ns);
         if constexpr (SPLIT) {
             __syncwarp();
             cluster_sync();
@@ -500,7 +501,7 @@ bp_pair_kernel(const __grid_constant__ CUtensorMap tmap, BpPairParams a) {
         }
         __syncwarp();
         if (lane == 0) tma::mbar_arrive(&empty[sl]);  // this warp is done with the slot
-        if (++sl == kPairSlots) {
+        if (++sl == SLOTS) {
             sl = 0;
             phase ^= 1u;
         }
@@ -548,18 +549,18 @@ bp_pair_kernel(const __grid_constant__ CUtensorMap tmap, BpPairParams a) {
 // elements per staged window of the pair kernel, a 128-byte multiple
 inline int pair_tile_stride(int es, int rows, int WD) { return (rows * WD + (128 / es - 1)) & ~(128 / es - 1); }
 
-// dynamic shared memory of the pair kernel: kPairSlots slots of VPS views,
-// two windows per view, plus the pads and the 128-byte alignment slack
-inline size_t pair_smem(int es, int vps, int tile_stride) {
-    return (size_t)es * kPairSlots * vps * 2 * tile_stride + 2 * kPairPad + 128;
+// dynamic shared memory of the pair kernel: `slots` slots of vps views, two
+// windows per view, plus the pads and the 128-byte alignment slack
+inline size_t pair_smem(int es, int vps, int slots, int tile_stride) {
+    return (size_t)es * slots * vps * 2 * tile_stride + 2 * kPairPad + 128;
 }
 
-template <typename TS, bool DIRECT, bool MIRROR, int WD, int ZP, int VPS, bool SPLIT = false>
+template <typename TS, bool DIRECT, bool MIRROR, int WD, int ZP, int VPS, int SLOTS, bool SPLIT = false>
 cudaError_t launch_pair_t(const CUtensorMap &map, const BpPairParams &prm, int nsq, cudaStream_t st) {
-    size_t smem = pair_smem((int)sizeof(TS), VPS, prm.tile_stride);
+    size_t smem = pair_smem((int)sizeof(TS), VPS, SLOTS, prm.tile_stride);
     // SPLIT: the ring also holds the CTA's sums
     if (SPLIT) smem = std::max(smem, sizeof(float2) * ZP * 32 * kPairConsumers + 2 * (size_t)kPairPad + 128);
-    cudaError_t e = ensure_smem<bp_pair_kernel<TS, DIRECT, MIRROR, WD, ZP, VPS, SPLIT>>(smem);
+    cudaError_t e = ensure_smem<bp_pair_kernel<TS, DIRECT, MIRROR, WD, ZP, VPS, SLOTS, SPLIT>>(smem);
     if (e != cudaSuccess) return e;
     constexpr int kSlices = MIRROR ? ZP : 2 * ZP;
     cudaLaunchConfig_t cfg{};
@@ -574,22 +575,27 @@ cudaError_t launch_pair_t(const CUtensorMap &map, const BpPairParams &prm, int n
     at.val.clusterDim.z = SPLIT ? (unsigned)prm.nsplit : 1u;
     cfg.attrs = &at;
     cfg.numAttrs = SPLIT ? 1 : 0;
-    return cudaLaunchKernelEx(&cfg, bp_pair_kernel<TS, DIRECT, MIRROR, WD, ZP, VPS, SPLIT>, map, prm);
+    return cudaLaunchKernelEx(&cfg, bp_pair_kernel<TS, DIRECT, MIRROR, WD, ZP, VPS, SLOTS, SPLIT>, map, prm);
 }
 
-// 32 slices per slab always come with 2 views per slot and no split, a split
-// with whole volumes (pair_shape)
+// the shapes pair_shape gives: 32 slices per slab with 2 views per slot and no
+// split, a split with whole volumes; 3 slots of 2 views, 2 of 2 or 3 of 1
+template <typename TS, bool DIRECT, bool MIRROR, int WD, int ZP, bool SPLIT = false>
+cudaError_t launch_pair_v(const PairShape &s, const CUtensorMap &map, const BpPairParams &prm, int nsq,
+                          cudaStream_t st) {
+    if (s.vps == 2 && s.slots == 3) return launch_pair_t<TS, DIRECT, MIRROR, WD, ZP, 2, 3, SPLIT>(map, prm, nsq, st);
+    if (s.vps == 2) return launch_pair_t<TS, DIRECT, MIRROR, WD, ZP, 2, 2, SPLIT>(map, prm, nsq, st);
+    if constexpr (ZP == 16) return launch_pair_t<TS, DIRECT, MIRROR, WD, ZP, 1, 3, SPLIT>(map, prm, nsq, st);
+    return cudaErrorInvalidValue;
+}
+
 template <typename TS, bool DIRECT, bool MIRROR, int WD>
 cudaError_t launch_pair_z(const PairShape &s, const CUtensorMap &map, const BpPairParams &prm, int nsq,
                           cudaStream_t st) {
-    if (s.zp == 32) return launch_pair_t<TS, DIRECT, MIRROR, WD, 32, 2>(map, prm, nsq, st);
-    if constexpr (MIRROR) {
-        if (s.nsplit > 1)
-            return s.vps == 2 ? launch_pair_t<TS, DIRECT, MIRROR, WD, 16, 2, true>(map, prm, nsq, st)
-                              : launch_pair_t<TS, DIRECT, MIRROR, WD, 16, 1, true>(map, prm, nsq, st);
-    }
-    return s.vps == 2 ? launch_pair_t<TS, DIRECT, MIRROR, WD, 16, 2>(map, prm, nsq, st)
-                      : launch_pair_t<TS, DIRECT, MIRROR, WD, 16, 1>(map, prm, nsq, st);
+    if (s.zp == 32) return launch_pair_v<TS, DIRECT, MIRROR, WD, 32>(s, map, prm, nsq, st);
+    if constexpr (MIRROR)
+        if (s.nsplit > 1) return launch_pair_v<TS, DIRECT, MIRROR, WD, 16, true>(s, map, prm, nsq, st);
+    return launch_pair_v<TS, DIRECT, MIRROR, WD, 16>(s, map, prm, nsq, st);
 }
 
 template <typename TS, bool DIRECT, bool MIRROR>
