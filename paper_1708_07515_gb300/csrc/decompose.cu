@@ -513,6 +513,15 @@ cudaError_t try_rows(const PlanImpl &p, const TQ *Q, float *out, cudaStream_t st
             jrange = jr;
         }
     }
+    // The 4-byte copies pay where a CTA's consumers have enough to do beside
+    // them -- one CTA as wide as the square, six segments or more -- and either
+    // the GPU is filled or the ranges are short (64 rows x 360 views: 963^3, 108
+    // columns a square, 974 us against 1299 with one thread per output, 56
+    // columns 2703 against 2797, windowed sinc 4138 against 2945, 132 columns 1829
+    // against 1424; 125^3 33 against 100, with the sinc and D = 16 349 against 108)
+    if (!TMA && (chunks > 1 || segs < 6 ||
+                 (ctas * ((p.Pd + jrange - 1) / jrange) < 2LL * sms && (jrange + kLead) * p.D > 128)))
+        return cudaSuccess;
     const size_t smem = smem_of(jrange);
     if (smem > 200 * 1024 || bands > 65535) return cudaSuccess;
     CUtensorMap map{};

@@ -54,8 +54,9 @@ def _forms(plan, Q):
     (250, 256, 35, 40, 0, 4, 3.0),   # three CTAs side by side
     (200, 200, 64, 400, 1, 2, 4.0),  # ranges of decimated views
     (61, 64, 70, 900, 3, 2, 1.6),    # many views, ragged squares, a near source
-    (61, 63, 45, 60, 1, 3, 2.5),     # odd detector: 4-byte copies
-    (150, 149, 40, 48, 0, 2, 4.0),   # and wider than 128 columns
+    (125, 125, 45, 60, 1, 3, 2.5),   # odd detector: 4-byte copies (81 to 128 columns a square)
+    (61, 63, 45, 60, 1, 3, 2.5),     # narrower
+    (150, 149, 40, 48, 0, 2, 4.0),   # wider than 128 columns
 ])
 def test_staged_equals_generic(fd, qtype, taps, N, Nu, Nv, P, s, D, r):
     Q = torch.from_numpy(np.random.default_rng(N + P).standard_normal((P, Nv, Nu)).astype(np.float32))
