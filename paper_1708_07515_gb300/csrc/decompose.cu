@@ -23,8 +23,6 @@
 namespace fdkod {
 namespace {
 
-constexpr int kTX = 64, kTY = 4;
-
 __device__ __forceinline__ float ld_q(const float *p) { return __ldg(p); }
 __device__ __forceinline__ float ld_q(const __nv_bfloat16 *p) { return __bfloat162float(__ldg(p)); }
 __device__ __forceinline__ float ld_q(const __half *p) { return __half2float(__ldg(p)); }
@@ -32,61 +30,83 @@ __device__ __forceinline__ float ld_q(const __half *p) { return __half2float(__l
 // floor(a / b) for b > 0
 __host__ __device__ __forceinline__ int floor_div(int a, int b) { return a >= 0 ? a / b : -((-a + b - 1) / b); }
 
-// Generic path: one thread per (q, v, t), consecutive threads on consecutive
-// t (each view's crop row is one coalesced segment).
+// Generic path: a warp takes 32 consecutive columns of kGenRows rows, straight
+// from global memory (each view's crop row is one run).  The rows share the
+// view's crop, shift and weights and keep their loads in flight together; the
+// next view's entries are read while this one's samples arrive.  Bound by the
+// two loads per sample.  Against one row per thread: 963^3 x 64 rows x 360 views
+// f16 1233 -> 688 us, 501^3 x 720 bf16 5.5 -> 3.7 ms (2 rows: 752, 3.7; 8: 749,
+// 3.9).  It also beat staging the crops by 4-byte asynchronous copies (501^3
+// f32 3.4 against 3.8 ms, 250^3 210 against 255 us).
+constexpr int kGenRows = 4, kGenWarps = 8;
 template <typename TQ, int H>
-__global__ void __launch_bounds__(kTX *kTY)
+__global__ void __launch_bounds__(32 * kGenWarps)
 decompose_kernel(const TQ *__restrict__ Q, float *__restrict__ Sp, const int32_t *__restrict__ crop,
                  const GeomEntry *__restrict__ geo, const int32_t *__restrict__ Tq, const float4 *__restrict__ tapw,
-                 int Tstride, int P, int D, int Pd, int Nv, int Nu, int rowoff, int rowend) {
-    const int t = blockIdx.x * kTX + threadIdx.x;
-    const int v = rowoff + blockIdx.y * kTY + threadIdx.y;
+                 int Tstride, int P, int D, int Pd, int Nv, int Nu, int rowoff, int rowend, int tiles, int jrange) {
+    // grid x: 32-column tiles of every range of decimated views j0 .. j1 - 1
+    const int range = blockIdx.x / tiles, j0 = range * jrange, j1 = min(j0 + jrange, Pd);
+    const int t = (blockIdx.x - range * tiles) * 32 + threadIdx.x;
+    const int v = rowoff + (blockIdx.y * kGenWarps + threadIdx.y) * kGenRows;
     const int q = blockIdx.z;
     if (t >= Tstride || v >= rowend) return;
     const size_t vstride = (size_t)Nv * Tstride;
     float *out = Sp + ((size_t)q * Pd * Nv + v) * Tstride + t;
+    const int rows = min(kGenRows, rowend - v);
     if (t >= Tq[q]) {
-        for (int j = 0; j < Pd; ++j) out[(size_t)j * vstride] = 0.f;
+        for (int j = j0; j < j1; ++j)
+            for (int r = 0; r < rows; ++r) out[(size_t)j * vstride + (size_t)r * Tstride] = 0.f;
         return;
     }
-    const size_t qo = (size_t)q * P;
-    const size_t row = (size_t)v * Nu;
+    const int32_t *cq = crop + (size_t)q * P;
+    const GeomEntry *gq = geo + (size_t)q * P;
     const size_t view = (size_t)Nv * Nu;
-    auto sample = [&](int k) -> float {
-        const int c = __ldg(crop + qo + k) + t;
-        const float f = __ldg(&geo[qo + k].frac);
-        const TQ *r = Q + (size_t)k * view + row;
-        const float a = (c >= 0 && c < Nu) ? ld_q(r + c) : 0.f;
-        const float b = (c + 1 >= 0 && c + 1 < Nu) ? ld_q(r + c + 1) : 0.f;
-        return fmaf(f, b - a, a);
-    };
-    float acc[2 * H];
+    const TQ *Qv = Q + (size_t)v * Nu;
+    float acc[kGenRows][2 * H];
 #pragma unroll
-    for (int m = 0; m < 2 * H; ++m) acc[m] = 0.f;
-    const int nstream = P + (2 * H - 1) * D - 1;
-    const int kp0 = -(H * D - 1);
-    int jb = floor_div(kp0, D), r = kp0 - jb * D, kk = ((kp0 % P) + P) % P;
-    for (int pos = 0; pos < nstream; ++pos) {
-        const float sm = sample(kk);
-        const float4 w = __ldg(tapw + r);
-        const float wm[4] = {w.x, w.y, w.z, w.w};
+    for (int r = 0; r < kGenRows; ++r)
 #pragma unroll
-        for (int m = 0; m < 2 * H; ++m) acc[m] = fmaf(wm[m], sm, acc[m]);
-        if (r == D - 1) {
-            const int jst = jb - H + 1;  // its support is complete
-            if (jst >= 0) out[(size_t)jst * vstride] = acc[0];
+        for (int m = 0; m < 2 * H; ++m) acc[r][m] = 0.f;
+    // block by block from the second view of block j0 - H (its end completes
+    // decimated view j0 + 1 - 2 H), the views taken mod P
+    int kk = (((j0 - H) * D + 1) % P + P) % P, r0 = 1;
+    int c = __ldg(cq + kk) + t;
+    float f = __ldg(&gq[kk].frac);
+    for (int jst = j0 + 1 - 2 * H; jst < j1; ++jst, r0 = 0) {
+        for (int rr = r0; rr < D; ++rr) {
+            const TQ *row = Qv + (size_t)kk * view + c;
+            const bool in0 = c >= 0 && c < Nu, in1 = c >= -1 && c < Nu - 1;
+            float a[kGenRows], b[kGenRows];
 #pragma unroll
-            for (int m = 0; m < 2 * H - 1; ++m) acc[m] = acc[m + 1];
-            acc[2 * H - 1] = 0.f;
-            r = 0;
-            ++jb;
-        } else {
-            ++r;
+            for (int r = 0; r < kGenRows; ++r) {
+                a[r] = in0 && r < rows ? ld_q(row + r * Nu) : 0.f;
+                b[r] = in1 && r < rows ? ld_q(row + r * Nu + 1) : 0.f;
+            }
+            const float fk = f;
+            const float4 w = __ldg(tapw + rr);
+            if (++kk == P) kk = 0;
+            c = __ldg(cq + kk) + t;
+            f = __ldg(&gq[kk].frac);
+            const float wm[4] = {w.x, w.y, w.z, w.w};
+#pragma unroll
+            for (int r = 0; r < kGenRows; ++r) {
+                const float smp = fmaf(fk, b[r] - a[r], a[r]);
+#pragma unroll
+                for (int m = 0; m < 2 * H; ++m) acc[r][m] = fmaf(wm[m], smp, acc[r][m]);
+            }
         }
-        if (++kk == P) kk = 0;
+        if (jst >= j0)
+#pragma unroll
+            for (int r = 0; r < kGenRows; ++r)
+                if (r < rows) out[(size_t)jst * vstride + (size_t)r * Tstride] = acc[r][0];
+#pragma unroll
+        for (int r = 0; r < kGenRows; ++r) {
+#pragma unroll
+            for (int m = 0; m < 2 * H - 1; ++m) acc[r][m] = acc[r][m + 1];
+            acc[r][2 * H - 1] = 0.f;
+        }
     }
 }
-
 
 // ---------------------------------------------------------------------------
 // Staged path: one CTA per (square q, band of detector rows, range of decimated
@@ -112,14 +132,6 @@ decompose_kernel(const TQ *__restrict__ Q, float *__restrict__ Sp, const int32_t
 // two scalar loads per sample, and columns in steps of 32 lanes (128 computed
 // for ~100 used).
 //
-// Where TMA cannot describe a float32 Q (its rows are not whole 16-byte units,
-// or it is not 16-byte aligned: odd detector widths), kLoaders warps copy the
-// crops with 4-byte asynchronous copies, starting at the crop's own column
-// (offset 0), into the same ring; the consumers are the same.  Bound by those
-// copies: 501^3 x 720 views 3.8 ms (windowed sinc 4.6 with 8 loader warps, 6.3
-// with 4) against 5.8 (6.0) with one thread per output, which 16-bit Q keeps
-// (staged by plain 2-byte loads it took 15 ms against 5.6).
-//
 // Everything else a view needs -- shift fraction, tap weights, crop offset --
 // is one 16-byte entry of a per-CTA table in stream order (H = 2: 8 more bytes
 // of weights), built once.  Views go block by block (D views): a block's end
@@ -137,8 +149,6 @@ template <typename TQ, int H>
 struct Ring {
     static constexpr int kG = sizeof(TQ) == 4 ? 1 : 3, kStages = sizeof(TQ) == 4 ? (H == 1 ? 3 : 4) : 2;
 };
-template <int H>
-constexpr int kLoaders = H == 1 ? 4 : 8;  // loader warps of the form without TMA
 constexpr int kRingSlack = 128;  // the last segment's loads run up to 16 bytes past a row's end
 constexpr uint64_t kDecWaitNs = 2000000000ull;
 
@@ -257,29 +267,18 @@ __host__ __device__ inline size_t dec_smem(int es, int stages, int tile_stride, 
            (size_t)nstream * (16 + (H == 2 ? 8 : 0) + 4);
 }
 
-// 4-byte asynchronous copy global -> shared (zero where !in), and the arrival
-// of this thread's earlier ones on `bar`
-__device__ __forceinline__ void cp_async4(uint32_t dst, const float *src, bool in) {
-    asm volatile("cp.async.ca.shared.global [%0], [%1], 4, %2;" ::"r"(dst), "l"(src), "r"(in ? 4u : 0u) : "memory");
-}
-__device__ __forceinline__ void cp_async_arrive(uint64_t *bar) {
-    asm volatile("cp.async.mbarrier.arrive.noinc.shared::cta.b64 [%0];" ::"r"(tma::smem_u32(bar)) : "memory");
-}
-
 // the thread bound only sets the register limit: 80 (24 warps per SM) for the
 // two running sums of the triangle, 128 (16 warps) for the four of 2D-tap filters
-template <typename TQ, int H, bool TMA>
+template <typename TQ, int H>
 __global__ void __launch_bounds__(H == 1 ? 768 : 512, 1)
-decompose_rows_kernel(const __grid_constant__ CUtensorMap tmap, const TQ *__restrict__ Q, float *__restrict__ Sp,
+decompose_rows_kernel(const __grid_constant__ CUtensorMap tmap, float *__restrict__ Sp,
                       const int32_t *__restrict__ crop, const GeomEntry *__restrict__ geo,
                       const int32_t *__restrict__ Tq, const float4 *__restrict__ tapw, int *status, int Tstride,
                       int P, int D, int Pd, int Nv, int Wc, int tile_stride, int segs, int chunks, int rowoff, int rowend,
-                      int jrange, int Nu) {
-    static_assert(TMA || sizeof(TQ) == 4, "plain copies: float32 only");
+                      int jrange) {
     constexpr int ES = (int)sizeof(TQ);
-    constexpr int kAlign = TMA ? 16 / ES : 1;
+    constexpr int kAlign = 16 / ES;
     constexpr int kG = Ring<TQ, H>::kG, kStages = Ring<TQ, H>::kStages;
-    constexpr int kProducers = TMA ? 1 : kLoaders<H>;
     extern __shared__ __align__(128) unsigned char smem_raw[];
     unsigned char *ring = smem_raw + ((128u - (tma::smem_u32(smem_raw) & 127u)) & 127u);
     const uint32_t tile_bytes = (uint32_t)(ES * tile_stride);
@@ -287,7 +286,7 @@ decompose_rows_kernel(const __grid_constant__ CUtensorMap tmap, const TQ *__rest
     // views streamed: k' = j0 D - (H D - 1) .. (j1 - 1) D + H D - 1 (view k' mod P)
     const int nstream = (j1 - j0) * D + (2 * H - 1) * D - 1;
     const int nstage = (nstream + kG - 1) / kG;
-    const int warps = (int)(blockDim.x >> 5) - kProducers;  // consumer warps
+    const int warps = (int)(blockDim.x >> 5) - 1;  // consumer warps
     float *tbuf = (float *)(ring + (size_t)tile_bytes * kStages * kG + kRingSlack);
     float4 *s_v = (float4 *)(tbuf + (size_t)warps * 32 * kTP);
     float2 *s_w2 = (float2 *)(s_v + nstream);
@@ -303,52 +302,14 @@ decompose_rows_kernel(const __grid_constant__ CUtensorMap tmap, const TQ *__rest
     build_stream_table<kAlign, H>(s_v, s_w2, s_c, crop, geo, tapw, q, P, D, j0, nstream);
     if (threadIdx.x == 0) {
         for (int i = 0; i < kStages; ++i) {
-            tma::mbar_init(&full[i], TMA ? 1 : 32 * kProducers);
+            tma::mbar_init(&full[i], 1);
             tma::mbar_init(&empty[i], warps);
         }
         tma::fence_mbar_init();
     }
     __syncthreads();
 
-    if constexpr (!TMA) {
-        if (warp >= warps) {  // loader: rows lw, lw + kProducers, ... of the band
-            const int lw = warp - warps;
-            int kk = ((j0 * D - (H * D - 1)) % P + P) % P, slot = 0;
-            uint32_t phase = 0;
-            for (int n = 0; n < nstream; ++n) {
-                static_assert(TMA || kG == 1, "one view per slot");
-                if (n >= kStages && !tma::mbar_wait_bounded(&empty[slot], phase ^ 1u, kDecWaitNs)) {
-                    if (lane == 0) atomicOr(status, 2);
-                    asm volatile("cp.async.wait_all;" ::: "memory");
-                    return;
-                }
-                const int c0 = s_c[n] + tc;
-                const float *src = Q + (ptrdiff_t)kk * Nv * Nu + c0 + lane;
-                const uint32_t dst = tma::smem_u32(ring + (size_t)tile_bytes * slot) + 4u * (uint32_t)lane;
-                constexpr int kCols = (kDecMaxSegs * kCW + 4 + 31) / 32;  // 32-column steps of the widest box
-#pragma unroll 4
-                for (int r = lw; r < band; r += kProducers) {
-                    const int v = v0 + r;
-                    const float *row = src + (ptrdiff_t)v * Nu;
-#pragma unroll
-                    for (int i = 0; i < kCols; ++i) {
-                        const int c = 32 * i + lane;
-                        const bool in = v < Nv && c0 + c >= 0 && c0 + c < Nu;  // else zeros
-                        if (c < Wc) cp_async4(dst + 4u * (uint32_t)(r * Wc + 32 * i), in ? row + 32 * i : Q, in);
-                    }
-                }
-                cp_async_arrive(&full[slot]);  // once this lane's copies have landed
-                if (++kk == P) kk = 0;
-                if (++slot == kStages) {
-                    slot = 0;
-                    phase ^= 1u;
-                }
-            }
-            // copies still in flight must land before the CTA may exit
-            asm volatile("cp.async.wait_all;" ::: "memory");
-            return;
-        }
-    } else if (warp == warps) {  // producer
+    if (warp == warps) {  // producer
         if (lane != 0) return;
         int kk = ((j0 * D - (H * D - 1)) % P + P) % P, n = 0, slot = 0;
         uint32_t phase = 0;  // parity of the slot's current round
@@ -419,8 +380,7 @@ decompose_rows_kernel(const __grid_constant__ CUtensorMap tmap, const TQ *__rest
                 wt[2] = e2.x;
                 wt[3] = e2.y;
             }
-            if constexpr (TMA) view_any<TQ, H>(__float_as_int(e.y), a, e.x, wt, acc);
-            else view_step<TQ, H, 0>(a, e.x, wt, acc);
+            view_any<TQ, H>(__float_as_int(e.y), a, e.x, wt, acc);
             a += tile_bytes;
             if (++w == kG) {
                 w = 0;
@@ -463,19 +423,19 @@ struct Rows {
     int layout, rowoff, rowend;
 };
 
-// Applies when S' is 16-byte aligned (vector stores), D <= 128 and the ring
-// plus the stream tables fit in shared memory; TMA: when Q is 16-byte aligned
-// and its rows are whole 16-byte units.
-template <typename TQ, int H, bool TMA>
+// Applies when Q and S' are 16-byte aligned (vector stores), Q's rows are whole
+// 16-byte units, D <= 128 and the ring plus the stream tables fit in shared
+// memory.
+template <typename TQ, int H>
 cudaError_t try_rows(const PlanImpl &p, const TQ *Q, float *out, cudaStream_t st, Rows rw, bool &launched) {
     launched = false;
     constexpr int kAlign = 16 / (int)sizeof(TQ);
-    if (TMA && ((p.g.Nu % kAlign) != 0 || ((uintptr_t)Q & 15) != 0)) return cudaSuccess;
-    if (((uintptr_t)out & 15) != 0 || p.D > kMaxTapD) return cudaSuccess;
+    if ((p.g.Nu % kAlign) != 0 || ((uintptr_t)Q & 15) != 0 || ((uintptr_t)out & 15) != 0) return cudaSuccess;
+    if (p.D > kMaxTapD) return cudaSuccess;
     const int all = (p.Tstride + kCW - 1) / kCW;  // column segments of a square
     const int chunks = (all + kDecMaxSegs - 1) / kDecMaxSegs, segs = (all + chunks - 1) / chunks;
     // the segments' columns + neighbour + crop offset, whole 16-byte units, an odd number of them
-    int Wc = (std::min(p.od.Tmax, segs * kCW) + 1 + (TMA ? kAlign - 1 : 0) + (kAlign - 1)) & ~(kAlign - 1);
+    int Wc = (std::min(p.od.Tmax, segs * kCW) + 1 + (kAlign - 1) + (kAlign - 1)) & ~(kAlign - 1);
     if ((Wc / kAlign) % 2 == 0) Wc += kAlign;
     const int nrows = rw.rowend - rw.rowoff;
     // narrow squares: several row groups per CTA, at least four consumer warps
@@ -498,7 +458,6 @@ cudaError_t try_rows(const PlanImpl &p, const TQ *Q, float *out, cudaStream_t st
     const long long ctas = (long long)p.od.nsq * chunks * bands;
     int per_sm = 0;
     if (cudaDeviceGetAttribute(&per_sm, cudaDevAttrMaxSharedMemoryPerMultiprocessor, dev) != cudaSuccess) per_sm = 0;
-    const int producers = TMA ? 1 : kLoaders<H>;
     int jrange = p.Pd;
     double best = 0.0;
     for (int r = 1; r <= 64; ++r) {
@@ -513,61 +472,47 @@ cudaError_t try_rows(const PlanImpl &p, const TQ *Q, float *out, cudaStream_t st
             jrange = jr;
         }
     }
-    // The 4-byte copies pay where a CTA's consumers have enough to do beside
-    // them -- one CTA as wide as the square, six segments or more -- and either
-    // the GPU is filled or the ranges are short (64 rows x 360 views: 963^3, 108
-    // columns a square, 974 us against 1299 with one thread per output, 56
-    // columns 2703 against 2797, windowed sinc 4138 against 2945, 132 columns 1829
-    // against 1424; 125^3 33 against 100, with the sinc and D = 16 349 against 108)
-    if (!TMA && (chunks > 1 || segs < 6 ||
-                 (ctas * ((p.Pd + jrange - 1) / jrange) < 2LL * sms && (jrange + kLead) * p.D > 128)))
-        return cudaSuccess;
     const size_t smem = smem_of(jrange);
     if (smem > 200 * 1024 || bands > 65535) return cudaSuccess;
-    CUtensorMap map{};
-    if constexpr (TMA) {
-        const uint64_t dims[3] = {(uint64_t)p.g.Nu, (uint64_t)rw.layout, (uint64_t)p.g.P};
-        const uint64_t strides[2] = {(uint64_t)p.g.Nu * sizeof(TQ), (uint64_t)p.g.Nu * rw.layout * sizeof(TQ)};
-        const uint32_t box[3] = {(uint32_t)Wc, (uint32_t)band, 1u};
-        const CUtensorMapDataType dt = sizeof(TQ) == 4 ? CU_TENSOR_MAP_DATA_TYPE_FLOAT32
-                                       : (std::is_same<TQ, __half>::value ? CU_TENSOR_MAP_DATA_TYPE_FLOAT16
-                                                                          : CU_TENSOR_MAP_DATA_TYPE_BFLOAT16);
-        if (encode_map_3d(&map, dt, Q, dims, strides, box) != cudaSuccess) return cudaSuccess;
-    }
+    CUtensorMap map;
+    const uint64_t dims[3] = {(uint64_t)p.g.Nu, (uint64_t)rw.layout, (uint64_t)p.g.P};
+    const uint64_t strides[2] = {(uint64_t)p.g.Nu * sizeof(TQ), (uint64_t)p.g.Nu * rw.layout * sizeof(TQ)};
+    const uint32_t box[3] = {(uint32_t)Wc, (uint32_t)band, 1u};
+    const CUtensorMapDataType dt = sizeof(TQ) == 4 ? CU_TENSOR_MAP_DATA_TYPE_FLOAT32
+                                   : (std::is_same<TQ, __half>::value ? CU_TENSOR_MAP_DATA_TYPE_FLOAT16
+                                                                      : CU_TENSOR_MAP_DATA_TYPE_BFLOAT16);
+    if (encode_map_3d(&map, dt, Q, dims, strides, box) != cudaSuccess) return cudaSuccess;
     launched = true;
-    cudaError_t e = ensure_smem<decompose_rows_kernel<TQ, H, TMA>>(smem);
+    cudaError_t e = ensure_smem<decompose_rows_kernel<TQ, H>>(smem);
     if (e != cudaSuccess) return e;
     dim3 grid(p.od.nsq * chunks, bands, (p.Pd + jrange - 1) / jrange);
-    decompose_rows_kernel<TQ, H, TMA><<<grid, 32 * (warps + producers), smem, st>>>(
-        map, Q, out, p.od.crop, p.od.geo, p.od.T, p.tapw, p.status, p.Tstride, p.g.P, p.D, p.Pd, rw.layout, Wc,
-        tile_stride, segs, chunks, rw.rowoff, rw.rowend, jrange, p.g.Nu);
+    decompose_rows_kernel<TQ, H><<<grid, 32 * (warps + 1), smem, st>>>(
+        map, out, p.od.crop, p.od.geo, p.od.T, p.tapw, p.status, p.Tstride, p.g.P, p.D, p.Pd, rw.layout, Wc,
+        tile_stride, segs, chunks, rw.rowoff, rw.rowend, jrange);
     return cudaGetLastError();
-}
-
-template <typename TQ, int H>
-cudaError_t try_staged(const PlanImpl &p, const TQ *Q, float *out, cudaStream_t st, Rows rw, bool &launched) {
-    cudaError_t e = try_rows<TQ, H, true>(p, Q, out, st, rw, launched);
-    if constexpr (sizeof(TQ) == 4)
-        if (!launched && e == cudaSuccess) e = try_rows<TQ, H, false>(p, Q, out, st, rw, launched);
-    return e;
 }
 
 template <typename TQ>
 cudaError_t launch_t(const PlanImpl &p, const TQ *Q, float *out, cudaStream_t st, Rows rw) {
     if (p.tap_blocks != 1 && p.tap_blocks != 2) return cudaErrorInvalidValue;
     bool launched = false;
-    cudaError_t te = p.tap_blocks == 2 ? try_staged<TQ, 2>(p, Q, out, st, rw, launched)
-                                       : try_staged<TQ, 1>(p, Q, out, st, rw, launched);
+    cudaError_t te = p.tap_blocks == 2 ? try_rows<TQ, 2>(p, Q, out, st, rw, launched)
+                                       : try_rows<TQ, 1>(p, Q, out, st, rw, launched);
     if (launched || te != cudaSuccess) return te;
-    dim3 grid((p.Tstride + kTX - 1) / kTX, (rw.rowend - rw.rowoff + kTY - 1) / kTY, p.od.nsq);
-    if (p.tap_blocks == 2)
-        decompose_kernel<TQ, 2><<<grid, dim3(kTX, kTY), 0, st>>>(Q, out, p.od.crop, p.od.geo, p.od.T, p.tapw,
-                                                                 p.Tstride, p.g.P, p.D, p.Pd, rw.layout, p.g.Nu,
-                                                                 rw.rowoff, rw.rowend);
-    else
-        decompose_kernel<TQ, 1><<<grid, dim3(kTX, kTY), 0, st>>>(Q, out, p.od.crop, p.od.geo, p.od.T, p.tapw,
-                                                                 p.Tstride, p.g.P, p.D, p.Pd, rw.layout, p.g.Nu,
-                                                                 rw.rowoff, rw.rowend);
+    constexpr int kBandRows = kGenWarps * kGenRows;
+    const int tiles = (p.Tstride + 31) / 32, bands = (rw.rowend - rw.rowoff + kBandRows - 1) / kBandRows;
+    // ranges of decimated views until every SM has eight CTAs, of at least twice
+    // the blocks that a range streams besides its own
+    int dev = 0, sms = 148;
+    if (cudaGetDevice(&dev) == cudaSuccess) cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
+    const long long ctas = (long long)tiles * bands * p.od.nsq;
+    const int want = (int)std::min<long long>(p.Pd, (8LL * sms + ctas - 1) / ctas);
+    const int jrange = std::min(p.Pd, std::max((p.Pd + want - 1) / want, 2 * (2 * p.tap_blocks - 1)));
+    const dim3 grid(tiles * ((p.Pd + jrange - 1) / jrange), bands, p.od.nsq);
+    const dim3 block(32, kGenWarps);
+    auto kernel = p.tap_blocks == 2 ? decompose_kernel<TQ, 2> : decompose_kernel<TQ, 1>;
+    kernel<<<grid, block, 0, st>>>(Q, out, p.od.crop, p.od.geo, p.od.T, p.tapw, p.Tstride, p.g.P, p.D, p.Pd, rw.layout,
+                                   p.g.Nu, rw.rowoff, rw.rowend, tiles, jrange);
     return cudaGetLastError();
 }
 

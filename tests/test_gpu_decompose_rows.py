@@ -2,10 +2,9 @@
 the generic kernel, bit for bit.
 
 All forms add the same products in the same order, so on the same Q they must
-agree exactly.  The staged kernel takes its crops by TMA, or (float32) by
-4-byte copies where Q is not 16-byte aligned or its rows are not whole 16-byte
-units; the generic kernel runs when the output is not 16-byte aligned, and is itself
-checked against the FP64 oracle here.  Shapes: squares whose shifted
+agree exactly.  The generic kernel runs when Q or the output is not 16-byte
+aligned or Q's rows are not whole 16-byte units, and is itself checked against
+the FP64 oracle here.  Shapes: squares whose shifted
 rows end on and beside a multiple of 16 columns, one to eight column segments,
 squares wider than 128 columns (several CTAs side by side), detectors of 1,
 31, 32, 33 and more rows, few and many views (ranges of decimated views), both
@@ -35,7 +34,7 @@ def _past_aligned(shape, dtype):
 
 
 def _forms(plan, Q):
-    """Decomposed data of the same Q: staged, staged from a misaligned Q, generic."""
+    """Decomposed data of the same Q: staged, from a misaligned Q, to a misaligned output."""
     off = _past_aligned(Q.shape, Q.dtype).copy_(Q)
     a, b = plan.decompose(Q), plan.decompose(off)
     c = plan.decompose(Q, _past_aligned(plan.decomposed_shape, torch.float32))
@@ -54,7 +53,7 @@ def _forms(plan, Q):
     (250, 256, 35, 40, 0, 4, 3.0),   # three CTAs side by side
     (200, 200, 64, 400, 1, 2, 4.0),  # ranges of decimated views
     (61, 64, 70, 900, 3, 2, 1.6),    # many views, ragged squares, a near source
-    (125, 125, 45, 60, 1, 3, 2.5),   # odd detector: 4-byte copies (81 to 128 columns a square)
+    (125, 125, 45, 60, 1, 3, 2.5),   # odd detector
     (61, 63, 45, 60, 1, 3, 2.5),     # narrower
     (150, 149, 40, 48, 0, 2, 4.0),   # wider than 128 columns
 ])
