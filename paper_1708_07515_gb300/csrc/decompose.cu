@@ -124,13 +124,19 @@ decompose_kernel(const TQ *__restrict__ Q, float *__restrict__ Sp, const int32_t
 // of 16-byte units long, which keeps those loads free of bank conflicts; the
 // crop's offset inside its aligned box is the same for all rows, so it picks
 // one of the unrolled bodies (a uniform branch).  Per view and lane: 5 (16-bit
-// Q: 3) loads, kCW lerps and kCW 2H tap FMAs.  A finished decimated view goes
-// through a per-warp transpose buffer, so that its rows leave in 64-byte runs.
+// Q: 3) loads, kCW lerps and kCW 2H tap FMAs.  A view's table entry is loaded
+// before the wait for its box (1-2 % faster than after it).  A finished decimated
+// view goes through a per-warp transpose buffer, so that its rows leave in
+// 64-byte runs, at a pointer that advances by one view per block (computed from
+// the view's number: 1 % slower at 512^3 f32, 3 % at 1024^3 bf16, 6 % with 2D taps).
 //
-// What bounds it: instruction issue, with the L2 -> shared traffic of the
-// crops (~14 |Q|) close behind.  The form before had lanes along the columns:
-// two scalar loads per sample, and columns in steps of 32 lanes (128 computed
-// for ~100 used).
+// What bounds it: instruction issue for 16-bit Q and 2D-tap filters; for float32
+// and the triangle the copies of the crops (~14 |Q| from L2) come close behind:
+// ring and copies alone take 0.90 ms of 1.08 at 512^3.  The form before had
+// lanes along the columns: two scalar loads per sample, and columns in steps of
+// 32 lanes (128 computed for ~100 used).  512^3 x 720 f32: 1.43 -> 1.08 ms with
+// the triangle, 2.30 -> 1.49 ms with 2D-tap filters; 1024^3 x 720 bf16 10.1 -> 6.9
+// ms; a 64-slice slab of 2000^3 from 720 bf16 views 7.1 -> 5.0 ms; 64^3 30 -> 8 us.
 //
 // Everything else a view needs -- shift fraction, tap weights, crop offset --
 // is one 16-byte entry of a per-CTA table in stream order (H = 2: 8 more bytes
@@ -142,9 +148,9 @@ constexpr int kTP = kCW + 4;  // row pitch of the transpose buffer (floats; 5 16
 constexpr int kDecMaxSegs = 8;  // column segments (consumer warps) per CTA; wider squares take several CTAs
 // ring shape per element type and tap length: slots of kG views, kStages slots.
 // float32, measured at 512^3: what counts is that the CTAs the registers allow
-// fit an SM (three with H = 1: 3 x 1 views 1.11 ms, 4 x 1 1.29; two with H = 2:
-// 4 x 1 1.61, 3 x 1 1.68).  16-bit, 2000^3: fewer waits, 2 x 3 views 5.1 ms, 3 x 2
-// 5.3, 2 x 2 5.4, 6 x 1 5.6.
+// fit an SM (three with H = 1: 4 x 1 views are 16 % slower than 3 x 1; two with
+// H = 2: 3 x 1 4 % slower than 4 x 1).  16-bit, 2000^3: fewer waits (3 x 2 views 4 %
+// slower than 2 x 3, 2 x 2 6 %, 6 x 1 10 %).
 template <typename TQ, int H>
 struct Ring {
     static constexpr int kG = sizeof(TQ) == 4 ? 1 : 3, kStages = sizeof(TQ) == 4 ? (H == 1 ? 3 : 4) : 2;
@@ -341,7 +347,7 @@ decompose_rows_kernel(const __grid_constant__ CUtensorMap tmap, float *__restric
     const int grp = warp / segs, seg = warp - grp * segs;
     const int rib = 32 * grp;  // first of the warp's rows in the band
     const int t0 = tc + seg * kCW;  // first of its columns
-    const int T = Tq[q];
+    const int ncol = Tq[q] - t0;  // columns of the warp that the square has
     float acc[2 * H][kCW];
 #pragma unroll
     for (int m = 0; m < 2 * H; ++m)
@@ -350,7 +356,7 @@ decompose_rows_kernel(const __grid_constant__ CUtensorMap tmap, float *__restric
     // coalesced store: lane writes 16 bytes at row rib + lane / 4 (+ 8, 16, 24), column t0 + 4 (lane % 4)
     const size_t vstride = (size_t)Nv * Tstride;
     const int srow = v0 + rib + (lane >> 2), scol = t0 + 4 * (lane & 3);
-    float *out = Sp + ((size_t)q * Pd * Nv + srow) * Tstride + scol;
+    float *o = Sp + ((size_t)((size_t)q * Pd + j0) * Nv + srow) * Tstride + scol;
     float *tb = tbuf + (size_t)warp * 32 * kTP;
     const uint32_t lane_addr = tma::smem_u32(ring) + (uint32_t)(ES * ((rib + lane) * Wc + seg * kCW));
     int slot = 0;
@@ -364,13 +370,6 @@ decompose_rows_kernel(const __grid_constant__ CUtensorMap tmap, float *__restric
     for (int jst = j0 - 2 * H + 1; jst < j1; ++jst, left = D) {
 #pragma unroll 1
         for (; left > 0; --left) {
-            if (w == 0) {
-                const bool ok = tma::mbar_wait_bounded(&full[slot], phase, kDecWaitNs);
-                if (!__all_sync(0xffffffffu, ok)) {
-                    if (lane == 0) atomicOr(status, 2);
-                    return;
-                }
-            }
             const float4 e = *pe++;
             float wt[2 * H];
             wt[0] = e.z;
@@ -379,6 +378,13 @@ decompose_rows_kernel(const __grid_constant__ CUtensorMap tmap, float *__restric
                 const float2 e2 = *pe2++;
                 wt[2] = e2.x;
                 wt[3] = e2.y;
+            }
+            if (w == 0) {
+                const bool ok = tma::mbar_wait_bounded(&full[slot], phase, kDecWaitNs);
+                if (!__all_sync(0xffffffffu, ok)) {
+                    if (lane == 0) atomicOr(status, 2);
+                    return;
+                }
             }
             view_any<TQ, H>(__float_as_int(e.y), a, e.x, wt, acc);
             a += tile_bytes;
@@ -394,18 +400,20 @@ decompose_rows_kernel(const __grid_constant__ CUtensorMap tmap, float *__restric
             }
         }
         if (jst >= j0) {  // decimated view jst is complete
+            // zero past the square's T columns
+#pragma unroll
+            for (int i = 0; i < kCW; ++i)
+                if (i >= ncol) acc[0][i] = 0.f;
             float4 *dst = (float4 *)(tb + lane * kTP);
 #pragma unroll
-            for (int i = 0; i < kCW; i += 4)
-                dst[i / 4] = make_float4(t0 + i < T ? acc[0][i] : 0.f, t0 + i + 1 < T ? acc[0][i + 1] : 0.f,
-                                         t0 + i + 2 < T ? acc[0][i + 2] : 0.f, t0 + i + 3 < T ? acc[0][i + 3] : 0.f);
+            for (int i = 0; i < kCW; i += 4) dst[i / 4] = make_float4(acc[0][i], acc[0][i + 1], acc[0][i + 2], acc[0][i + 3]);
             __syncwarp();
-            float *o = out + (size_t)jst * vstride;
 #pragma unroll
             for (int i = 0; i < 4; ++i) {
                 const float4 val = *(const float4 *)(tb + (8 * i + (lane >> 2)) * kTP + 4 * (lane & 3));
                 if (srow + 8 * i < rowend && scol < Tstride) *(float4 *)(o + (size_t)(8 * i) * Tstride) = val;
             }
+            o += vstride;
             __syncwarp();
         }
 #pragma unroll
@@ -453,8 +461,8 @@ cudaError_t try_rows(const PlanImpl &p, const TQ *Q, float *out, cudaStream_t st
     // order, so the same result) of at least 4 kLead decimated views, by a
     // model of the time: CTAs per SM times streamed views per CTA (8 more for
     // its set-up) over the share of its rate that an SM reaches with 1, 2 or 3
-    // resident CTAs (512^3 f32: 1.88, 1.29, 1.11 ms; a shorter table can let one
-    // more fit).  352^3 x 514, 352 CTAs: 3 ranges 285 us, 2 362.
+    // resident CTAs (512^3 f32; a shorter table can let one more fit).
+    // 352^3 x 514, 352 CTAs: 3 ranges 285 us, 2 362.
     const long long ctas = (long long)p.od.nsq * chunks * bands;
     int per_sm = 0;
     if (cudaDeviceGetAttribute(&per_sm, cudaDevAttrMaxSharedMemoryPerMultiprocessor, dev) != cudaSuccess) per_sm = 0;
