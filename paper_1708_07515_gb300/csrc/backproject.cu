@@ -659,7 +659,7 @@ bool pair_ring(int es, int zp, int rows, PairShape &s) {
 // The pair kernel's shape for `pairs` pairs of slices per column; false where
 // it does not apply (no window width, or windows too large to stage).  32
 // pairs per thread halve the per-view set-up and stage fewer margin rows
-// (512^3: 8.30 ms against 8.75 at 16), but need enough CTAs: 2 per SM, half as
+// (512^3: 8.35 ms against 8.77 at 16), but need enough CTAs: 2 per SM, half as
 // many of them (from 160^3 to 256^3 both take the same time within 4 %), and
 // they must not compute much more than they keep (the last slab's excess).
 bool pair_shape(const PlanImpl &p, const SquareSet &ss, bool direct, bool mirror, int pairs, PairShape &s) {
