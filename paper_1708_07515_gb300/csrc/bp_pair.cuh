@@ -127,9 +127,18 @@ __device__ __forceinline__ float rcp_approx(float x) {
     return y;
 }
 
-// barrier over all threads of the cluster, ordering their shared memory
+// Barriers over all threads of the cluster (ordering their shared memory) and
+// over the consumer warps.  Both take whole warps and have no time limit, so
+// each brings its warp together first: callers come from code that diverges
+// (one lane hands a slot back, ragged tiles store under a condition).
 __device__ __forceinline__ void cluster_sync() {
+    __syncwarp();
     asm volatile("barrier.cluster.arrive.release.aligned;\n\tbarrier.cluster.wait.acquire.aligned;" ::: "memory");
+}
+template <int THREADS>
+__device__ __forceinline__ void consumers_sync() {
+    __syncwarp();
+    asm volatile("bar.sync 1, %0;" ::"n"(THREADS) : "memory");
 }
 // two floats at this CTA's shared address a, of the cluster's CTA `rank`
 __device__ __forceinline__ float2 ld_cluster(uint32_t a, uint32_t rank) {
@@ -436,7 +445,6 @@ bp_pair_kernel(const __grid_constant__ CUtensorMap tmap, BpPairParams a) {
             for (int m = max(0, c - SLOTS); m < c; ++m)
                 tma::mbar_wait_bounded(&full[m % SLOTS], (uint32_t)((m / SLOTS) & 1), a.wait_ns);
         if constexpr (SPLIT) {
-            __syncwarp();
             cluster_sync();
             cluster_sync();
         }
@@ -508,7 +516,7 @@ bp_pair_kernel(const __grid_constant__ CUtensorMap tmap, BpPairParams a) {
     }
     if constexpr (SPLIT) {
         // every warp is done with the ring: it takes this CTA's sums [i][thread]
-        asm volatile("bar.sync 1, %0;" ::"n"(32 * kPairConsumers) : "memory");
+        consumers_sync<32 * kPairConsumers>();
         float2 *part = (float2 *)sm + threadIdx.x;
 #pragma unroll
         for (int i = 0; i < ZP; ++i) part[i * 32 * kPairConsumers] = acc[i];

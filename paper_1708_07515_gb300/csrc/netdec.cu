@@ -114,10 +114,16 @@ __host__ __device__ inline size_t net_smem(const NetChunk &c, int HD) {
            sizeof(float) * (size_t)c.J * kG + sizeof(float) * (size_t)HD;
 }
 
-// barrier 1: the consumer warps only (the producers run ahead)
-__device__ __forceinline__ void consumers_sync() { asm volatile("bar.sync 1, %0;" ::"n"(kNetThreads) : "memory"); }
+// barrier 1: the consumer warps only (the producers run ahead).  It takes whole
+// warps, and thread 0 comes from branches of its own (waits, MMAs): each
+// brings its warp together first.
+__device__ __forceinline__ void consumers_sync() {
+    __syncwarp();
+    asm volatile("bar.sync 1, %0;" ::"n"(kNetThreads) : "memory");
+}
 __device__ __forceinline__ bool consumers_and(bool v) {
     uint32_t r;
+    __syncwarp();
     asm volatile(
         "{\n\t.reg .pred p, q;\n\t"
         "setp.ne.u32 p, %1, 0;\n\t"

@@ -42,8 +42,10 @@ __host__ __device__ constexpr uint32_t idesc_bf16_f32(int M, int N) {
 }
 
 // Allocate ncols (a power of two >= 32) tensor-memory columns; the base
-// address lands in *slot (shared).  Warp-wide: one whole warp calls it.
+// address lands in *slot (shared).  Warp-wide: one whole warp calls it (and is
+// brought together first: its lane 0 may come from a branch of its own).
 __device__ __forceinline__ void alloc(uint32_t *slot, uint32_t ncols) {
+    __syncwarp();
     asm volatile("tcgen05.alloc.cta_group::1.sync.aligned.shared::cta.b32 [%0], %1;" ::"r"(
                      (uint32_t)__cvta_generic_to_shared(slot)),
                  "r"(ncols)
