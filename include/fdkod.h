@@ -456,7 +456,9 @@ void fdkod_batch_destroy(fdkod_batch_t *batch);
  * 32, 48, 64, 96, 128.  By default a plan takes the narrowest one that holds
  * every tile's footprint.  fdkod_set_tile(plan, cols) selects a wider one
  * (cols = 0: back to the default); results are the same bit for bit, only
- * the shared-memory layout (bank conflicts) and occupancy change.
+ * the shared-memory layout (bank conflicts) and occupancy change.  A launch
+ * whose staging ring does not fit with the selected width runs with the
+ * default one.
  * fdkod_get_tile returns the width in use (float32 windows) and the
  * narrowest valid one (0 when no window fits: the unstaged kernels run).
  * Call while no launch of the plan is in flight.  Errors: INVALID_ARG,

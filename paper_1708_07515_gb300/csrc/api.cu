@@ -75,6 +75,16 @@ void square_range(int q, int m, int N, int &i0, int &i1) {
 
 namespace fdkod {
 
+namespace {
+constexpr int kTileWidths[] = {32, 48, 64, 96, 128};  // the backprojection's instantiated windows
+}
+
+int window_width(int need) {
+    for (int w : kTileWidths)
+        if (need <= w) return w;
+    return 0;
+}
+
 // Staging window of the backprojection kernel: the largest column and row
 // extent any 16 x 16 x kZT voxel tile of this square set can touch in one
 // view, from an FP64 sweep over all tiles and views (column coordinate
@@ -128,11 +138,8 @@ void size_windows(const PlanImpl &p, SquareSet &ss, const double2 *cs) {
     const int need = (int)ceil(ext_t) + 8, need16 = (int)ceil(ext_t) + 12;
     ss.need = need;
     ss.need16 = need16;
-    ss.WdT = ss.WdT16 = 0;
-    for (int w : {128, 96, 64, 48, 32}) {
-        if (need <= w) ss.WdT = w;
-        if (need16 <= w) ss.WdT16 = w;
-    }
+    ss.WdT = window_width(need);
+    ss.WdT16 = window_width(need16);
 }
 
 void triangle_taps(int D, double *h) {
@@ -601,28 +608,19 @@ void fdkod_batch_destroy(fdkod_batch_t *batch) {
     delete batch;
 }
 
-namespace {
-constexpr int kTileWidths[] = {32, 48, 64, 96, 128};  // the backprojection's instantiated windows
-int auto_width(int need) {
-    for (int w : kTileWidths)
-        if (need <= w) return w;
-    return 0;
-}
-}  // namespace
-
 int fdkod_set_tile(fdkod_plan_t *plan, int window_cols) {
     if (!plan || window_cols < 0) return FDKOD_ERR_INVALID_ARG;
     fdkod::SquareSet &ss = plan->impl.od;
     if (window_cols == 0) {
-        ss.WdT = auto_width(ss.need);
-        ss.WdT16 = auto_width(ss.need16);
+        ss.WdT = fdkod::window_width(ss.need);
+        ss.WdT16 = fdkod::window_width(ss.need16);
         return FDKOD_OK;
     }
     bool instantiated = false;
-    for (int w : kTileWidths) instantiated = instantiated || w == window_cols;
+    for (int w : fdkod::kTileWidths) instantiated = instantiated || w == window_cols;
     if (!instantiated || window_cols < ss.need || ss.Rw > 256) return FDKOD_ERR_UNSUPPORTED;
     ss.WdT = window_cols;
-    ss.WdT16 = window_cols >= ss.need16 ? window_cols : auto_width(ss.need16);
+    ss.WdT16 = window_cols >= ss.need16 ? window_cols : fdkod::window_width(ss.need16);
     return FDKOD_OK;
 }
 
@@ -630,6 +628,6 @@ int fdkod_get_tile(const fdkod_plan_t *plan, int *window_cols, int *min_cols) {
     if (!plan) return FDKOD_ERR_INVALID_ARG;
     const fdkod::SquareSet &ss = plan->impl.od;
     if (window_cols) *window_cols = ss.WdT;
-    if (min_cols) *min_cols = auto_width(ss.need);
+    if (min_cols) *min_cols = fdkod::window_width(ss.need);
     return FDKOD_OK;
 }

@@ -656,18 +656,16 @@ bool pair_ring(int es, int zp, int rows, PairShape &s) {
     return pair_smem(es, 1, 3, ts) <= budget;
 }
 
-// The pair kernel's shape for `pairs` pairs of slices per column; false where
-// it does not apply (no window width, or windows too large to stage).  32
+// What rounds in the pair kernel's shape for `pairs` pairs of slices per column
+// (slices per slab, CTAs that share the views), with the ring of s.WD columns;
+// false where the windows are too large to stage.  32
 // pairs per thread halve the per-view set-up and stage fewer margin rows
 // (512^3: 8.35 ms against 8.77 at 16), but need enough CTAs: 2 per SM, half as
 // many of them (from 160^3 to 256^3 both take the same time within 4 %), and
 // they must not compute much more than they keep (the last slab's excess).
-bool pair_shape(const PlanImpl &p, const SquareSet &ss, bool direct, bool mirror, int pairs, PairShape &s) {
+bool pair_slabs(const PlanImpl &p, const SquareSet &ss, bool direct, bool mirror, int pairs, PairShape &s) {
     const int es = (direct && p.qtype != FDKOD_F32) ? 2 : 4;
-    s.WD = es == 4 ? ss.WdT : ss.WdT16;
-    s.mirror = mirror;
     s.nsplit = 1;
-    if (s.WD == 0) return false;
     const long long tiles = (long long)ss.nsq * ss.tiles_per_side * ss.tiles_per_side;
     int dev = 0, sms = 148;
     if (cudaGetDevice(&dev) == cudaSuccess) cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
@@ -693,6 +691,23 @@ bool pair_shape(const PlanImpl &p, const SquareSet &ss, bool direct, bool mirror
         if (s.nsplit == 1 && ctas * 4 <= 5 * slots && views >= 32) s.nsplit = 2;
     }
     return ss.Rw2 <= 256 && pair_ring(es, 16, ss.Rw2, s);
+}
+
+// The pair kernel's shape; false where it does not apply (no window width, or
+// windows too large to stage).  The narrowest window decides what rounds, so
+// that a wider one chosen by fdkod_set_tile gives the same result; it is
+// taken where the shape has a ring of its width (512^3: up to 64 columns with
+// 32 slices per slab; 16 slices would fit 96, and round otherwise).
+bool pair_shape(const PlanImpl &p, const SquareSet &ss, bool direct, bool mirror, int pairs, PairShape &s) {
+    const int es = (direct && p.qtype != FDKOD_F32) ? 2 : 4;
+    s.mirror = mirror;
+    s.WD = window_width(es == 4 ? ss.need : ss.need16);
+    if (s.WD == 0 || !pair_slabs(p, ss, direct, mirror, pairs, s)) return false;
+    PairShape wide = s;
+    wide.WD = es == 4 ? ss.WdT : ss.WdT16;
+    if (wide.WD != s.WD && pair_ring(es, s.zp, s.zp == 32 ? ss.Rw : ss.Rw2, wide) && (s.zp == 16 || wide.vps == 2))
+        s = wide;
+    return true;
 }
 
 // The staged kernel over the slices of b (mirror: over the whole detector and

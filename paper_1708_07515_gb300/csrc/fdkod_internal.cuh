@@ -135,6 +135,9 @@ cudaError_t ensure_smem(size_t bytes) {
     return e;
 }
 
+// host: the narrowest instantiated window of at least `need` columns (0: none)
+int window_width(int need);
+
 // host: backprojection staging windows of a square set (cs = cos/sin per view)
 void size_windows(const PlanImpl &p, SquareSet &ss, const double2 *cs);
 
