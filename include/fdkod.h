@@ -490,6 +490,27 @@ int fdkod_get_tile(const fdkod_plan_t *plan, int *window_cols, int *min_cols);
 #define FDKOD_TEST_SMALL_WINDOW 2
 int fdkod_set_test_fault(fdkod_plan_t *plan, int kind, int64_t wait_ns);
 
+/*
+ * The kernel forms this plan's calls take, for tests that have to know which
+ * one they cover (the paper has no counterpart).  They follow from sizes and
+ * the device alone; 16-byte aligned buffers are assumed.  nz = 0: the whole
+ * volume, else fdkod_backproject_slab of nz slices.
+ *  bp_slices: slices per slab of the staged backprojection, two slabs per CTA
+ *    (0: the staged kernel does not apply); bp_columns: window columns;
+ *    bp_views, bp_slots: views per ring slot, slots; bp_split: CTAs of a
+ *    cluster that share the views (1: none).
+ *  dec_warps: consumer warps per CTA of the staged decomposition (0: D = 1, a
+ *    learned decimation, or the staged kernel does not apply); dec_ranges:
+ *    ranges of decimated views; dec_resident: CTAs per SM that the choice of
+ *    ranges reckons with; dec_occupancy: the runtime's count of them.
+ * Host only.  Errors: INVALID_ARG (null pointers, nz out of range), CUDA.
+ */
+typedef struct {
+    int32_t bp_slices, bp_columns, bp_views, bp_slots, bp_split;
+    int32_t dec_warps, dec_ranges, dec_resident, dec_occupancy;
+} fdkod_forms;
+int fdkod_get_forms(const fdkod_plan_t *plan, int nz, fdkod_forms *out);
+
 /* Static message for a status code. */
 const char *fdkod_strerror(int status);
 

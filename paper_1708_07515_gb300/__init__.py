@@ -26,6 +26,7 @@ from .fdkod import (  # noqa: F401
     fdkod_get_bounds,
     fdkod_get_decimation_net,
     fdkod_get_decimation_taps,
+    fdkod_get_forms,
     fdkod_net_adjoint,
     fdkod_net_backward,
     fdkod_noalloc_device_status,

@@ -556,6 +556,13 @@ int fdkod_set_test_fault(fdkod_plan_t *plan, int kind, int64_t wait_ns) {
     return FDKOD_OK;
 }
 
+int fdkod_get_forms(const fdkod_plan_t *plan, int nz, fdkod_forms *out) {
+    if (!plan || !out || nz < 0 || nz > plan->impl.g.N) return FDKOD_ERR_INVALID_ARG;
+    *out = fdkod_forms{};
+    fdkod::backproject_form(plan->impl, nz, *out);
+    return cuda_status(fdkod::decompose_form(plan->impl, *out));
+}
+
 const char *fdkod_strerror(int status) {
     switch (status) {
         case FDKOD_OK: return "ok";

@@ -777,6 +777,18 @@ int pair_slab(const PlanImpl &p, const SquareSet &ss, bool direct) {
     return pair_shape(p, ss, direct, true, (p.g.N + 1) / 2, s) ? s.zp : 16;
 }
 
+void backproject_form(const PlanImpl &p, int nz, fdkod_forms &f) {
+    const bool direct = p.D == 1, whole = nz == 0 || nz == p.g.N;
+    const int es = (direct && p.qtype != FDKOD_F32) ? 2 : 4, pairs = ((whole ? p.g.N : nz) + 1) / 2;
+    PairShape s;
+    if ((direct && ((size_t)p.g.Nu * es) % 16 != 0) || !pair_shape(p, p.od, direct, whole, pairs, s)) return;
+    f.bp_slices = s.zp;
+    f.bp_columns = s.WD;
+    f.bp_views = s.vps;
+    f.bp_slots = s.slots;
+    f.bp_split = s.nsplit;
+}
+
 cudaError_t launch_backproject(const PlanImpl &p, const SquareSet &ss, bool direct, const void *src, float *vol,
                                cudaStream_t st, Band b) {
     const bool whole = b.row0 == 0 && (b.nrows < 0 || b.nrows == p.g.Nv) && b.zoff == 0 && (b.nz < 0 || b.nz == p.g.N);

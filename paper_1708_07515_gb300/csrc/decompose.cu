@@ -431,31 +431,39 @@ struct Rows {
     int layout, rowoff, rowend;
 };
 
-// Applies when Q and S' are 16-byte aligned (vector stores), Q's rows are whole
-// 16-byte units, D <= 128 and the ring plus the stream tables fit in shared
-// memory.
+// Shape of the staged kernel's launch over `nrows` detector rows.
+struct RowsShape {
+    int Wc, tile_stride;              // columns of a crop box; elements per staged box
+    int segs, chunks, warps;          // column segments per CTA, CTAs side by side, consumer warps
+    int band, bands;                  // rows per CTA, bands of rows
+    int jrange, resident;             // decimated views per CTA; CTAs that an SM holds at once
+    size_t smem;
+};
+
+// False where the staged kernel does not apply: Q's rows must be whole 16-byte
+// units, D <= 128 and the ring plus the stream tables fit in shared memory.
 template <typename TQ, int H>
-cudaError_t try_rows(const PlanImpl &p, const TQ *Q, float *out, cudaStream_t st, Rows rw, bool &launched) {
-    launched = false;
+bool rows_shape(const PlanImpl &p, int nrows, RowsShape &r) {
     constexpr int kAlign = 16 / (int)sizeof(TQ);
-    if ((p.g.Nu % kAlign) != 0 || ((uintptr_t)Q & 15) != 0 || ((uintptr_t)out & 15) != 0) return cudaSuccess;
-    if (p.D > kMaxTapD) return cudaSuccess;
+    if ((p.g.Nu % kAlign) != 0 || p.D > kMaxTapD) return false;
     const int all = (p.Tstride + kCW - 1) / kCW;  // column segments of a square
-    const int chunks = (all + kDecMaxSegs - 1) / kDecMaxSegs, segs = (all + chunks - 1) / chunks;
+    r.chunks = (all + kDecMaxSegs - 1) / kDecMaxSegs;
+    r.segs = (all + r.chunks - 1) / r.chunks;
     // the segments' columns + neighbour + crop offset, whole 16-byte units, an odd number of them
-    int Wc = (std::min(p.od.Tmax, segs * kCW) + 1 + (kAlign - 1) + (kAlign - 1)) & ~(kAlign - 1);
-    if ((Wc / kAlign) % 2 == 0) Wc += kAlign;
-    const int nrows = rw.rowend - rw.rowoff;
+    r.Wc = (std::min(p.od.Tmax, r.segs * kCW) + 1 + (kAlign - 1) + (kAlign - 1)) & ~(kAlign - 1);
+    if ((r.Wc / kAlign) % 2 == 0) r.Wc += kAlign;
     // narrow squares: several row groups per CTA, at least four consumer warps
-    const int groups = std::max(1, std::min((nrows + 31) / 32, 4 / segs));
-    const int warps = segs * groups, band = 32 * groups;
-    const int bands = (nrows + band - 1) / band;
-    const int tile_stride = (band * Wc + 63) & ~63;  // elements; 128-byte multiple for every type
+    const int groups = std::max(1, std::min((nrows + 31) / 32, 4 / r.segs));
+    r.warps = r.segs * groups;
+    r.band = 32 * groups;
+    r.bands = (nrows + r.band - 1) / r.band;
+    r.tile_stride = (r.band * r.Wc + 63) & ~63;  // elements; 128-byte multiple for every type
     int dev = 0, sms = 148;
     if (cudaGetDevice(&dev) == cudaSuccess) cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
     constexpr int kLead = 2 * H - 1;  // a range streams kLead D - 1 views besides its own
     auto smem_of = [&](int jr) {
-        return dec_smem((int)sizeof(TQ), Ring<TQ, H>::kStages * Ring<TQ, H>::kG, tile_stride, warps, (jr + kLead) * p.D - 1, H);
+        return dec_smem((int)sizeof(TQ), Ring<TQ, H>::kStages * Ring<TQ, H>::kG, r.tile_stride, r.warps,
+                        (jr + kLead) * p.D - 1, H);
     };
     // The decimated views are split into ranges (the same sums in the same
     // order, so the same result) of at least 4 kLead decimated views, by a
@@ -463,41 +471,66 @@ cudaError_t try_rows(const PlanImpl &p, const TQ *Q, float *out, cudaStream_t st
     // its set-up) over the share of its rate that an SM reaches with 1, 2 or 3
     // resident CTAs (512^3 f32; a shorter table can let one more fit).
     // 352^3 x 514, 352 CTAs: 3 ranges 285 us, 2 362.
-    const long long ctas = (long long)p.od.nsq * chunks * bands;
+    const long long ctas = (long long)p.od.nsq * r.chunks * r.bands;
     int per_sm = 0;
     if (cudaDeviceGetAttribute(&per_sm, cudaDevAttrMaxSharedMemoryPerMultiprocessor, dev) != cudaSuccess) per_sm = 0;
-    int jrange = p.Pd;
+    r.jrange = p.Pd;
+    r.resident = 0;
     double best = 0.0;
-    for (int r = 1; r <= 64; ++r) {
-        const int jr = (p.Pd + r - 1) / r;
-        if (r > 1 && jr < 4 * kLead) break;
+    for (int n = 1; n <= 64; ++n) {
+        const int jr = (p.Pd + n - 1) / n;
+        if (n > 1 && jr < 4 * kLead) break;
         const long long per = (ctas * ((p.Pd + jr - 1) / jr) + sms - 1) / sms;  // CTAs per SM
         const long long fit = std::min<long long>(H == 1 ? 3 : 2, (long long)(per_sm / (smem_of(jr) + 2048)));
         const double rate[] = {0.1, 0.59, 0.86, 1.0};
         const double cost = (double)per * ((jr + kLead) * p.D + 8) / rate[std::max(0LL, std::min(fit, per))];
-        if (r == 1 || cost < best) {
+        if (n == 1 || cost < best) {
             best = cost;
-            jrange = jr;
+            r.jrange = jr;
+            r.resident = (int)fit;
         }
     }
-    const size_t smem = smem_of(jrange);
-    if (smem > 200 * 1024 || bands > 65535) return cudaSuccess;
+    r.smem = smem_of(r.jrange);
+    return r.smem <= 200 * 1024 && r.bands <= 65535;
+}
+
+// The staged kernel, where it applies and Q and S' are 16-byte aligned (bulk
+// copies, vector stores).
+template <typename TQ, int H>
+cudaError_t try_rows(const PlanImpl &p, const TQ *Q, float *out, cudaStream_t st, Rows rw, bool &launched) {
+    launched = false;
+    RowsShape r;
+    if (((uintptr_t)Q & 15) != 0 || ((uintptr_t)out & 15) != 0) return cudaSuccess;
+    if (!rows_shape<TQ, H>(p, rw.rowend - rw.rowoff, r)) return cudaSuccess;
     CUtensorMap map;
     const uint64_t dims[3] = {(uint64_t)p.g.Nu, (uint64_t)rw.layout, (uint64_t)p.g.P};
     const uint64_t strides[2] = {(uint64_t)p.g.Nu * sizeof(TQ), (uint64_t)p.g.Nu * rw.layout * sizeof(TQ)};
-    const uint32_t box[3] = {(uint32_t)Wc, (uint32_t)band, 1u};
+    const uint32_t box[3] = {(uint32_t)r.Wc, (uint32_t)r.band, 1u};
     const CUtensorMapDataType dt = sizeof(TQ) == 4 ? CU_TENSOR_MAP_DATA_TYPE_FLOAT32
                                    : (std::is_same<TQ, __half>::value ? CU_TENSOR_MAP_DATA_TYPE_FLOAT16
                                                                       : CU_TENSOR_MAP_DATA_TYPE_BFLOAT16);
     if (encode_map_3d(&map, dt, Q, dims, strides, box) != cudaSuccess) return cudaSuccess;
     launched = true;
-    cudaError_t e = ensure_smem<decompose_rows_kernel<TQ, H>>(smem);
+    cudaError_t e = ensure_smem<decompose_rows_kernel<TQ, H>>(r.smem);
     if (e != cudaSuccess) return e;
-    dim3 grid(p.od.nsq * chunks, bands, (p.Pd + jrange - 1) / jrange);
-    decompose_rows_kernel<TQ, H><<<grid, 32 * (warps + 1), smem, st>>>(
-        map, out, p.od.crop, p.od.geo, p.od.T, p.tapw, p.status, p.Tstride, p.g.P, p.D, p.Pd, rw.layout, Wc,
-        tile_stride, segs, chunks, rw.rowoff, rw.rowend, jrange);
+    dim3 grid(p.od.nsq * r.chunks, r.bands, (p.Pd + r.jrange - 1) / r.jrange);
+    decompose_rows_kernel<TQ, H><<<grid, 32 * (r.warps + 1), r.smem, st>>>(
+        map, out, p.od.crop, p.od.geo, p.od.T, p.tapw, p.status, p.Tstride, p.g.P, p.D, p.Pd, rw.layout, r.Wc,
+        r.tile_stride, r.segs, r.chunks, rw.rowoff, rw.rowend, r.jrange);
     return cudaGetLastError();
+}
+
+template <typename TQ, int H>
+cudaError_t form_t(const PlanImpl &p, fdkod_forms &f) {
+    RowsShape r;
+    if (!rows_shape<TQ, H>(p, p.g.Nv, r)) return cudaSuccess;
+    f.dec_warps = r.warps;
+    f.dec_ranges = (p.Pd + r.jrange - 1) / r.jrange;
+    f.dec_resident = r.resident;
+    cudaError_t e = ensure_smem<decompose_rows_kernel<TQ, H>>(r.smem);
+    if (e != cudaSuccess) return e;
+    return cudaOccupancyMaxActiveBlocksPerMultiprocessor(&f.dec_occupancy, decompose_rows_kernel<TQ, H>,
+                                                         32 * (r.warps + 1), r.smem);
 }
 
 template <typename TQ>
@@ -538,6 +571,17 @@ cudaError_t launch_decompose(const PlanImpl &p, const void *Q, float *out, cudaS
         case FDKOD_F32: return launch_t(p, (const float *)Q, out, st, rw);
         case FDKOD_BF16: return launch_t(p, (const __nv_bfloat16 *)Q, out, st, rw);
         case FDKOD_F16: return launch_t(p, (const __half *)Q, out, st, rw);
+    }
+    return cudaErrorInvalidValue;
+}
+
+cudaError_t decompose_form(const PlanImpl &p, fdkod_forms &f) {
+    if (p.D == 1 || p.net) return cudaSuccess;
+    const bool wide = p.tap_blocks == 2;
+    switch (p.qtype) {
+        case FDKOD_F32: return wide ? form_t<float, 2>(p, f) : form_t<float, 1>(p, f);
+        case FDKOD_BF16: return wide ? form_t<__nv_bfloat16, 2>(p, f) : form_t<__nv_bfloat16, 1>(p, f);
+        case FDKOD_F16: return wide ? form_t<__half, 2>(p, f) : form_t<__half, 1>(p, f);
     }
     return cudaErrorInvalidValue;
 }

@@ -183,6 +183,11 @@ cudaError_t launch_backproject_pairs(const PlanImpl &p, const SquareSet &ss, boo
 // the pairs start at a multiple of it, so that they round as the whole launch
 int pair_slab(const PlanImpl &p, const SquareSet &ss, bool direct);
 
+// host: what fdkod_get_forms reports of each stage (fields of kernels that do
+// not apply are left alone)
+void backproject_form(const PlanImpl &p, int nz, fdkod_forms &f);
+cudaError_t decompose_form(const PlanImpl &p, fdkod_forms &f);
+
 // A batch of plans backprojected by one persistent launch (backproject.cu):
 // per plan its FDK-OD source (Q when D = 1, else the decomposed data) and
 // volume.  supported = false (and *out null) when a plan cannot take the

@@ -39,6 +39,11 @@ class PlanInfo(ctypes.Structure):
                 ("device_bytes", ctypes.c_int64)]
 
 
+class Forms(ctypes.Structure):
+    _fields_ = [(f, ctypes.c_int32) for f in ("bp_slices", "bp_columns", "bp_views", "bp_slots", "bp_split",
+                                              "dec_warps", "dec_ranges", "dec_resident", "dec_occupancy")]
+
+
 def lib_path() -> str:
     return _LIB_PATH
 
@@ -71,6 +76,7 @@ def load():
                 "fdkod_backproject_noalloc": (i, [ctypes.POINTER(Geometry), i, i, vp, vp, u]),
                 "fdkod_noalloc_device_status": (i, [u]),
                 "fdkod_set_test_fault": (i, [vp, i, ctypes.c_int64]),
+                "fdkod_get_forms": (i, [vp, i, ctypes.POINTER(Forms)]),
                 "fdkod_get_bounds": (i, [vp, vp, vp, vp, vp, vp, vp]),
                 "fdkod_last_device_status": (i, [vp, u]),
                 "fdkod_strerror": (ctypes.c_char_p, [i]),
@@ -219,6 +225,14 @@ FDKOD_TEST_NONE, FDKOD_TEST_SKIP_COPY, FDKOD_TEST_SMALL_WINDOW = 0, 1, 2
 def fdkod_set_test_fault(plan: int, kind: int, wait_ns: int = 0) -> None:
     """Test hook of the backprojection's failure paths (see include/fdkod.h)."""
     _check(load().fdkod_set_test_fault(plan, int(kind), int(wait_ns)), "fdkod_set_test_fault")
+
+
+def fdkod_get_forms(plan: int, nz: int = 0) -> dict:
+    """The kernel forms the plan's calls take (see include/fdkod.h): the whole
+    volume, or a slab of nz slices."""
+    f = Forms()
+    _check(load().fdkod_get_forms(plan, int(nz), ctypes.byref(f)), "fdkod_get_forms")
+    return {name: getattr(f, name) for name, _ in Forms._fields_}
 
 
 def fdkod_get_bounds(plan: int, n_squares: int, P: int) -> dict:
