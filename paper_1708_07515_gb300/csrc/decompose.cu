@@ -145,7 +145,17 @@ decompose_kernel(const TQ *__restrict__ Q, float *__restrict__ Sp, const int32_t
 
 constexpr int kCW = 16;       // shifted columns per warp
 constexpr int kTP = kCW + 4;  // row pitch of the transpose buffer (floats; 5 16-byte units: no conflicts)
-constexpr int kDecMaxSegs = 8;  // column segments (consumer warps) per CTA; wider squares take several CTAs
+// Column segments (consumer warps) per CTA; wider squares take several CTAs.
+// With the producer 8 warps, so that three CTAs (H = 1) or two (H = 2) share an
+// SM's registers; nine warps leave room for two and one.  Squares of 113-128
+// columns, 8 segments in one CTA against 4 + 4: 280^3 x 400 f32 156 -> 115 us,
+// 300^3 x 420 2D taps 244 -> 177 us, 600^3 x 720 f32 1704 -> 1581 us.
+constexpr int kDecMaxSegs = 7;
+// Warps that the registers of an SM hold (80 and 128 a thread, see the kernel)
+template <int H>
+constexpr int kDecSmWarps = H == 1 ? 24 : 16;
+static_assert((kDecMaxSegs + 1) * 3 <= kDecSmWarps<1> && (kDecMaxSegs + 1) * 2 <= kDecSmWarps<2>,
+              "whole CTAs fill an SM's registers");
 // ring shape per element type and tap length: slots of kG views, kStages slots.
 // float32, measured at 512^3: what counts is that the CTAs the registers allow
 // fit an SM (three with H = 1: 4 x 1 views are 16 % slower than 3 x 1; two with
@@ -155,7 +165,11 @@ template <typename TQ, int H>
 struct Ring {
     static constexpr int kG = sizeof(TQ) == 4 ? 1 : 3, kStages = sizeof(TQ) == 4 ? (H == 1 ? 3 : 4) : 2;
 };
-constexpr int kRingSlack = 128;  // the last segment's loads run up to 16 bytes past a row's end
+// The last segment's 16-byte loads run past a row's end where the square uses
+// few of its columns: up to 32 bytes (float32, one or five columns used, the crop
+// three columns into its box: 20 columns read, 12 staged), in the last row of
+// the last box past the ring.
+constexpr int kRingSlack = 128;
 constexpr uint64_t kDecWaitNs = 2000000000ull;
 
 // Per-CTA tables over the stream of decimated views j0 .. j1 - 1: position
@@ -276,7 +290,7 @@ __host__ __device__ inline size_t dec_smem(int es, int stages, int tile_stride, 
 // the thread bound only sets the register limit: 80 (24 warps per SM) for the
 // two running sums of the triangle, 128 (16 warps) for the four of 2D-tap filters
 template <typename TQ, int H>
-__global__ void __launch_bounds__(H == 1 ? 768 : 512, 1)
+__global__ void __launch_bounds__(32 * kDecSmWarps<H>, 1)
 decompose_rows_kernel(const __grid_constant__ CUtensorMap tmap, float *__restrict__ Sp,
                       const int32_t *__restrict__ crop, const GeomEntry *__restrict__ geo,
                       const int32_t *__restrict__ Tq, const float4 *__restrict__ tapw, int *status, int Tstride,
@@ -406,7 +420,8 @@ decompose_rows_kernel(const __grid_constant__ CUtensorMap tmap, float *__restric
                 if (i >= ncol) acc[0][i] = 0.f;
             float4 *dst = (float4 *)(tb + lane * kTP);
 #pragma unroll
-            for (int i = 0; i < kCW; i += 4) dst[i / 4] = make_float4(acc[0][i], acc[0][i + 1], acc[0][i + 2], acc[0][i + 3]);
+            for (int i = 0; i < kCW; i += 4)
+                dst[i / 4] = make_float4(acc[0][i], acc[0][i + 1], acc[0][i + 2], acc[0][i + 3]);
             __syncwarp();
 #pragma unroll
             for (int i = 0; i < 4; ++i) {
@@ -423,6 +438,14 @@ decompose_rows_kernel(const __grid_constant__ CUtensorMap tmap, float *__restric
             acc[2 * H - 1][i] = 0.f;
         }
     }
+}
+
+// Share of its rate that an SM reaches with w resident consumer warps (512^3
+// f32: 7, 14 and 21 of them)
+double sm_rate(double w) {
+    return w <= 7.0    ? 0.59 * w / 7.0
+           : w <= 14.0 ? 0.59 + 0.27 * (w - 7.0) / 7.0
+                       : std::min(1.0, 0.86 + 0.14 * (w - 14.0) / 7.0);
 }
 
 // Rows of a launch: the arrays hold `layout` rows per view (S' included)
@@ -467,31 +490,37 @@ bool rows_shape(const PlanImpl &p, int nrows, RowsShape &r) {
     };
     // The decimated views are split into ranges (the same sums in the same
     // order, so the same result) of at least 4 kLead decimated views, by a
-    // model of the time: CTAs per SM times streamed views per CTA (8 more for
-    // its set-up) over the share of its rate that an SM reaches with 1, 2 or 3
-    // resident CTAs (512^3 f32; a shorter table can let one more fit).
-    // 352^3 x 514, 352 CTAs: 3 ranges 285 us, 2 362.
+    // model of the time of the SM with the most CTAs: as many of them at once
+    // as its registers and shared memory hold (a shorter table can let one more
+    // fit), wave after wave, each wave the views its CTAs stream at the rate
+    // of its resident warps; and a fifth of a CTA more, for CTAs that don't
+    // end together.  Of 148 shapes (37 sizes from 64^3 to 1000^3, float32 and
+    // bfloat16, both tap lengths) measured with 1 to 64 ranges, the choice is
+    // 0.4 % behind the best one in the mean.
     const long long ctas = (long long)p.od.nsq * r.chunks * r.bands;
     int per_sm = 0;
-    if (cudaDeviceGetAttribute(&per_sm, cudaDevAttrMaxSharedMemoryPerMultiprocessor, dev) != cudaSuccess) per_sm = 0;
-    r.jrange = p.Pd;
+    if (cudaDeviceGetAttribute(&per_sm, cudaDevAttrMaxSharedMemoryPerMultiprocessor, dev) != cudaSuccess) return false;
     r.resident = 0;
     double best = 0.0;
     for (int n = 1; n <= 64; ++n) {
         const int jr = (p.Pd + n - 1) / n;
         if (n > 1 && jr < 4 * kLead) break;
-        const long long per = (ctas * ((p.Pd + jr - 1) / jr) + sms - 1) / sms;  // CTAs per SM
-        const long long fit = std::min<long long>(H == 1 ? 3 : 2, (long long)(per_sm / (smem_of(jr) + 2048)));
-        const double rate[] = {0.1, 0.59, 0.86, 1.0};
-        const double cost = (double)per * ((jr + kLead) * p.D + 8) / rate[std::max(0LL, std::min(fit, per))];
-        if (n == 1 || cost < best) {
+        const size_t smem = smem_of(jr);
+        const int fit = std::min(kDecSmWarps<H> / (r.warps + 1), (int)((size_t)per_sm / (smem + 2048)));
+        if (fit < 1 || smem > 200 * 1024) continue;
+        const long long per = (ctas * ((p.Pd + jr - 1) / jr) + sms - 1) / sms;  // CTAs of an SM, at most
+        const long long rest = per % fit;
+        const double last = rest ? (double)rest / sm_rate((double)rest * r.warps) : 0.0;
+        const double waves = (double)(per - rest) / sm_rate((double)fit * r.warps) + last;
+        const double cost = (waves + 0.2) * ((jr + kLead) * p.D + 1);
+        if (r.resident == 0 || cost < best) {
             best = cost;
             r.jrange = jr;
-            r.resident = (int)fit;
+            r.resident = fit;
+            r.smem = smem;
         }
     }
-    r.smem = smem_of(r.jrange);
-    return r.smem <= 200 * 1024 && r.bands <= 65535;
+    return r.resident > 0 && r.bands <= 65535;
 }
 
 // The staged kernel, where it applies and Q and S' are 16-byte aligned (bulk
