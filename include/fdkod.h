@@ -499,10 +499,11 @@ int fdkod_set_test_fault(fdkod_plan_t *plan, int kind, int64_t wait_ns);
  *    (0: the staged kernel does not apply); bp_columns: window columns;
  *    bp_views, bp_slots: views per ring slot, slots; bp_split: CTAs of a
  *    cluster that share the views (1: none).
- *  dec_warps: consumer warps per CTA of the staged decomposition (0: D = 1, a
- *    learned decimation, or the staged kernel does not apply); dec_ranges:
- *    ranges of decimated views; dec_resident: CTAs per SM that the choice of
- *    ranges reckons with; dec_occupancy: the runtime's count of them.
+ *  dec_warps: consumer warps per CTA of the staged decomposition (0: the
+ *    generic kernel); dec_ranges: ranges of decimated views of either;
+ *    dec_resident: CTAs per SM that the staged kernel's choice of ranges
+ *    reckons with; dec_occupancy: the runtime's count of them.  All 0 for
+ *    D = 1 and with a learned decimation.
  * Host only.  Errors: INVALID_ARG (null pointers, nz out of range), CUDA.
  */
 typedef struct {

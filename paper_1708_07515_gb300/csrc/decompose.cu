@@ -489,22 +489,22 @@ bool rows_shape(const PlanImpl &p, int nrows, RowsShape &r) {
                         (jr + kLead) * p.D - 1, H);
     };
     // The decimated views are split into ranges (the same sums in the same
-    // order, so the same result) of at least 4 kLead decimated views, by a
-    // model of the time of the SM with the most CTAs: as many of them at once
-    // as its registers and shared memory hold (a shorter table can let one more
-    // fit), wave after wave, each wave the views its CTAs stream at the rate
-    // of its resident warps; and a fifth of a CTA more, for CTAs that don't
-    // end together.  Of 148 shapes (37 sizes from 64^3 to 1000^3, float32 and
-    // bfloat16, both tap lengths) measured with 1 to 64 ranges, the choice is
-    // 0.4 % behind the best one in the mean.
+    // order, so the same result), by a model of the time of the SM with the
+    // most CTAs: as many of them at once as its registers and shared memory
+    // hold (a shorter table can let one more fit), wave after wave, each wave
+    // the views its CTAs stream at the rate of its resident warps; and a fifth
+    // of a CTA more, for CTAs that don't end together.  Of 148 shapes (37 sizes
+    // from 64^3 to 1000^3, float32 and bfloat16, both tap lengths) measured with
+    // 1 to 64 ranges of at least 4 kLead views, the choice is 0.4 % behind the
+    // best one in the mean.  Small grids take ranges down to one view (of 4
+    // kLead or more: 128^3 x 128 bf16, D = 8, 2D taps 58 us against 19).
     const long long ctas = (long long)p.od.nsq * r.chunks * r.bands;
     int per_sm = 0;
     if (cudaDeviceGetAttribute(&per_sm, cudaDevAttrMaxSharedMemoryPerMultiprocessor, dev) != cudaSuccess) return false;
     r.resident = 0;
     double best = 0.0;
-    for (int n = 1; n <= 64; ++n) {
+    for (int n = 1; n <= std::min(64, p.Pd); ++n) {
         const int jr = (p.Pd + n - 1) / n;
-        if (n > 1 && jr < 4 * kLead) break;
         const size_t smem = smem_of(jr);
         const int fit = std::min(kDecSmWarps<H> / (r.warps + 1), (int)((size_t)per_sm / (smem + 2048)));
         if (fit < 1 || smem > 200 * 1024) continue;
@@ -549,10 +549,42 @@ cudaError_t try_rows(const PlanImpl &p, const TQ *Q, float *out, cudaStream_t st
     return cudaGetLastError();
 }
 
+constexpr int kBandRows = kGenWarps * kGenRows;  // rows per CTA of the generic kernel
+
+// Decimated views per CTA of the generic kernel, from the `ctas` of one range:
+// up to eight CTAs per SM, by the views that a CTA streams times the CTAs of an
+// SM, of which `idle` run as fast as one: eight, or three where 2D taps (four
+// running sums) meet a small grid.  49^3 x 72 bf16, D = 6, 2D taps: 27 us where a
+// range had to have twice the blocks that it streams besides its own, 15 now;
+// 331^3 x 328 f32 333 us, both.
+int generic_range(const PlanImpl &p, long long ctas) {
+    int dev = 0, sms = 148;
+    if (cudaGetDevice(&dev) == cudaSuccess) cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
+    const int most = (int)std::min<long long>(p.Pd, (8LL * sms + ctas - 1) / ctas);
+    const double idle = p.tap_blocks == 2 && ctas < 2LL * sms ? 3.0 : 8.0;
+    int jrange = p.Pd;
+    double best = 0.0;
+    for (int n = 1; n <= most; ++n) {
+        const int jr = (p.Pd + n - 1) / n;
+        const double per = (double)(ctas * ((p.Pd + jr - 1) / jr)) / sms;
+        const double cost = (jr + 2 * p.tap_blocks - 1) * std::max(idle, per);
+        if (n == 1 || cost < best) {
+            best = cost;
+            jrange = jr;
+        }
+    }
+    return jrange;
+}
+
 template <typename TQ, int H>
 cudaError_t form_t(const PlanImpl &p, fdkod_forms &f) {
     RowsShape r;
-    if (!rows_shape<TQ, H>(p, p.g.Nv, r)) return cudaSuccess;
+    if (!rows_shape<TQ, H>(p, p.g.Nv, r)) {
+        const int tiles = (p.Tstride + 31) / 32, bands = (p.g.Nv + kBandRows - 1) / kBandRows;
+        const int jrange = generic_range(p, (long long)tiles * bands * p.od.nsq);
+        f.dec_ranges = (p.Pd + jrange - 1) / jrange;
+        return cudaSuccess;
+    }
     f.dec_warps = r.warps;
     f.dec_ranges = (p.Pd + r.jrange - 1) / r.jrange;
     f.dec_resident = r.resident;
@@ -569,15 +601,8 @@ cudaError_t launch_t(const PlanImpl &p, const TQ *Q, float *out, cudaStream_t st
     cudaError_t te = p.tap_blocks == 2 ? try_rows<TQ, 2>(p, Q, out, st, rw, launched)
                                        : try_rows<TQ, 1>(p, Q, out, st, rw, launched);
     if (launched || te != cudaSuccess) return te;
-    constexpr int kBandRows = kGenWarps * kGenRows;
     const int tiles = (p.Tstride + 31) / 32, bands = (rw.rowend - rw.rowoff + kBandRows - 1) / kBandRows;
-    // ranges of decimated views until every SM has eight CTAs, of at least twice
-    // the blocks that a range streams besides its own
-    int dev = 0, sms = 148;
-    if (cudaGetDevice(&dev) == cudaSuccess) cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
-    const long long ctas = (long long)tiles * bands * p.od.nsq;
-    const int want = (int)std::min<long long>(p.Pd, (8LL * sms + ctas - 1) / ctas);
-    const int jrange = std::min(p.Pd, std::max((p.Pd + want - 1) / want, 2 * (2 * p.tap_blocks - 1)));
+    const int jrange = generic_range(p, (long long)tiles * bands * p.od.nsq);
     const dim3 grid(tiles * ((p.Pd + jrange - 1) / jrange), bands, p.od.nsq);
     const dim3 block(32, kGenWarps);
     auto kernel = p.tap_blocks == 2 ? decompose_kernel<TQ, 2> : decompose_kernel<TQ, 1>;

@@ -41,3 +41,24 @@ def test_resident_ctas_fit_the_sm(fd, qtype, taps, N, s, P):
         off = torch.empty(Q.numel() + 1, dtype=Q.dtype, device="cuda")[1:].view(Q.shape).copy_(Q)
         assert torch.equal(plan.decompose(Q), plan.decompose(off))
         assert plan.device_status() == 0
+
+
+@pytest.mark.parametrize("qtype", ["f32", "bf16"])
+@pytest.mark.parametrize("taps", ["triangle", "sinc"])
+@pytest.mark.parametrize("N,Nu,P,s,D", [
+    (72, 72, 96, 0, 8),     # staged
+    (40, 40, 24, 0, 2),
+    (49, 49, 72, 0, 6),     # generic: rows TMA cannot describe
+    (33, 33, 32, 0, 16),    # two decimated views
+])
+def test_few_ctas_take_every_range(fd, qtype, taps, N, Nu, P, s, D):
+    """Grids far smaller than the GPU split into ranges of one decimated view
+    (a CTA walks its views one after the other), with the same bits as one
+    launch that reads from another address takes."""
+    with fd.Plan(4.0 * N, N, Nu, N, P, s, D, qtype=qtype, taps=taps) as plan:
+        form = fd.fdkod_get_forms(plan.handle)
+        assert form["dec_ranges"] == P // D and (form["dec_warps"] > 0) == (Nu % 8 == 0), form
+        Q = torch.randn(plan.q_shape, device="cuda").to(_TYPES[qtype])
+        off = torch.empty(Q.numel() + 1, dtype=Q.dtype, device="cuda")[1:].view(Q.shape).copy_(Q)
+        assert torch.equal(plan.decompose(Q), plan.decompose(off))
+        assert plan.device_status() == 0
