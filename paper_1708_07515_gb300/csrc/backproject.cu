@@ -656,6 +656,15 @@ bool pair_ring(int es, int zp, int rows, PairShape &s) {
     return pair_smem(es, 1, 3, ts) <= budget;
 }
 
+// CTAs of the pair kernel that an SM holds at once: the registers' count, or
+// what the ring leaves room for
+int pair_resident(int es, int zp, int rows, const PairShape &s) {
+    size_t per_sm = 0;
+    smem_budget(&per_sm);
+    const size_t smem = pair_smem(es, s.vps, s.slots, pair_tile_stride(es, rows, s.WD)) + 2048;
+    return std::max(1, (int)std::min<size_t>((size_t)pair_ctas(zp), per_sm / smem));
+}
+
 // What rounds in the pair kernel's shape for `pairs` pairs of slices per column
 // (slices per slab, CTAs that share the views), with the ring of s.WD columns;
 // false where the windows are too large to stage.  32
@@ -675,22 +684,27 @@ bool pair_slabs(const PlanImpl &p, const SquareSet &ss, bool direct, bool mirror
         pair_ring(es, 32, ss.Rw, s) && s.vps == 2)
         return true;
     s.zp = 16;
+    if (ss.Rw2 > 256 || !pair_ring(es, 16, ss.Rw2, s)) return false;
     // Clusters share the views where the tiles leave SMs idle: as many CTAs as
     // fit the GPU at once, at least 5 views each (64^3 x 45 views, 32 CTAs: 36.4
     // us alone, 16.8 in clusters of 8; 96^3 x 67, 108 CTAs: 51.7, 37.3 in 4,
     // 44.9 in 8).  Up to two waves, smaller pieces still fill the last wave
     // better where they are long enough (128^3 x 64, 256 CTAs: 74.3, 69.4 in 4;
     // x 179: 196, 167; 160^3 x 55, 500 CTAs: 115, 109 in 2), but not beyond
-    // (192^3 x 67, 864 CTAs: 203, 211 in 2).
+    // (192^3 x 67, 864 CTAs: 203, 211 in 2).  What fits at once is what the ring
+    // leaves room for: with R = 1.2 N one CTA per SM, where 128^3 x 64 takes 162 us
+    // alone, 227 in 4, and a second wave does not pay (96^3 x 67, 108 CTAs: 107, 113
+    // in 4).
     if (mirror) {
         const int views = direct ? p.g.P : p.Pd;
-        const long long ctas = tiles * n16, slots = (long long)pair_ctas(16) * sms;
+        const int resident = pair_resident(es, 16, ss.Rw2, s);
+        const long long ctas = tiles * n16, slots = (long long)resident * sms;
         for (int n = 8; n >= 2 && s.nsplit == 1; n /= 2)
             if (ctas * n <= slots && views >= 5 * n) s.nsplit = n;
-        if (s.nsplit == 1 && ctas * 4 <= 3 * slots && views >= 64) s.nsplit = 4;
-        if (s.nsplit == 1 && ctas * 4 <= 5 * slots && views >= 32) s.nsplit = 2;
+        if (s.nsplit < 4 && resident > 1 && ctas * 4 <= 3 * slots && views >= 64) s.nsplit = 4;
+        if (s.nsplit == 1 && resident > 1 && ctas * 4 <= 5 * slots && views >= 32) s.nsplit = 2;
     }
-    return ss.Rw2 <= 256 && pair_ring(es, 16, ss.Rw2, s);
+    return true;
 }
 
 // The pair kernel's shape; false where it does not apply (no window width, or
