@@ -122,6 +122,7 @@ void size_windows(const PlanImpl &p, SquareSet &ss, const double2 *cs) {
                             umax = std::max(umax, iu);
                         }
                     ext_t = std::max(ext_t, tmax - tmin);
+                    ss.drift = std::max(ss.drift, std::max(umax - 1.0, 1.0 - umin));
                     ext_v = std::max(ext_v, (double)(kZT - 1) * umax + zabs * (umax - umin));
                     ext_v2 = std::max(ext_v2, (double)(kZP - 1) * umax + zabs * (umax - umin));
                 }

@@ -679,8 +679,12 @@ bool pair_slabs(const PlanImpl &p, const SquareSet &ss, bool direct, bool mirror
     int dev = 0, sms = 148;
     if (cudaGetDevice(&dev) == cudaSuccess) cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
     const int n32 = (pairs + 31) / 32, n16 = (pairs + 15) / 16;
+    // 16-bit windows: only far sources and 16 waves of CTAs (512^3 x 180 bf16, R = 6 N:
+    // 9.61 ms, 9.78 with 16 slices; R = 3 N 10.56, 10.40; R = 2 N 11.9, 11.0; 256^3 x
+    // 90 f16, R = 4 N 722 us, 692).
+    const bool far = es == 4 || ss.drift < 0.25;
     s.zp = 32;
-    if (ss.Rw <= 256 && tiles * n32 >= 2LL * pair_ctas(32) * sms && 64 * n32 <= 34 * n16 &&
+    if (far && ss.Rw <= 256 && tiles * n32 >= (es == 4 ? 2LL : 16LL) * pair_ctas(32) * sms && 64 * n32 <= 34 * n16 &&
         pair_ring(es, 32, ss.Rw, s) && s.vps == 2)
         return true;
     s.zp = 16;

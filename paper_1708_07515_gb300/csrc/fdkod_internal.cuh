@@ -40,6 +40,7 @@ struct SquareSet {
     // when no instantiation is wide enough)
     int Wd = 0, Rw = 0, WdT = 0, WdT16 = 0;  // WdT16: the same for 16-bit windows
     int Rw2 = 0;  // rows of a window of kZP slices (the mirrored-pair kernel; Rw: of kZT slices)
+    double drift = 0.0;        // the largest |1/U - 1|: rows per slice, less one
     int need = 0, need16 = 0;  // the narrowest TMA windows that hold every tile's footprint
     int tiles_per_side = 1;  // 16-voxel tiles per square side
 };

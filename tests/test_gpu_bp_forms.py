@@ -44,9 +44,10 @@ def _q(seed, P, Nv, Nu, dtype):
     (192, 67, 2, 1, "f32", 16),     # views 67: a short last chunk
     (192, 130, 2, 2, "f32", 16),
     (184, 64, 2, 1, "bf16", 16),
-    (250, 65, 2, 1, "f32", 32),     # at 1.6 N the windows of 32 float32 slices are too large: 16
+    (250, 65, 2, 1, "f32", 32),     # at 1.6 N the windows of 32 slices are too large: 16
     (245, 128, 2, 2, "f32", 32),
-    (248, 61, 2, 1, "f16", 32),     # 32 at both
+    (248, 61, 2, 1, "f16", 16),     # 16-bit windows: 32 for far sources and many tiles only
+    (432, 26, 0, 1, "f16", 32),
 ])
 def test_many_views_without_a_cluster(fd, oracle_mod, N, P, s, D, qtype, slices, ratio):
     R, Nu = ratio * N, N + (-N) % 8
@@ -54,7 +55,7 @@ def test_many_views_without_a_cluster(fd, oracle_mod, N, P, s, D, qtype, slices,
     zs = np.array([0, 15, 16, 31, 32, N // 2, N - 33, N - 1])
     with fd.Plan(R, N, Nu, N - 1, P, s, D, qtype=qtype) as plan:
         form = fd.fdkod_get_forms(plan.handle)
-        if ratio < 2.0 and qtype == "f32":
+        if ratio < 2.0:
             slices = 16
         assert form["bp_slices"] == slices and form["bp_split"] == 1, form
         assert P // D > 2 * form["bp_views"] * form["bp_slots"]
