@@ -1,19 +1,21 @@
 // Cone-beam backprojection for FDK-OD (Sec. 2.2) and plain FDK (Sec. 2.1).
 //
-// One CTA of 16 x 16 threads owns a 16 x 16 column tile of one square and
-// kZT consecutive slices; each thread owns one (x, y) column and kZT voxels
-// along z in registers.  For every chunk of up to 8 views the CTA
-//   1. finds, per view, the detector window its voxels can touch: the
-//      column coordinate (Eq. 1 in square-local form) and the row
-//      coordinate z/U + (Nv-1)/2 are monotone in x, y and z, so the tile's
-//      corners bound them;
-//   2. stages each window (rows x columns, zero outside the detector) from
-//      global memory into shared memory with coalesced row loads;
-//   3. accumulates U^-2 times the bilinear sample for each of its voxels.
-// The gather is a sum over views of interpolated samples, not a dense
-// contraction, so it runs on the FP32 pipes and the shared-memory path.
+// For every square (a tile of 16 x 16 columns at a time), slab of slices and
+// view, the detector window that the voxels touch is bounded by the tile's
+// corners -- the column coordinate (Eq. 1 in square-local form) and the row
+// coordinate z/U + (Nv-1)/2 are monotone in x, y and z -- and staged in shared
+// memory, zero outside the detector; each thread adds U^-2 times the bilinear
+// sample to the voxels of its column.  The gather is a sum over views of
+// interpolated samples, not a dense contraction, so it runs on the FP32 pipes
+// and the shared-memory path.  The kernels, in the order they are tried:
+//   bp_pair_kernel (bp_pair.cuh): windows by TMA, two slabs per CTA; whole
+//     volumes (a slab and its mirror image) and slabs of slices;
+//   bp_generic_kernel: windows by plain loads, where TMA cannot describe the
+//     source or a ring of the larger windows does not fit;
+//   bp_global_kernel: no staging, where not even one window fits;
+//   bp_persistent_kernel: a batch of plans in one launch.
 //
-// Two sources share the kernel:
+// Two sources share each of them:
 //   direct (D = 1 and the plain FDK baseline): Q_k itself, cropped per
 //     (square, view) at crop = floor(phi + w0); column offset frac - w0;
 //   decomposed (D > 1): the square's decimated data S'_q[j][v][t] at the
@@ -58,12 +60,13 @@ __device__ __forceinline__ float ld_s(const float *p) { return __ldg(p); }
 __device__ __forceinline__ float ld_s(const __nv_bfloat16 *p) { return __bfloat162float(__ldg(p)); }
 __device__ __forceinline__ float ld_s(const __half *p) { return __half2float(__ldg(p)); }
 
-// Where TMA cannot describe the source (a detector whose rows are not whole
-// 16-byte units).  WD: window columns at compile time (0: a.Wd), so that a
-// sample's four loads take one address; a warp stages four rows of a window
-// at a time, all their loads in flight together; the row coordinate's floor
-// is one rounded-down addition.  253^3, 253 columns, 120 views, plain FDK: 3.63
-// ms before (row by row, every address and clamp per sample), 1.94.
+// One CTA of 16 x 16 threads owns a 16 x 16 column tile of one square and kZT
+// consecutive slices, each thread one column's kZT voxels in registers; up to
+// 8 views' windows are staged at a time.  WD: window columns at compile time
+// (0: a.Wd), so that a sample's four loads take one address; a warp stages four
+// rows of a window at a time, all their loads in flight together; the row
+// coordinate's floor is one rounded-down addition.  253^3, 253 columns, 120 views,
+// plain FDK: 3.63 ms before (row by row, every address and clamp per sample), 1.94.
 template <typename TS, bool DIRECT, int WD>
 __global__ void __launch_bounds__(kThreads, WD == 0 ? 1 : 3)
 bp_generic_kernel(BpParams a) {
@@ -363,8 +366,6 @@ struct BpTmaParams {
     int row0;             // detector row held in the source's row 0
     int zoff, nz;         // slices zoff .. zoff + nz - 1, written to vol[z - zoff]
     float scale;
-    unsigned long long wait_ns;  // limit of every bounded wait (ns)
-    int fault;                   // test hook (kTestFault*), 0 = none
 };
 
 // address bias: (row + kMagicBits) * 4 WD wraps to row * 4 WD in 32 bits once
@@ -586,11 +587,10 @@ bool source_map(const PlanImpl &p, const SquareSet &ss, bool direct, const void 
 }
 
 // Tensor map, parameters and window width of a plan in the batch's persistent
-// launch; false when it cannot take it.
+// launch (float32 windows; it has no test hooks); false when it cannot take it.
 bool make_tma_launch(const PlanImpl &p, const SquareSet &ss, bool direct, const void *src, float *vol,
                      const Band &b, CUtensorMap &map, BpTmaParams &a, int &WD) {
-    const int es = (direct && p.qtype != FDKOD_F32) ? 2 : 4;
-    WD = es == 4 ? ss.WdT : ss.WdT16;
+    WD = ss.WdT;
     if (!source_map(p, ss, direct, src, b.nrows, WD, ss.Rw, map)) return false;
     a = BpTmaParams{};
     a.vol = vol;
@@ -608,10 +608,7 @@ bool make_tma_launch(const PlanImpl &p, const SquareSet &ss, bool direct, const 
     a.row0 = b.row0;
     a.zoff = b.zoff;
     a.nz = b.nz;
-    a.wait_ns = p.wait_ns > 0 ? (unsigned long long)p.wait_ns : kWaitLimitNs;
-    a.fault = p.test_fault;
-    // elements per staged window, a 128-byte multiple
-    a.tile_stride = (ss.Rw * WD + (128 / es - 1)) & ~(128 / es - 1);
+    a.tile_stride = pair_tile_stride(4, ss.Rw, WD);  // elements per staged window, a 128-byte multiple
     if (direct) {
         a.nviews = p.g.P;
         a.vstep = 1;
@@ -905,8 +902,6 @@ cudaError_t batch_create(const PlanImpl *const *plans, const void *const *src, f
         b.nz = p.g.N;
         int WD = 0;
         if (!make_tma_launch(p, p.od, direct, src[i], vols[i], b, maps[i], insts[i].a, WD)) return cudaSuccess;
-        insts[i].a.wait_ns = kWaitLimitNs;  // the persistent form has no test hooks
-        insts[i].a.fault = 0;
         insts[i].direct = direct ? 1 : 0;
         insts[i].WD = WD;
         smem = std::max(smem, sizeof(float) * (size_t)2 * kViewsPerStage * insts[i].a.tile_stride + 128);

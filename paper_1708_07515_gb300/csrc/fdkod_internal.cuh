@@ -49,7 +49,7 @@ constexpr int kTile = 16;      // tile side in x and y (threads per CTA = 256)
 constexpr int kZT = 32;        // z voxels per thread
 constexpr int kZP = 16;        // slices per half of the mirrored-pair kernel's smaller form (the larger: kZT)
 constexpr int kViewsPerChunk = 8;  // generic backprojection kernel
-constexpr int kViewsPerStage = 4;  // TMA backprojection kernel (two stages)
+constexpr int kViewsPerStage = 4;  // the batch's persistent kernel (two stages)
 constexpr int kMaxTapD = 128;      // largest decimation factor with a tap table
 
 // learned angular decimation: 16 channels, 5 taps, 1440 weights
