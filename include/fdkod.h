@@ -440,8 +440,8 @@ int fdkod_net_backward(fdkod_plan_t *plan, const void *Q, const float *w, const 
  * source.  Device-side status (window overflow, wait timeout) goes to each
  * plan's status word (fdkod_last_device_status).  Errors: INVALID_ARG (null
  * pointers, count < 1, NULL source for a plan without one), UNSUPPORTED (a
- * plan with 16-bit Q and D = 1, or windows that no TMA box holds: use the
- * per-plan entry points), OOM, CUDA.
+ * plan with 16-bit Q and D = 1, or windows that no TMA box or too little
+ * shared memory holds: use the per-plan entry points), OOM, CUDA.
  */
 typedef struct fdkod_batch fdkod_batch_t;
 int fdkod_batch_create(fdkod_plan_t *const *plans, const void *const *src, float *const *vols, int count,

@@ -907,6 +907,7 @@ cudaError_t batch_create(const PlanImpl *const *plans, const void *const *src, f
         smem = std::max(smem, sizeof(float) * (size_t)2 * kViewsPerStage * insts[i].a.tile_stride + 128);
         order.push_back({-(double)p.g.N * p.g.N * p.g.N * (double)insts[i].a.nviews, i});
     }
+    if (smem > smem_budget()) return cudaSuccess;  // two stages of the widest windows do not fit
     std::sort(order.begin(), order.end());
     std::vector<int4> items;
     for (const auto &oi : order) {
