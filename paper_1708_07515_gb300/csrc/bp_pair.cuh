@@ -466,10 +466,28 @@ bp_pair_kernel(const __grid_constant__ CUtensorMap tmap, BpPairParams a) {
 
     // A warp wholly outside a ragged tile only hands the slots back: its work
     // would take issue slots from the others (367^3, squares of 23 voxels: 4.30 ->
-    // 3.21 ms; 306^3 x 428 bf16, squares of 38, D = 1: 8.41 -> 7.27 ms).
-    const int mine = __any_sync(0xffffffffu, active) ? VPS : 0;
+    // 3.21 ms; 306^3 x 428 bf16, squares of 38, D = 1: 8.41 -> 7.02 ms).  Where it
+    // is asked is a matter of registers: mirrored slabs in the view loop (512^3 8.26
+    // ms, 8.40 with a loop of its own), others in a loop of its own (a 64-slice slab
+    // of 2000^3 5.47 ms, 5.58 in the view loop).
+    const bool idle = !__any_sync(0xffffffffu, active);
+    const int mine = MIRROR && idle ? 0 : VPS;
     int sl = 0, left = nviews;
     uint32_t phase = 0;
+    if (!MIRROR && idle) {
+        for (; left > 0; left -= VPS) {
+            const bool ok = tma::mbar_wait_bounded(&full[sl], phase, a.wait_ns);
+            if (!__all_sync(0xffffffffu, ok)) {
+                if (lane == 0) atomicOr(a.status, 2);
+                return;
+            }
+            if (lane == 0) tma::mbar_arrive(&empty[sl]);
+            if (++sl == SLOTS) {
+                sl = 0;
+                phase ^= 1u;
+            }
+        }
+    }
     for (; left > 0; left -= VPS) {
         const bool ok = tma::mbar_wait_bounded(&full[sl], phase, a.wait_ns);
         if (!__all_sync(0xffffffffu, ok)) {
