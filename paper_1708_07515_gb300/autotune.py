@@ -114,9 +114,13 @@ def tile_candidates(min_cols: int, count: int = 3) -> list[int]:
 def choose_tile(plan, reps: int = 3, count: int = 3) -> tuple[int, dict]:
     """Time the plan's FDK-OD backprojection (from its decomposed workspace,
     or from Q when D = 1) with each candidate window width, keep the fastest
-    (set on the plan) and return (width, {width: ms}).  Data values do not
-    change the timing, so zero inputs serve."""
+    (set on the plan) and return (width, {width: ms}).  Widths that the
+    launch would not take (no room for its ring) are left out: they would time
+    the default one.  Data values do not change the timing, so zero inputs
+    serve."""
     import torch
+
+    from .fdkod import fdkod_get_forms
     _, narrowest = plan.tile
     cands = tile_candidates(narrowest, count)
     if len(cands) < 2:
@@ -128,6 +132,8 @@ def choose_tile(plan, reps: int = 3, count: int = 3) -> tuple[int, dict]:
     times = {}
     for w in cands:
         plan.set_tile(w)
+        if fdkod_get_forms(plan.handle)["bp_columns"] != w:
+            continue
         run = (lambda: plan.backproject(Q, vol)) if plan.D == 1 else \
             (lambda: plan.backproject_decomposed_workspace(vol))
         run()
@@ -139,6 +145,9 @@ def choose_tile(plan, reps: int = 3, count: int = 3) -> tuple[int, dict]:
         b.record()
         torch.cuda.synchronize()
         times[w] = a.elapsed_time(b) / reps
+    if not times:   # the staged kernel does not apply
+        plan.set_tile(0)
+        return plan.tile[0], {}
     best = min(times, key=times.get)
     plan.set_tile(best)
     return best, times

@@ -52,3 +52,22 @@ def test_every_width_gives_the_same_bits(fd, N, P, s, D, r, qtype):
             for a, b, what in zip(got, want, ("volume", "slab")):
                 assert torch.equal(a, b), (w, what, float((a - b).abs().max()))
         assert plan.device_status() == 0
+
+
+def test_the_tuner_times_the_widths_that_launches_take(fd):
+    """choose_tile leaves out widths for which a launch would keep the default
+    one (their times say nothing about the width, and the batch's persistent
+    kernel would take them), and detectors the staged kernel cannot read."""
+    from paper_1708_07515_gb300 import autotune
+    with fd.Plan(4.0 * 245, 245, 248, 245, 24, 2, 2) as plan:
+        taken = []
+        for w in autotune.tile_candidates(plan.tile[1], count=5):
+            plan.set_tile(w)
+            if fd.fdkod_get_forms(plan.handle)["bp_columns"] == w:
+                taken.append(w)
+        assert taken and taken != autotune.tile_candidates(plan.tile[1], count=5)
+        plan.set_tile(0)
+        best, times = autotune.choose_tile(plan, count=5)
+        assert sorted(times) == taken and plan.tile[0] == best and best in taken
+    with fd.Plan(4.0 * 64, 64, 63, 64, 24, 1, 1) as plan:
+        assert autotune.choose_tile(plan) == (plan.tile[1], {})
