@@ -248,7 +248,7 @@ __device__ __forceinline__ void pair_slices_any(float2 (&acc)[ZP], float w, floa
 // the windows, writes the view parameters and issues the copies into a ring
 // of SLOTS slots); warps 0-7 consume.  A slot is full when its copies
 // have landed (full[slot], which also publishes the producer's parameters)
-// and free again when all eight consumer warps have arrived on empty[slot]:
+// and free again when the consumer warps have arrived on empty[slot]:
 // no block-wide barrier inside the view loop, so consumer warps drift within
 // the ring instead of waiting for the slowest.  Every wait is bounded
 // (FDKOD_ERR_TIMEOUT); a producer that gives up waits for its copies in
@@ -324,9 +324,12 @@ bp_pair_kernel(const __grid_constant__ CUtensorMap tmap, BpPairParams a) {
     auto win = [&](int sl, int w, int h) { return (uint32_t)((sl * VPS + w) * 2 + h) * (uint32_t)a.tile_stride; };
 
     if (threadIdx.x == 0) {
+        // warps with a column of the tile (8 x 4 each); the others leave at once
+        // unless MIRROR
+        const int busy = ((xe - x0) / 8 + 1) * ((ye - y0) / 4 + 1);
         for (int i = 0; i < SLOTS; ++i) {
             tma::mbar_init(&full[i], 1);
-            tma::mbar_init(&empty[i], kPairConsumers);
+            tma::mbar_init(&empty[i], MIRROR ? kPairConsumers : busy);
         }
         tma::fence_mbar_init();
     }
@@ -464,30 +467,20 @@ bp_pair_kernel(const __grid_constant__ CUtensorMap tmap, BpPairParams a) {
 #pragma unroll
     for (int i = 0; i < ZP; ++i) acc[i] = make_float2(0.f, 0.f);
 
-    // A warp wholly outside a ragged tile only hands the slots back: its work
-    // would take issue slots from the others (367^3, squares of 23 voxels: 4.30 ->
-    // 3.21 ms; 306^3 x 428 bf16, squares of 38, D = 1: 8.41 -> 7.02 ms).  Where it
-    // is asked is a matter of registers: mirrored slabs in the view loop (512^3 8.26
-    // ms, 8.40 with a loop of its own), others in a loop of its own (a 64-slice slab
-    // of 2000^3 5.47 ms, 5.58 in the view loop).
-    const bool idle = !__any_sync(0xffffffffu, active);
+    // A warp wholly outside a ragged tile takes no part: its work would take issue
+    // slots from the others (367^3, squares of 23 voxels: 4.30 -> 3.21 ms; 306^3 x 428
+    // bf16, squares of 38, D = 1: 8.41 -> 7.02 ms).  Not mirrored, it leaves (`empty`
+    // does not count it); mirrored, it hands the slots back.  How it is asked
+    // moves the registers of the view loop: mirrored, this vote inside the loop
+    // saves spills (512^3 8.35 -> 8.25 ms; 8.34 by the tile's extent); otherwise the
+    // extent (a 64-slice slab of 2000^3 with its decomposition 10.40 -> 10.38 ms; 10.53
+    // by the vote, 10.43 with a loop that hands the slots back).
+    const bool idle = MIRROR ? !__any_sync(0xffffffffu, active)
+                             : (warp & 1) * 8 > xe - x0 || (warp >> 1) * 4 > ye - y0;
+    if (!MIRROR && idle) return;
     const int mine = MIRROR && idle ? 0 : VPS;
     int sl = 0, left = nviews;
     uint32_t phase = 0;
-    if (!MIRROR && idle) {
-        for (; left > 0; left -= VPS) {
-            const bool ok = tma::mbar_wait_bounded(&full[sl], phase, a.wait_ns);
-            if (!__all_sync(0xffffffffu, ok)) {
-                if (lane == 0) atomicOr(a.status, 2);
-                return;
-            }
-            if (lane == 0) tma::mbar_arrive(&empty[sl]);
-            if (++sl == SLOTS) {
-                sl = 0;
-                phase ^= 1u;
-            }
-        }
-    }
     for (; left > 0; left -= VPS) {
         const bool ok = tma::mbar_wait_bounded(&full[sl], phase, a.wait_ns);
         if (!__all_sync(0xffffffffu, ok)) {
