@@ -470,8 +470,14 @@ bool rows_shape(const PlanImpl &p, int nrows, RowsShape &r) {
     constexpr int kAlign = 16 / (int)sizeof(TQ);
     if ((p.g.Nu % kAlign) != 0 || p.D > kMaxTapD) return false;
     const int all = (p.Tstride + kCW - 1) / kCW;  // column segments of a square
+    // as few CTAs side by side as hold them, or one more where that leaves fewer
+    // segments empty: 16 segments 4 x 4 rather than 3 x 6 (584^3 x 720, s = 2: 865 ->
+    // 795 us, 2D taps 1243 -> 992), 9 as 3 x 3 rather than 2 x 5 (660^3 x 400 1107 ->
+    // 1030 us, 2D taps 1766 -> 1392), but 13 as 2 x 7 (256^3 x 360, s = 1: 56 us, 57 in 3 x 5)
     r.chunks = (all + kDecMaxSegs - 1) / kDecMaxSegs;
-    r.segs = (all + r.chunks - 1) / r.chunks;
+    auto segs_of = [&](int chunks) { return (all + chunks - 1) / chunks; };
+    if ((r.chunks + 1) * segs_of(r.chunks + 1) < r.chunks * segs_of(r.chunks)) ++r.chunks;
+    r.segs = segs_of(r.chunks);
     // the segments' columns + neighbour + crop offset, whole 16-byte units, an odd number of them
     r.Wc = (std::min(p.od.Tmax, r.segs * kCW) + 1 + (kAlign - 1) + (kAlign - 1)) & ~(kAlign - 1);
     if ((r.Wc / kAlign) % 2 == 0) r.Wc += kAlign;

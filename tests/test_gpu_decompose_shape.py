@@ -26,7 +26,7 @@ def fd():
 @pytest.mark.parametrize("N,s,P", [
     (16, 1, 24), (16, 0, 24), (40, 1, 48), (48, 0, 64), (64, 0, 96), (72, 0, 96),   # 1 to 7 segments
     (80, 0, 240), (84, 0, 96), (300, 2, 420),                                       # 8: two CTAs of four
-    (96, 0, 128), (150, 0, 200), (165, 0, 200), (176, 0, 96), (352, 1, 480),        # wider
+    (96, 0, 128), (150, 0, 200), (165, 0, 200), (170, 0, 96), (176, 0, 96), (352, 1, 480),   # wider
     (64, 2, 6000),                                                                  # tables as large as the ring
 ])
 def test_resident_ctas_fit_the_sm(fd, qtype, taps, N, s, P):
@@ -41,6 +41,15 @@ def test_resident_ctas_fit_the_sm(fd, qtype, taps, N, s, P):
         off = torch.empty(Q.numel() + 1, dtype=Q.dtype, device="cuda")[1:].view(Q.shape).copy_(Q)
         assert torch.equal(plan.decompose(Q), plan.decompose(off))
         assert plan.device_status() == 0
+
+
+@pytest.mark.parametrize("N,s,segments,warps", [(84, 0, 8, 4), (96, 0, 9, 3), (142, 0, 13, 7), (170, 0, 16, 4)])
+def test_segments_split_evenly(fd, N, s, segments, warps):
+    """As few CTAs side by side as hold a square's column segments, or one more
+    where fewer segments stay empty."""
+    with fd.Plan(4.0 * N, N, (N + 7) // 8 * 8, 64, 24, s, 2) as plan:
+        assert (plan.info["T_stride"] + 15) // 16 == segments, plan.info["T_stride"]
+        assert fd.fdkod_get_forms(plan.handle)["dec_warps"] == warps
 
 
 @pytest.mark.parametrize("qtype", ["f32", "bf16"])
