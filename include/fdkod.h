@@ -437,7 +437,7 @@ int fdkod_net_backward(fdkod_plan_t *plan, const void *Q, const float *w, const 
  * holds; each takes items until none are left (asynchronous on `stream`,
  * no allocation: it can be captured into a CUDA graph).  The result equals
  * each plan's fdkod_backproject_decomposed / fdkod_backproject of the same
- * source.  Device-side status (window overflow, wait timeout) goes to each
+ * source to float32 rounding (another kernel).  Device-side status (window overflow, wait timeout) goes to each
  * plan's status word (fdkod_last_device_status).  Errors: INVALID_ARG (null
  * pointers, count < 1, NULL source for a plan without one), UNSUPPORTED (a
  * plan with 16-bit Q and D = 1, or windows that no TMA box or too little

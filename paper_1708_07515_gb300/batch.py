@@ -11,9 +11,9 @@ persistent=True the backprojections of all volumes -- most of the work --
 are instead one persistent launch after every decomposition
 (fdkod_batch_backproject: a work list of (volume, tile, z-slab) items,
 largest volumes first, taken by as many CTAs as the GPU holds); it gives
-the same volumes bit for bit but gives up that overlap (a kernel cannot
-wait for another launch's results), which costs more than it saves (207
-against 187 ms for 64 volumes of N 64-384).  The whole batch is captured
+the same volumes to float32 rounding (another kernel, one voxel at a time)
+and gives up that overlap (a kernel cannot wait for another launch's
+results): 199 ms against 116.5 for 64 volumes of N 64-384.  The whole batch is captured
 once into a single CUDA graph and runs as one graph launch.  All kernels
 are libfdkod's; torch only provides memory, streams and the graph object.
 """

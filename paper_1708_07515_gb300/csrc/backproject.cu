@@ -640,7 +640,7 @@ size_t smem_budget(size_t *per_sm = nullptr) {
 // registers allow (each with its static shared memory and the runtime's
 // reserve, 2 KiB together at most), else 3 of 1 if one CTA fits; false if not.
 // (250^3, R = 2.5 N: 3 x 1 views 917 us, 2 x 2 846; 512^3: 3 x 2 8.35 ms, 2 x 2
-// 8.38.)
+// 8.38; all four 1-2 % less since warps outside a tile take no part.)
 bool pair_ring(int es, int zp, int rows, PairShape &s) {
     size_t per_sm = 0;
     const size_t budget = smem_budget(&per_sm);
@@ -666,7 +666,7 @@ int pair_resident(int es, int zp, int rows, const PairShape &s) {
 // (slices per slab, CTAs that share the views), with the ring of s.WD columns;
 // false where the windows are too large to stage.  32
 // pairs per thread halve the per-view set-up and stage fewer margin rows
-// (512^3: 8.35 ms against 8.77 at 16), but need enough CTAs: 2 per SM, half as
+// (512^3: 8.25 ms against 8.61 at 16), but need enough CTAs: 2 per SM, half as
 // many of them (from 160^3 to 256^3 both take the same time within 4 %), and
 // they must not compute much more than they keep (the last slab's excess).
 bool pair_slabs(const PlanImpl &p, const SquareSet &ss, bool direct, bool mirror, int pairs, PairShape &s) {

@@ -45,11 +45,11 @@ cudaError_t launch_pair_f16(const PairShape &s, const CUtensorMap &map, const Bp
 // offsets from one address (pair_slices): no address, row or fraction
 // arithmetic in integers per slice, and each row is loaded and
 // column-interpolated once per group, also where 1/U > 1 (before: both rows
-// of every such slice).  ncu, 256^3 x 90 views: 28.7 -> 19.5 warp instructions
+// of every such slice).  ncu, 256^3 x 90 views: 28.7 -> 20.3 warp instructions
 // and 6.5 -> 4.9 shared loads per slice pair.  A warp covers 8 x 4 columns (16 x 2:
 // 5 % bank conflicts, now none).  Backprojection of 512^3 x 180 views:
-// 10.80 ms before, 8.77 ms with ZP = 16, 8.35 ms with ZP = 32 (1024^3 x 180
-// views 42.9 -> 33.4 ms); a 64-slice slab of 2000^3 from 45 views, not mirrored:
+// 10.80 ms before, 8.61 ms with ZP = 16, 8.25 ms with ZP = 32 (1024^3 x 90
+// views 42.9 -> 33.0 ms); a 64-slice slab of 2000^3 from 45 views, not mirrored:
 // 6.9 ms before (one voxel at a time, 18.7 instructions each), 5.4 ms.
 struct BpPairParams {
     float *vol;

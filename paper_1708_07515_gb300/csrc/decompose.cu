@@ -135,8 +135,8 @@ decompose_kernel(const TQ *__restrict__ Q, float *__restrict__ Sp, const int32_t
 // ring and copies alone take 0.90 ms of 1.08 at 512^3.  The form before had
 // lanes along the columns: two scalar loads per sample, and columns in steps of
 // 32 lanes (128 computed for ~100 used).  512^3 x 720 f32: 1.43 -> 1.08 ms with
-// the triangle, 2.30 -> 1.49 ms with 2D-tap filters; 1024^3 x 720 bf16 10.1 -> 6.9
-// ms; a 64-slice slab of 2000^3 from 720 bf16 views 7.1 -> 5.0 ms; 64^3 30 -> 8 us.
+// the triangle, 2.30 -> 1.475 ms with 2D-tap filters; 1024^3 x 720 bf16 10.1 -> 6.9
+// ms; a 64-slice slab of 2000^3 from 720 bf16 views 7.1 -> 5.0 ms; 64^3 30 -> 6 us.
 //
 // Everything else a view needs -- shift fraction, tap weights, crop offset --
 // is one 16-byte entry of a per-CTA table in stream order (H = 2: 8 more bytes
