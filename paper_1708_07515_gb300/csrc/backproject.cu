@@ -907,7 +907,14 @@ cudaError_t batch_create(const PlanImpl *const *plans, const void *const *src, f
         smem = std::max(smem, sizeof(float) * (size_t)2 * kViewsPerStage * insts[i].a.tile_stride + 128);
         order.push_back({-(double)p.g.N * p.g.N * p.g.N * (double)insts[i].a.nviews, i});
     }
-    if (smem > smem_budget()) return cudaSuccess;  // two stages of the widest windows do not fit
+    // two stages of the widest windows must fit a block beside the static shared memory
+    cudaFuncAttributes fa{};
+    int optin = 0, dev0 = 0;
+    cudaError_t ae = cudaFuncGetAttributes(&fa, bp_persistent_kernel);
+    if (ae == cudaSuccess) ae = cudaGetDevice(&dev0);
+    if (ae == cudaSuccess) ae = cudaDeviceGetAttribute(&optin, cudaDevAttrMaxSharedMemoryPerBlockOptin, dev0);
+    if (ae != cudaSuccess) return ae;
+    if (smem + fa.sharedSizeBytes > (size_t)optin) return cudaSuccess;
     std::sort(order.begin(), order.end());
     std::vector<int4> items;
     for (const auto &oi : order) {

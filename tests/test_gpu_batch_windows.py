@@ -35,3 +35,20 @@ def test_large_windows_are_unsupported(fd):
         assert torch.equal(br.plans[0].backproject(br.Q[0]), want)
     finally:
         br.close()
+
+
+@pytest.mark.parametrize("N,ratio", [(64, 1.156), (144, 1.328)])
+def test_the_largest_windows_that_fit_are_taken(fd, N, ratio):
+    """48 x 150 and 64 x 113 windows: 230528 and 231552 bytes of the 232448 a
+    block can have.  Per-volume launches to float32 rounding, as elsewhere."""
+    P = 48
+    Q = torch.randn((P, N, N), device="cuda", generator=torch.Generator(device="cuda").manual_seed(N))
+    with fd.Plan(ratio * N, N, N, N, P, 1, 2) as plan:
+        vol = torch.empty(plan.vol_shape, device="cuda")
+        want = plan.backproject(Q)
+        batch = fd.BatchBackprojection([plan], [None], [vol])
+        batch.run()
+        assert plan.device_status() == 0
+        d = vol.double() - want.double()
+        assert float(d.norm() / want.double().norm()) <= 1e-5
+        batch.close()
